@@ -146,10 +146,17 @@ __global__ void __launch_bounds__(128) combine_generic_kernel(int32_t B, int32_t
     if (lse != nullptr && threadIdx.x == 0) lse[r] = dead ? -INFINITY : mx + logf(den);
 }
 
-// Vectorised log-sum-exp merge for d_out % 4 == 0: one thread per (row, four output columns).  Every
-// thread of a row recomputes the row's S weights from lse_part (a handful of cached, broadcast loads),
-// so there is no cross-thread step and all its 16-byte loads of the partials are independent and in
-// flight together; consecutive threads read consecutive float4, i.e. whole rows are streamed.
+// Vectorised log-sum-exp merge for d_out % 4 == 0.  A block of 256 threads owns 256 / G items of V output columns each
+// (V / 4 float4 of one row, consecutive items on consecutive float4: every load of a warp is contiguous) and splits the
+// S slots of an item over G thread groups, whose sums meet in shared memory.  The weights of the block's rows are
+// computed once, with a row's slots over adjacent lanes, and staged in shared memory, so the loads of the
+// partials depend on nothing but them: those of 16 / V slots are in flight per thread.
+// What bounds it: the latency of that chain (lse -> weights -> partials) at small row counts, HBM at large ones.  The
+// form it replaces (every thread walked all S slots, one load round trip per slot, 16 columns per thread whatever the
+// size) took 14 us on 128 rows x 128 columns x 13 slots (4 blocks) and 20 us on 512 x 512 x 20; whole steps around
+// such merges went from 22.5 to 16.4 us and from 198 to 175 us.
+constexpr int kCombineThreads = 256;
+constexpr int kCombineWeights = 1024;  // staged weights of a block: rows x slots at a time
 __device__ __forceinline__ void store4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 __device__ __forceinline__ void store4(__nv_bfloat16* p, float4 v) {
     __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
@@ -165,70 +172,125 @@ __device__ __forceinline__ float4 ld_stream4(const float* p) {  // read once: do
                  : "l"(p));
     return v;
 }
-// V = 4, 8 or 16 output columns per thread (as many as d_out allows: the kernel's CTAs wait, resident beside those of
-// the decode kernel, for it to finish, and only a grid small enough to be resident as a whole runs as one wave;
-// 16-byte stores of bf16).
-template <typename TO, int V>
-__global__ void __launch_bounds__(256) combine_vec_kernel(int64_t rows, int32_t rows_per_seq, int32_t S, int32_t d_out,
-                                                          const float* __restrict__ o_part,
-                                                          const float* __restrict__ lse_part, TO* __restrict__ out,
-                                                          float* __restrict__ lse) {
+template <typename TO, int V, int G>
+__global__ void __launch_bounds__(kCombineThreads, V == 4 ? 2 : 4) combine_vec_kernel(int64_t rows, int32_t rows_per_seq, int32_t S,
+                                                                      int32_t d_out, const float* __restrict__ o_part,
+                                                                      const float* __restrict__ lse_part,
+                                                                      TO* __restrict__ out, float* __restrict__ lse) {
+    constexpr int kItems = kCombineThreads / G;  // items of a block
+    constexpr int kF4 = V / 4;                   // float4 of an item
+    constexpr int kAhead = 16 / V;               // slots whose loads are in flight together: 64 bytes per thread
+    // a block touches at most kItems / (items per row) + 2 rows, kItems of them when a row is one item
+    __shared__ float sw[kCombineWeights], smax[kItems], sden[kItems];
+    __shared__ float4 red[G > 1 ? (G - 1) * kItems * kF4 : 1];
     // (dependent-launch instructions; no-ops when the kernel is launched the ordinary way)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int32_t per_row = d_out / V;  // items of a row
+    const int64_t item0 = (int64_t)blockIdx.x * kItems, items = rows * per_row;
+    const int64_t last = (item0 + kItems < items ? item0 + kItems : items) - 1;
+    const int64_t row0 = item0 / per_row;
+    const int n_rows = (int)(last / per_row - row0) + 1;
+    const int it = tid % kItems, grp = tid / kItems;
+    const int64_t idx = item0 + it;
+    const bool active = idx < items;
+    const int64_t r = active ? idx / per_row : row0;
+    const int c = active ? (int)(idx - r * per_row) * 4 : 0;  // float4 u sits at column c + 4 * per_row * u
+    const int rl = (int)(r - row0);
+    const int kc = S < kCombineWeights / n_rows ? S : kCombineWeights / n_rows;  // slots staged at a time
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int32_t vec_per_row = d_out / V;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t r = idx / vec_per_row;
-    if (r >= rows) return;
-    const int c = (int)(idx % vec_per_row) * V;
-    const int64_t b = r / rows_per_seq;
-    const int rr = (int)(r % rows_per_seq);
-    const float* lp = lse_part + b * S * rows_per_seq + rr;
-    float mx = -INFINITY;
-    for (int k = 0; k < S; ++k) mx = fmaxf(mx, __ldg(lp + (int64_t)k * rows_per_seq));
-    const bool dead = !(mx > -INFINITY);
-    const float* op = o_part + (b * S * rows_per_seq + rr) * d_out + c;
-    const int64_t kstride = (int64_t)rows_per_seq * d_out;
-    float4 acc[V / 4];
-#pragma unroll
-    for (int u = 0; u < V / 4; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-    float den = 0.f;
-    for (int k = 0; k < S; ++k) {
-        const float wk = dead ? 0.f : expf(__ldg(lp + (int64_t)k * rows_per_seq) - mx);
-        den += wk;
-        if (wk == 0.f) continue;  // an empty split's partial is never read
-#pragma unroll
-        for (int u = 0; u < V / 4; ++u) {
-            const float4 x = ld_stream4(op + k * kstride + 4 * u);
-            acc[u].x = fmaf(wk, x.x, acc[u].x);
-            acc[u].y = fmaf(wk, x.y, acc[u].y);
-            acc[u].z = fmaf(wk, x.z, acc[u].z);
-            acc[u].w = fmaf(wk, x.w, acc[u].w);
+
+    // weights of the block's rows: `span` lanes per row (the slot count rounded up to a power of two, at most a warp)
+    int span = 1;
+    while (span < S && span < 32) span *= 2;
+    const int kl = lane & (span - 1);
+    for (int base = warp * (32 / span); base < n_rows; base += kCombineThreads / span) {
+        const int i = base + lane / span;
+        const bool have = i < n_rows;
+        const int64_t b = (row0 + (have ? i : 0)) / rows_per_seq;
+        const float* lp = lse_part + b * (S - 1) * rows_per_seq + row0 + (have ? i : 0);  // slot 0; + k * rows_per_seq
+        float mx = -INFINITY;
+        for (int k = kl; k < S; k += span) mx = fmaxf(mx, __ldg(lp + (int64_t)k * rows_per_seq));
+        for (int o = span >> 1; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        float den = 0.f;
+        for (int k = kl; k < S; k += span) {
+            const float e = mx > -INFINITY ? expf(__ldg(lp + (int64_t)k * rows_per_seq) - mx) : 0.f;
+            den += e;
+            if (have && k < kc) sw[i * kc + k] = e;
         }
+        for (int o = span >> 1; o > 0; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
+        if (have && kl == 0) { smax[i] = mx; sden[i] = den; }
     }
+    __syncthreads();
+
+    const int64_t b = r / rows_per_seq;
+    const int64_t kstride = (int64_t)rows_per_seq * d_out;
+    const float* op = o_part + (b * (S - 1) * rows_per_seq + r) * d_out + c;
+    float4 acc[kF4];
+#pragma unroll
+    for (int u = 0; u < kF4; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k0 = 0; k0 < S; k0 += kc) {
+        if (k0 > 0) {  // more slots than the staging holds: the next ones
+            __syncthreads();
+            for (int i = tid; i < n_rows * kc; i += kCombineThreads) {
+                const int row = i / kc, k = k0 + i % kc;
+                const int64_t bb = (row0 + row) / rows_per_seq;
+                const float mx = smax[row];
+                sw[i] = k < S && mx > -INFINITY
+                            ? expf(__ldg(lse_part + (bb * (S - 1) + k) * rows_per_seq + row0 + row) - mx) : 0.f;
+            }
+            __syncthreads();
+        }
+        const int ke = k0 + kc < S ? kc : S - k0;
+        if (active)
+            for (int k = grp; k < ke; k += kAhead * G) {
+                float w[kAhead];
+                float4 x[kAhead][kF4];
+#pragma unroll
+                for (int a = 0; a < kAhead; ++a) {
+                    w[a] = k + a * G < ke ? sw[rl * kc + k + a * G] : 0.f;
+                    if (w[a] != 0.f) {  // an empty split's partial is never read
+#pragma unroll
+                        for (int u = 0; u < kF4; ++u) x[a][u] = ld_stream4(op + (k0 + k + a * G) * kstride + 4 * per_row * u);
+                    }
+                }
+#pragma unroll
+                for (int a = 0; a < kAhead; ++a)
+                    if (w[a] != 0.f) {
+#pragma unroll
+                        for (int u = 0; u < kF4; ++u) {
+                            acc[u].x = fmaf(w[a], x[a][u].x, acc[u].x);
+                            acc[u].y = fmaf(w[a], x[a][u].y, acc[u].y);
+                            acc[u].z = fmaf(w[a], x[a][u].z, acc[u].z);
+                            acc[u].w = fmaf(w[a], x[a][u].w, acc[u].w);
+                        }
+                    }
+            }
+    }
+    if constexpr (G > 1) {
+        if (grp > 0) {
+#pragma unroll
+            for (int u = 0; u < kF4; ++u) red[((grp - 1) * kF4 + u) * kItems + it] = acc[u];
+        }
+        __syncthreads();
+        if (grp > 0) return;
+#pragma unroll
+        for (int g = 0; g < G - 1; ++g)
+#pragma unroll
+            for (int u = 0; u < kF4; ++u) {
+                const float4 x = red[(g * kF4 + u) * kItems + it];
+                acc[u].x += x.x; acc[u].y += x.y; acc[u].z += x.z; acc[u].w += x.w;
+            }
+    }
+    if (!active) return;
+    const float den = sden[rl], mx = smax[rl];
     const float inv = den > 0.f ? 1.f / den : 0.f;
 #pragma unroll
-    for (int u = 0; u < V / 4; ++u) {
+    for (int u = 0; u < kF4; ++u) {
         acc[u].x *= inv; acc[u].y *= inv; acc[u].z *= inv; acc[u].w *= inv;
+        store4(out + r * d_out + c + 4 * per_row * u, acc[u]);
     }
-    if constexpr (V >= 8 && sizeof(TO) == 2) {  // eight bf16 per 16-byte store
-#pragma unroll
-        for (int u = 0; u < V / 8; ++u) {
-            __nv_bfloat162 h0 = __floats2bfloat162_rn(acc[2 * u].x, acc[2 * u].y), h1 = __floats2bfloat162_rn(acc[2 * u].z, acc[2 * u].w);
-            __nv_bfloat162 h2 = __floats2bfloat162_rn(acc[2 * u + 1].x, acc[2 * u + 1].y),
-                           h3 = __floats2bfloat162_rn(acc[2 * u + 1].z, acc[2 * u + 1].w);
-            uint4 u4;
-            u4.x = *reinterpret_cast<uint32_t*>(&h0);
-            u4.y = *reinterpret_cast<uint32_t*>(&h1);
-            u4.z = *reinterpret_cast<uint32_t*>(&h2);
-            u4.w = *reinterpret_cast<uint32_t*>(&h3);
-            *reinterpret_cast<uint4*>(out + r * d_out + c + 8 * u) = u4;
-        }
-    } else {
-#pragma unroll
-        for (int u = 0; u < V / 4; ++u) store4(out + r * d_out + c + 4 * u, acc[u]);
-    }
-    if (lse != nullptr && c == 0) lse[r] = dead ? -INFINITY : mx + logf(den);
+    if (lse != nullptr && c == 0) lse[r] = mx > -INFINITY ? mx + logf(den) : -INFINITY;
 }
 
 // q_hat[row, r] = sum_d W_UK[j][r][d] * q_c[row, d]  (r < r_kv);  q_hat[row, r_kv + d] = q_r[row, d].

@@ -24,6 +24,9 @@ gqla_status check_dims(const gqla_dims* d) {
 }
 gqla_status check_dtype(gqla_dtype t) { return (t == GQLA_BF16 || t == GQLA_F32) ? GQLA_OK : GQLA_ERR_DTYPE; }
 
+// gqla_combine_splits: grids of up to this many threads get narrower items and split slots
+constexpr int64_t kCombineFewThreads = 65536;
+
 gqla_status launch_status() { return cudaGetLastError() == cudaSuccess ? GQLA_OK : GQLA_ERR_CUDA; }
 
 gqla_status launch_decode_generic(gqla_dtype dtype, const DecodeArgs& a, cudaStream_t st) {
@@ -474,19 +477,30 @@ gqla_status gqla_combine_splits(int32_t B, int32_t rows_per_seq, int32_t num_spl
     if (rows > 0x7fffffffLL) return GQLA_ERR_SHAPE;
     cudaStream_t st = (cudaStream_t)stream;
     if (d_out % 4 == 0) {
-        const int vec = d_out % 16 == 0 ? 16 : (d_out % 8 == 0 ? 8 : 4);  // output columns per thread
+        // Columns per thread (V) and thread groups that share a row's slots (G): the widest item while it still gives
+        // half of the threads that fit beside a decode kernel's CTAs (such a grid is resident as one wave while it
+        // waits for them), narrower ones and split slots below that, where the chain of loads is what takes the time.
+        int vec = d_out % 16 == 0 ? 16 : (d_out % 8 == 0 ? 8 : 4);
+        while (vec > 4 && rows * (d_out / vec) <= kCombineFewThreads) vec /= 2;
+        int groups = 1;
+        while (vec == 4 && groups < 8 && 2 * groups <= num_splits && rows * (d_out / 4) * groups <= 2 * kCombineFewThreads) groups *= 2;
         const int64_t items = rows * (d_out / vec);
-        const int64_t nblk = (items + 255) / 256;
+        const int64_t nblk = (items * groups + kCombineThreads - 1) / kCombineThreads;
         if (nblk > 0x7fffffffLL) return GQLA_ERR_SHAPE;
-        const dim3 blocks((unsigned)nblk), threads(256);
+        const dim3 blocks((unsigned)nblk), threads(kCombineThreads);
         const bool bf = out_dtype == GQLA_BF16;
         cudaError_t e;
-#define GQLA_COMBINE(TO, V)                                                                                              \
-    e = tc::launch_pdl(combine_vec_kernel<TO, V>, blocks, threads, 0, st, rows, rows_per_seq, num_splits, d_out, o_part, \
-                       lse_part, (TO*)out, lse)
-        if (vec == 16) { if (bf) GQLA_COMBINE(__nv_bfloat16, 16); else GQLA_COMBINE(float, 16); }
-        else if (vec == 8) { if (bf) GQLA_COMBINE(__nv_bfloat16, 8); else GQLA_COMBINE(float, 8); }
-        else { if (bf) GQLA_COMBINE(__nv_bfloat16, 4); else GQLA_COMBINE(float, 4); }
+#define GQLA_COMBINE(V, G)                                                                                                   \
+    e = bf ? tc::launch_pdl(combine_vec_kernel<__nv_bfloat16, V, G>, blocks, threads, 0, st, rows, rows_per_seq, num_splits, \
+                            d_out, o_part, lse_part, (__nv_bfloat16*)out, lse)                                               \
+           : tc::launch_pdl(combine_vec_kernel<float, V, G>, blocks, threads, 0, st, rows, rows_per_seq, num_splits, d_out,  \
+                            o_part, lse_part, (float*)out, lse)
+        if (vec == 16) GQLA_COMBINE(16, 1);
+        else if (vec == 8) GQLA_COMBINE(8, 1);
+        else if (groups == 1) GQLA_COMBINE(4, 1);
+        else if (groups == 2) GQLA_COMBINE(4, 2);
+        else if (groups == 4) GQLA_COMBINE(4, 4);
+        else GQLA_COMBINE(4, 8);
 #undef GQLA_COMBINE
         return e == cudaSuccess ? GQLA_OK : GQLA_ERR_CUDA;
     }

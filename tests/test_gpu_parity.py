@@ -759,3 +759,33 @@ def test_c4_long_context_split_sweep(s_q):
         gq = dec.gqa_step(q, S).float().cpu().numpy()[b:b + 1]
         assert_close(gq, ref_g, f"C4 gqa S={S}")
     dec.check_status()
+
+
+@pytest.mark.parametrize("rows,S,d_out", [(1, 1, 4), (3, 2, 4), (131, 13, 128), (128, 8, 512), (2050, 5, 128), (300, 20, 512), (37, 70, 24),
+                                          (7, 1100, 16), (300, 40, 4), (8200, 2, 128), (16500, 3, 128)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_split_merge_over_the_ways_it_is_cut(rows, S, d_out, dtype):
+    """Column widths, slot groups and weight staging of the merge change with rows x d_out and the slot count; rows that
+    share a block belong to different sequences, empty slots hold NaN partials (never read), one row has no live slot.
+    fp32 sums of S terms: |error| <= (S + 8) * 2^-24 * max|o| (expf is good to 2 ulp), plus the
+    rounding of the result (at most 2^-8 of it in bf16)."""
+    from oracle import gqla_oracle as O
+    from tests.parity_util import assert_close
+    g = torch.Generator().manual_seed(rows * 1000 + S)
+    per_seq = 1 if rows % 2 else 2
+    Bn = rows // per_seq
+    o_part = torch.randn((Bn, S, per_seq, d_out), generator=g)
+    lse = 3 * torch.randn((Bn, S, per_seq), generator=g)
+    dead = torch.rand(lse.shape, generator=g) < 0.3
+    dead[Bn // 2] = True
+    lse[dead] = -np.inf
+    o_part[dead] = np.nan
+    out = torch.empty((Bn, 1, per_seq, d_out), dtype=dtype, device="cuda")
+    lse_out = torch.empty((Bn, 1, per_seq), device="cuda")
+    B.gqla_combine_splits(o_part.cuda().view(Bn, S, 1, per_seq, d_out), lse.cuda().view(Bn, S, 1, per_seq), out, lse_out)
+    clean = torch.nan_to_num(o_part).double().numpy()
+    o_ref, l_ref = O.combine_splits(clean.reshape(Bn, S, 1, per_seq, d_out), lse.double().numpy().reshape(Bn, S, 1, per_seq))
+    u = (S + 8) * 2.0 ** -24
+    assert_close(out.double().cpu().numpy(), o_ref, "merge", rel=2.0 ** -8 if dtype == torch.bfloat16 else 0.0,
+                 abs_=u * float(np.abs(clean).max()))
+    assert_close(lse_out.double().cpu().numpy(), l_ref, "merge lse", rel=u, abs_=2.0 ** -22)
