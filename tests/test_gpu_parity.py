@@ -789,3 +789,27 @@ def test_split_merge_over_the_ways_it_is_cut(rows, S, d_out, dtype):
     assert_close(out.double().cpu().numpy(), o_ref, "merge", rel=2.0 ** -8 if dtype == torch.bfloat16 else 0.0,
                  abs_=u * float(np.abs(clean).max()))
     assert_close(lse_out.double().cpu().numpy(), l_ref, "merge lse", rel=u, abs_=2.0 ** -22)
+
+
+@pytest.mark.parametrize("h_q,g,Bn,s_q,S", [(128, 8, 1, 1, 2), (128, 8, 5, 2, 4), (28, 4, 9, 1, 3), (32, 8, 35, 1, 64), (64, 8, 3, 3, 17), (8, 8, 70, 1, 9)])
+def test_fused_merge_up_projection_over_slots(h_q, g, Bn, s_q, S):
+    """Every builder warp's rows, padded head slots, slot counts up to the most the kernel stages; empty slots hold NaN."""
+    from oracle import gqla_oracle as O
+    from tests.parity_util import assert_close
+    gen = torch.Generator().manual_seed(h_q * S)
+    o_part = torch.randn((Bn, S, s_q, h_q, 512), generator=gen)
+    lse = 3 * torch.randn((Bn, S, s_q, h_q), generator=gen)
+    dead = torch.rand(lse.shape, generator=gen) < 0.4
+    dead[Bn - 1, :, 0, 0] = True
+    lse[dead] = -np.inf
+    o_part[dead] = np.nan
+    w_uv = (torch.randn((g, 512, 128), generator=gen) / 512 ** 0.5).bfloat16()
+    o = torch.empty((Bn, s_q, h_q, 128), dtype=torch.bfloat16, device="cuda")
+    lse_out = torch.empty((Bn, s_q, h_q), device="cuda")
+    bd = B.make_dims(h_q, g, 128, 512, 64)
+    assert B.kernel_for(bd, torch.bfloat16, s_q, "projections") == "tcgen05"
+    B.gqla_combine_up_proj(bd, o_part.cuda(), lse.cuda(), w_uv.cuda(), o, lse_out)
+    oh, l_ref = O.combine_splits(torch.nan_to_num(o_part).double().numpy(), lse.double().numpy())
+    ref = O.up_proj(O.Dims(h_q, g, 128, 512, 64), oh, synth.to_f64(w_uv))
+    assert_close(o.float().cpu().numpy(), ref, "combine_up_proj")
+    assert_close(lse_out.cpu().numpy(), l_ref, "lse", rel=1e-5, abs_=1e-5)
