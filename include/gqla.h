@@ -198,9 +198,13 @@ gqla_status gqla_decode_gqa_noalloc(const gqla_dims* dims, gqla_dtype dtype, int
  * with block_table an int32 [B, max_pages] device array whose entries below ceil(seqlens[b] / page_size)
  * must name pages inside the cache (page * page_size + page_size <= cache_rows / n_rows); later entries
  * are never read.  Everything else is as for gqla_decode_absorb / gqla_decode_gqa, and the outputs are
- * the same as for the packed cache holding the same rows.  The tensor-core kernels take page sizes that
- * are multiples of 128 rows with num_splits == 1 or the balanced plan (num_splits <= -2); other
- * combinations run on the generic kernels. */
+ * the same as for the packed cache holding the same rows (rows of a sequence's last page behind its end
+ * must hold finite values, as rows outside a sequence do there).  With a page size that is a multiple of
+ * 128 rows and num_splits == 1 or the balanced plan (num_splits <= -2) the tensor-core kernels run as over
+ * a packed cache.  Other page sizes that are a multiple of 16, and num_splits >= 2, run on forms of them
+ * that fetch by pages and keep the probabilities to 16 bits (on the absorb path with 33 to 64 query rows
+ * the balanced plan is then cut for half the SMs per 128 query rows, as in gqla_decode_absorb_fp8; on the
+ * GQA path up to 32 padded query rows per group); everything else runs on the generic kernels. */
 gqla_status gqla_decode_absorb_paged(const gqla_dims* dims, gqla_dtype dtype, int32_t B, int32_t s_q, float scale,
                                      int32_t num_splits, const void* q_hat, const void* cache,
                                      int64_t cache_row_stride, int64_t cache_rows, const int32_t* block_table,

@@ -36,6 +36,11 @@ struct RowMap {
         if (block_table == nullptr) return seq_start[b] + t;
         return (int64_t)block_table[(int64_t)b * max_pages + t / page_size] * page_size + t % page_size;
     }
+    // First cache row of a run of rows t.. that lies within one page; `beyond` where the sequence (T rows) has ended:
+    // the block table says nothing about pages behind it.
+    __device__ __forceinline__ int32_t run_row(int32_t b, int32_t t, int32_t T, int32_t beyond) const {
+        return t < T ? (int32_t)row(b, t) : beyond;
+    }
 };
 
 // FP8 E4M3 storage (4 exponent bits, bias 7; 3 mantissa bits; no infinity; largest finite value 448).

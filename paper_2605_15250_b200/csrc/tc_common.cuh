@@ -446,6 +446,10 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&v);
 }
+// What the bf16 pair `hi` of (lo, hi) values left over, as a second bf16 pair: value = hi term + rest to 16 bits.
+__device__ __forceinline__ uint32_t pack_bf16_rest(float x0, float x1, uint32_t hi) {
+    return pack_bf16(x0 - __uint_as_float(hi << 16), x1 - __uint_as_float(hi & 0xffff0000u));
+}
 
 // ----------------------------------------------------------------------------- host: tensor maps
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,

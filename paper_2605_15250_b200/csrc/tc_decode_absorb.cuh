@@ -27,6 +27,14 @@
 // warps 2-9 softmax, warp 10 TMA producer of V.  A softmax thread owns one TMEM lane = (row, token half)
 // and one half of that lane's 64 score columns, so a row's 128 scores of a tile sit in four threads of
 // four different warps; they share the tile maximum through shared memory and keep separate partial sums.
+//
+// Small pages (template parameter PG = rows of a box: 64, 32 or 16; 0 = the form above).  A paged cache whose pages are
+// no multiple of the 128-row tile is fetched in boxes of PG rows that no page boundary cuts (PG divides the page size
+// and the tile's halves): the boxes of a group go out together, one lane of the producer warp each, after every lane has
+// looked its page up; boxes behind the sequence's end start behind the cache's last row and are filled with zeros.  Such
+// calls keep 32-bit probabilities: P is split into two bf16 terms (hi + lo, 16 bits) and P V is issued for both, the
+// second P buffer taking the place of one K group.  These calls ran one warp per query row on the SIMT kernel before,
+// which read every cache row h_q times from L2: 13.7 ms for 32 sequences of 300-8000 rows in pages of 64 rows.
 #pragma once
 #include "common.cuh"
 #include "sched.cuh"
@@ -39,22 +47,26 @@ struct AbsorbParams {
     int32_t B, S, s_q, h_q, rows_total /* s_q*h_q */, row_blocks /* ceil(rows_total/128) */;
     int32_t balanced, W;  // balanced plan: W pairs per row block, grid = 2 * W * row_blocks
     float scale_log2;
-    RowMap rows;      // packed or paged (pages a multiple of 128 rows, pieces starting on tile boundaries)
+    RowMap rows;      // packed or paged (PG = 0: pages a multiple of 128 rows, pieces starting on tile boundaries)
     const int32_t* seqlens;
     float* o_part;    // [B, S, s_q*h_q, 512]
     float* lse_part;  // [B, S, s_q*h_q]
     __nv_bfloat16* o_final;  // not null: S = 1, fixed plan; the normalised output goes here as bf16 [B, s_q*h_q, 512]
                              // (o_part unused, lse_part may be null)
     int32_t* status;
+    int32_t n_rows;   // rows of the cache (small pages: where the zero-filled boxes start)
 };
 
-struct AbsorbSmem {
+template <int PG>
+struct AbsorbSmemT {
     static constexpr int kBox = 8192;              // 64 rows x 64 bf16, 128-byte swizzle
     static constexpr int kQBytes = 9 * kBox;       // 64 query rows x 576
-    static constexpr int kPBytes = 2 * kBox;       // 64 rows x 128 tokens (two 64-token k-blocks)
+    static constexpr int kPTerms = PG != 0 ? 2 : 1;  // bf16 terms of a probability
+    static constexpr int kPTerm = 2 * kBox;        // 64 rows x 128 tokens (two 64-token k-blocks)
+    static constexpr int kPBytes = kPTerms * kPTerm;
     static constexpr int kKGroup = 3 * kBox;       // three column blocks of this CTA's 64 rows of a tile
     static constexpr int kVGroup = 4 * kBox;       // 64 tokens x this CTA's 2 x 128 latent columns
-    static constexpr int kNK = 3;                  // ring of K groups (Qh Kh^T operand): one tile
+    static constexpr int kNK = PG != 0 ? 2 : 3;    // ring of K groups (Qh Kh^T operand): one tile
     static constexpr int kNV = 2;                  // ring of V groups (P V operand): one tile
     static constexpr int kOffK = kQBytes;
     static constexpr int kOffP = kOffK + kNK * kKGroup;
@@ -76,16 +88,18 @@ struct AbsorbSmem {
     static_assert(2 * 4 * 64 >= kThreads + 4, "plan scratch must fit in sm_max");
     static_assert(kTotal <= 232448, "shared memory budget of one CTA");
     static_assert(OneCtaPerSM<kTotal>::value, "");
+    static_assert(PG == 0 || PG == 64 || PG == 32 || PG == 16, "");
 };
+using AbsorbSmem = AbsorbSmemT<0>;
 
 constexpr uint32_t kAColO = 0;    // O: MMA m (latent columns [256m, 256m+256)) at TMEM columns [128m, 128m+128)
 constexpr uint32_t kAColS = 256;  // two 64-column score buffers
 
-template <int DUMMY>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(AbsorbSmem::kThreads, 1)
+template <int PG>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(AbsorbSmemT<PG>::kThreads, 1)
 decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap tmQ,
                         const __grid_constant__ CUtensorMap tmC) {
-    using L = AbsorbSmem;
+    using L = AbsorbSmemT<PG>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* tiles = smem_raw;
     if ((smem_u32(tiles) & 1023u) != 0) {  // swizzled tiles need 1 KB alignment; same answer in both CTAs
@@ -159,7 +173,39 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer of Q and the K ring
         // (both CTAs).  Every "full" barrier lives in the leader and counts the bytes of BOTH CTAs.
-        if (elect_one()) {
+        if constexpr (PG != 0) {
+            constexpr int NB = 64 / PG;  // boxes per column block of this CTA's 64 rows
+            const int run = lane % NB, blk = lane / NB;
+            const uint32_t q_full_l = mapa(smem_u32(q_full), 0);
+            int ks = 0;
+            uint32_t kph = 1;
+            bool ok = true;
+            while (ok && walk.next(pc)) {
+                if (pc.n_tiles == 0) continue;
+                const int32_t T = p.seqlens[pc.b];
+                if (pi > 0 && !(ok = __all_sync(0xffffffffu, mbar_wait(q_empty, (pi - 1) & 1, ab, 13)))) break;
+                if (cta == 0 && lane == 0) mbar_expect_tx(q_full, 2 * L::kQBytes);
+                __syncwarp();
+                if (lane < 9) tma_load_2d_pair(tiles + lane * L::kBox, &tmQ, lane * 64, pc.b * p.rows_total + rho0, q_full_l);
+                const int32_t tok = pc.tok_begin + (int)cta * 64 + run * PG;  // this lane's run of rows in the first tile
+                int32_t next_row = p.rows.run_row(pc.b, tok, T, p.n_rows);
+                for (int kt = 0; kt < pc.n_tiles && ok; ++kt) {
+                    const int32_t row = next_row;
+                    if (kt + 1 < pc.n_tiles) next_row = p.rows.run_row(pc.b, tok + (kt + 1) * 128, T, p.n_rows);
+#pragma unroll 1
+                    for (int kg = 0; kg < 3; ++kg) {
+                        if (!(ok = __all_sync(0xffffffffu, mbar_wait(&kempty[ks], kph, ab, 1)))) break;
+                        if (cta == 0 && lane == 0) mbar_expect_tx(&kfull[ks], 2 * L::kKGroup);
+                        __syncwarp();
+                        if (blk < 3)
+                            tma_load_2d_pair(tiles + L::kOffK + ks * L::kKGroup + blk * L::kBox + run * PG * 128, &tmC,
+                                             (3 * kg + blk) * 64, row, mapa(smem_u32(&kfull[ks]), 0));
+                        if (++ks == L::kNK) { ks = 0; kph ^= 1; }
+                    }
+                }
+                ++pi;
+            }
+        } else if (elect_one()) {
             tma_prefetch_desc(&tmQ);
             tma_prefetch_desc(&tmC);
             const uint32_t q_full_l = mapa(smem_u32(q_full), 0);
@@ -200,7 +246,32 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
         // the two rings are fed by two threads.  V groups in the order (tile, token half); a V slot is free
         // only after P.V of the previous tile, i.e. after Qh Kh^T of this tile has read the same cache rows
         // as K boxes, so the V boxes come out of L2.
-        if (elect_one()) {
+        if constexpr (PG != 0) {
+            constexpr int NB = 64 / PG;
+            const int run = lane % NB, mi = lane / NB;
+            int vs = 0;
+            uint32_t vph = 1;
+            bool ok = true;
+            while (ok && walk.next(pc)) {
+                if (pc.n_tiles == 0) continue;
+                const int32_t T = p.seqlens[pc.b];
+                if (pi > 0 && !(ok = __all_sync(0xffffffffu, mbar_wait(epi_done, (pi - 1) & 1, ab, 16)))) break;
+                const int32_t tok = pc.tok_begin + run * PG;
+                int32_t next_row = p.rows.run_row(pc.b, tok, T, p.n_rows);
+                for (int vg = 0; vg < 2 * pc.n_tiles; ++vg) {  // (tile, token half)
+                    const int32_t row = next_row;
+                    if (vg + 1 < 2 * pc.n_tiles) next_row = p.rows.run_row(pc.b, tok + (vg + 1) * 64, T, p.n_rows);
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(&vempty[vs], vph, ab, 2)))) break;
+                    if (cta == 0 && lane == 0) mbar_expect_tx(&vfull[vs], 2 * L::kVGroup);
+                    __syncwarp();
+                    if (mi < 4)
+                        tma_load_2d_pair(tiles + L::kOffV + vs * L::kVGroup + mi * L::kBox + run * PG * 128, &tmC,
+                                         256 * (mi >> 1) + 128 * (int)cta + 64 * (mi & 1), row, mapa(smem_u32(&vfull[vs]), 0));
+                    if (++vs == L::kNV) { vs = 0; vph ^= 1; }
+                }
+                ++pi;
+            }
+        } else if (elect_one()) {
             int vs = 0;
             uint32_t vph = 1;
             bool ok = true;
@@ -300,6 +371,12 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
 #pragma unroll
                             for (int kk = 1; kk < 4; ++kk)
                                 umma_ss2_lo<true>(dm, pd + ((kk * 32) >> 4), vd + ((m * 2 * L::kBox + kk * 2048) >> 4), idesc_pv);
+                            if constexpr (L::kPTerms == 2) {
+#pragma unroll
+                                for (int kk = 0; kk < 4; ++kk)
+                                    umma_ss2_lo<true>(dm, pd + ((L::kPTerm + kk * 32) >> 4),
+                                                      vd + ((m * 2 * L::kBox + kk * 2048) >> 4), idesc_pv);
+                            }
                         }
                         umma_commit2(&vempty[vs], 3);
                         if (++vs == L::kNV) { vs = 0; vph ^= 1; }
@@ -384,7 +461,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                     m_used = m_t;
                 }
                 const float m_sub = m_used == -INFINITY ? 0.f : m_used;
-                uint32_t pk[16];
+                uint32_t pk[16], pl[L::kPTerms == 2 ? 16 : 1];
                 if (full) {
 #pragma unroll
                     for (int c = 0; c < 32; c += 2) {
@@ -392,6 +469,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                         const float e1 = ex2(fmaf(__uint_as_float(x[c + 1]), p.scale_log2, -m_sub));
                         l += e0 + e1;
                         pk[c / 2] = pack_bf16(e0, e1);
+                        if constexpr (L::kPTerms == 2) pl[c / 2] = pack_bf16_rest(e0, e1, pk[c / 2]);
                     }
                 } else {
 #pragma unroll
@@ -401,6 +479,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                             tok0 + c + 1 < lim ? ex2(fmaf(__uint_as_float(x[c + 1]), p.scale_log2, -m_sub)) : 0.f;
                         l += e0 + e1;
                         pk[c / 2] = pack_bf16(e0, e1);
+                        if constexpr (L::kPTerms == 2) pl[c / 2] = pack_bf16_rest(e0, e1, pk[c / 2]);
                     }
                 }
                 // O may be rescaled, and the P buffer rewritten, only once P.V(n-1) has completed
@@ -429,6 +508,12 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 for (int c4 = 0; c4 < 4; ++c4)
                     *reinterpret_cast<uint4*>(prow + (((ch * 4 + c4) ^ (r & 7)) << 4)) =
                         make_uint4(pk[4 * c4], pk[4 * c4 + 1], pk[4 * c4 + 2], pk[4 * c4 + 3]);
+                if constexpr (L::kPTerms == 2) {
+#pragma unroll
+                    for (int c4 = 0; c4 < 4; ++c4)
+                        *reinterpret_cast<uint4*>(prow + L::kPTerm + (((ch * 4 + c4) ^ (r & 7)) << 4)) =
+                            make_uint4(pl[4 * c4], pl[4 * c4 + 1], pl[4 * c4 + 2], pl[4 * c4 + 3]);
+                }
                 fence_proxy_async_smem();  // generic-proxy writes of P -> visible to the tensor core
                 tc_fence_before();
                 __syncwarp();

@@ -36,7 +36,9 @@
 namespace gqla {
 namespace tc {
 
-template <int R>
+// PG: rows of a box for caches in small pages, 0 otherwise (see tc_decode_absorb.cuh: boxes within pages, probabilities in
+// two bf16 terms).  With 64 query rows the second term does not fit; the pair kernel serves those calls.
+template <int R, int PG = 0>
 struct AbsorbTSmem {
     static constexpr int kTile = 64;                          // tokens per tile
     static constexpr int kQBlock = R * 128;                   // one k-block of Qh: R rows x 64 bf16
@@ -46,7 +48,9 @@ struct AbsorbTSmem {
     static constexpr int kStages = 2;
     static constexpr int kPRow = 2 * R;                       // one token's R probabilities (bf16)
     static constexpr int kPSwzBits = R == 64 ? 3 : (R == 32 ? 2 : 1);  // swizzle span = row length (128 / 64 / 32 bytes)
-    static constexpr int kPBuf = (kTile * kPRow + 1023) / 1024 * 1024;
+    static constexpr int kPTerms = PG != 0 ? 2 : 1;           // bf16 terms of a probability
+    static constexpr int kPTerm = (kTile * kPRow + 1023) / 1024 * 1024;
+    static constexpr int kPBuf = kPTerms * kPTerm;
     static constexpr int kPBufs = R == 64 ? 1 : 2;            // P^T buffers (one where Qh takes 72 KB: P(n) waits for P.V(n-1))
     static constexpr int kGroup = 3 * kBox;                   // boxes land in groups of three, one barrier each
     static constexpr int kOffStage = kQBytes;
@@ -72,10 +76,10 @@ struct AbsorbTSmem {
 constexpr int kPrefetchAhead = GQLA_ABSORB_T_PREFETCH;  // tiles between a load and the L2 prefetch issued with it
 constexpr uint32_t kPollSpins = 1u << 25;  // polls of the MMA issuer without progress before it gives up
 
-template <int R>
-__global__ void __launch_bounds__(AbsorbTSmem<R>::kThreads, 1)
+template <int R, int PG = 0>
+__global__ void __launch_bounds__(AbsorbTSmem<R, PG>::kThreads, 1)
 decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmC) {
-    using L = AbsorbTSmem<R>;
+    using L = AbsorbTSmem<R, PG>;
     constexpr int RW = L::kRowsPerWarp;
     constexpr int NJ = RW / 4;  // query rows per softmax thread
     constexpr int kSmT = 32 * L::kSoftmaxWarps;
@@ -139,7 +143,42 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (elect_one()) {
+        if constexpr (PG != 0) {
+            constexpr int NB = TK / PG;  // boxes per column block of a tile; one lane of the warp each
+            const int run = lane % NB, blk = lane / NB;
+            bool ok = true;
+            while (ok && walk.next(pc)) {
+                if (pc.n_tiles == 0) continue;
+                const int nt = (pc.tok_end - pc.tok_begin + TK - 1) / TK;
+                const int32_t T = p.seqlens[pc.b], tok = pc.tok_begin + run * PG;
+                if (pi > 0 && !(ok = __all_sync(0xffffffffu, mbar_wait(q_empty, (pi - 1) & 1, ab, 13)))) break;
+                if (lane == 0) mbar_expect_tx(q_full, L::kQBytes);
+                __syncwarp();
+                if (lane < 9) tma_load_2d(q_smem + lane * L::kQBlock, &tmQ, lane * 64, pc.b * p.rows_total, q_full);
+                // rows of this tile, the next and the one that is asked into L2 (looked up two tiles ahead)
+                int32_t row = p.rows.run_row(pc.b, tok, T, p.n_rows), row1 = p.rows.run_row(pc.b, tok + TK, T, p.n_rows);
+                for (int t = 0; t < nt; ++t, ++gt) {
+                    const int s = gt & 1;
+                    const int32_t row2 = p.rows.run_row(pc.b, tok + (t + 2) * TK, T, p.n_rows);
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(&empty[s], ((gt >> 1) & 1) ^ 1, ab, 1)))) break;
+#pragma unroll
+                    for (int g = 0; g < 3; ++g) {
+                        if (lane == 0) mbar_expect_tx(&full[s * 3 + g], L::kGroup);
+                        __syncwarp();
+                        if (blk < 3)
+                            tma_load_2d(stage0 + s * L::kStageBytes + (3 * g + blk) * L::kBox + run * PG * 128, &tmC,
+                                        (3 * g + blk) * 64, row, &full[s * 3 + g]);
+                    }
+                    if (blk < 3 && t + 2 < nt && row2 != p.n_rows) {
+#pragma unroll
+                        for (int g = 0; g < 3; ++g) tma_prefetch_l2_2d(&tmC, (3 * g + blk) * 64, row2);
+                    }
+                    row = row1;
+                    row1 = row2;
+                }
+                ++pi;
+            }
+        } else if (elect_one()) {
             tma_prefetch_desc(&tmQ);
             tma_prefetch_desc(&tmC);
             bool ok = true;
@@ -212,6 +251,14 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                                     for (int ks = 0; ks < 4; ++ks)  // 16 tokens per step
                                         umma_ss_lo(tmem_base + kColO + m * R, v_lo + ((2 * m * L::kBox + ks * 2048) >> 4), v_hi,
                                                    p_lo + ((ks * 16 * L::kPRow) >> 4), p_hi, idesc_pv, (pv_tile | ks) != 0);
+                                if constexpr (L::kPTerms == 2) {
+#pragma unroll
+                                    for (int m = 0; m < 4; ++m)
+#pragma unroll
+                                        for (int ks = 0; ks < 4; ++ks)
+                                            umma_ss_lo(tmem_base + kColO + m * R, v_lo + ((2 * m * L::kBox + ks * 2048) >> 4),
+                                                       v_hi, p_lo + ((L::kPTerm + ks * 16 * L::kPRow) >> 4), p_hi, idesc_pv, 1);
+                                }
                                 umma_commit(&empty[s]);
                                 umma_commit(&pv_done[s]);
                                 ++pv_tile;
@@ -368,6 +415,7 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                 // probabilities: a bf16 pair (the thread's two rows) into each of its two tokens' rows of P^T
                 const int pbi = n % L::kPBufs;
                 uint32_t pk[NJ];  // [2 h + pair]: the bf16 pair of token h for the thread's row pair
+                uint32_t pl[NJ];  // (small pages) the pair's second term
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -378,6 +426,8 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                         l[jp] += e0;
                         l[jp + 1] += e1;
                         pk[(NJ / 2) * h + (jp >> 1)] = pack_bf16(e0, e1);
+                        if constexpr (L::kPTerms == 2)
+                            pl[(NJ / 2) * h + (jp >> 1)] = pack_bf16_rest(e0, e1, pk[(NJ / 2) * h + (jp >> 1)]);
                     }
                 // a single P^T buffer is still being read by P.V(n-1)
                 if (L::kPBufs == 1 && t > 0 && okl)
@@ -389,8 +439,10 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
 #pragma unroll
                     for (int jp = 0; jp < NJ; jp += 2) {
                         const uint32_t col = (uint32_t)(r0 + rj(jp)) * 2;                      // byte of that row pair in it
-                        *reinterpret_cast<uint32_t*>(p_smem + pbi * L::kPBuf + off + (((col >> 4) ^ pswz) << 4) + (col & 15)) =
-                            pk[(NJ / 2) * h + (jp >> 1)];
+                        uint8_t* dst = p_smem + pbi * L::kPBuf + off + (((col >> 4) ^ pswz) << 4) + (col & 15);
+                        *reinterpret_cast<uint32_t*>(dst) = pk[(NJ / 2) * h + (jp >> 1)];
+                        if constexpr (L::kPTerms == 2)
+                            *reinterpret_cast<uint32_t*>(dst + L::kPTerm) = pl[(NJ / 2) * h + (jp >> 1)];
                     }
                 }
                 fence_proxy_async_smem();  // generic-proxy writes of P^T -> visible to the tensor core

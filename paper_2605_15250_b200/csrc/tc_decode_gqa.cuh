@@ -32,11 +32,12 @@ struct GqaParams {
     int32_t v_blocks, d_v;  // value head dim d_v = 128 * v_blocks: a CTA computes one 128-column block of the output
                             // (v_blocks = 1 unless the value head dim differs from d_h, Sec. 3.2)
     float scale_log2;
-    RowMap rows;  // packed or paged (pages a multiple of 128 rows, pieces starting on tile boundaries)
+    RowMap rows;  // packed or paged (PG = 0: pages a multiple of 128 rows, pieces starting on tile boundaries)
     const int32_t* seqlens;
     float* o_part;    // [B, S, s_q, h_q, d_v]
     float* lse_part;  // [B, S, s_q, h_q]
     int32_t* status;
+    int32_t n_rows;   // rows of the planes (small pages: where the zero-filled boxes start)
 };
 
 struct GqaSmem {

@@ -31,7 +31,9 @@
 namespace gqla {
 namespace tc {
 
-template <int R>
+// PG: rows of a box for caches in small pages, 0 otherwise (see tc_decode_absorb.cuh: boxes within pages, probabilities in
+// two bf16 terms).
+template <int R, int PG = 0>
 struct GqaTSmem {
     static constexpr int kQBlock = R * 128;                  // one k-block of Q: R rows x 64 bf16
     static constexpr int kQBytes = 3 * kQBlock;              // rounded up to 1 KB below
@@ -43,7 +45,9 @@ struct GqaTSmem {
     static constexpr int kStages = 2;
     static constexpr int kPRow = 2 * R;                      // one token's R probabilities (bf16)
     static constexpr int kPSwzBits = R == 64 ? 3 : (R == 32 ? 2 : 1);  // swizzle span = row length: 128 / 64 / 32 bytes
-    static constexpr int kPBuf = (128 * kPRow + 1023) / 1024 * 1024;   // 128 tokens, 1 KB aligned
+    static constexpr int kPTerms = PG != 0 ? 2 : 1;                    // bf16 terms of a probability
+    static constexpr int kPTerm = (128 * kPRow + 1023) / 1024 * 1024;  // 128 tokens, 1 KB aligned
+    static constexpr int kPBuf = kPTerms * kPTerm;
     static constexpr int kOffStage = kQRegion;
     static constexpr int kOffP = kOffStage + kStages * kStageBytes;
     static constexpr int kOffRed = kOffP + 2 * kPBuf;        // [4 warps][R] floats: row maxima / sums across warps
@@ -88,11 +92,11 @@ __device__ __forceinline__ void tmem_st_n(uint32_t taddr, const uint32_t* r, int
     else tmem_st16(taddr, r);
 }
 
-template <int R>
-__global__ void __launch_bounds__(GqaTSmem<R>::kThreads, 1)
+template <int R, int PG = 0>
+__global__ void __launch_bounds__(GqaTSmem<R, PG>::kThreads, 1)
 decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmV) {
-    using L = GqaTSmem<R>;
+    using L = GqaTSmem<R, PG>;
     constexpr int RW = L::kRowsPerThread;    // query rows per softmax thread (the others belong to its partner warps)
     constexpr int CH = RW;                   // rows handled per pass (TMEM columns per load)
     constexpr int NCH = RW / CH;
@@ -160,7 +164,44 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (elect_one()) {
+        if constexpr (PG != 0) {
+            constexpr int NB = 128 / PG;  // boxes per column block of a tile; one lane of the warp each
+            const int run = lane % NB, blk = lane / NB;
+            bool ok = true;
+            while (ok && walk.next(pc)) {
+                if (pc.n_tiles == 0) continue;
+                const int32_t T = p.seqlens[pc.b], tok = pc.tok_begin + run * PG;
+                if (pi > 0 && !(ok = __all_sync(0xffffffffu, mbar_wait(q_empty, (pi - 1) & 1, ab, 13)))) break;
+                if (lane == 0) mbar_expect_tx(q_full, L::kQBytes);
+                __syncwarp();
+                if (lane < 3)
+                    asm volatile(
+                        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
+                        "[%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(q_smem + lane * L::kQBlock)),
+                        "l"(reinterpret_cast<uint64_t>(&tmQ)), "r"(smem_u32(q_full)), "r"(lane * 64), "r"(0), "r"(j),
+                        "r"(pc.b * p.s_q)
+                        : "memory");
+                int32_t next_row = p.rows.run_row(pc.b, tok, T, p.n_rows);
+                for (int t = 0; t < pc.n_tiles; ++t, ++gt) {
+                    const int s = gt & 1;
+                    const uint32_t ph = (gt >> 1) & 1;
+                    uint8_t* st = stage0 + s * L::kStageBytes + blk * 16384 + run * PG * 128;
+                    const int32_t row = next_row;
+                    if (t + 1 < pc.n_tiles) next_row = p.rows.run_row(pc.b, tok + (t + 1) * 128, T, p.n_rows);
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(&kempty[s], ph ^ 1, ab, 1)))) break;
+                    if (lane == 0) mbar_expect_tx(&kfull[s], L::kKcBytes + L::kKrBytes);
+                    __syncwarp();
+                    if (blk < 2) tma_load_3d(st, &tmK, blk * 64, j, row, &kfull[s]);
+                    else if (blk == 2) tma_load_2d(st, &tmR, 0, row, &kfull[s]);
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(&vempty[s], ph ^ 1, ab, 2)))) break;
+                    if (lane == 0) mbar_expect_tx(&vfull[s], L::kVBytes);
+                    __syncwarp();
+                    if (blk < 2)
+                        tma_load_3d(st + L::kKcBytes + L::kKrBytes, &tmV, vb * 128 + blk * 64, j, row, &vfull[s]);
+                }
+                ++pi;
+            }
+        } else if (elect_one()) {
             tma_prefetch_desc(&tmQ);
             tma_prefetch_desc(&tmK);
             tma_prefetch_desc(&tmR);
@@ -248,6 +289,12 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                     for (int ks = 0; ks < 8; ++ks)  // 16 tokens per step: rows [16 ks, +16) of the V boxes and of P^T
                         umma_ss_lo(tmem_base + kColO, (uint32_t)vd + ((ks * 2048) >> 4), (uint32_t)(vd >> 32),
                                    (uint32_t)pd + ((ks * 16 * L::kPRow) >> 4), (uint32_t)(pd >> 32), idesc_pv, (uint32_t)(t | ks));
+                    if constexpr (L::kPTerms == 2) {
+#pragma unroll
+                        for (int ks = 0; ks < 8; ++ks)
+                            umma_ss_lo(tmem_base + kColO, (uint32_t)vd + ((ks * 2048) >> 4), (uint32_t)(vd >> 32),
+                                       (uint32_t)pd + ((L::kPTerm + ks * 16 * L::kPRow) >> 4), (uint32_t)(pd >> 32), idesc_pv, 1);
+                    }
                     umma_commit(&vempty[s]);
                     umma_commit(&pv_done[s]);
                 }
@@ -358,7 +405,7 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                         }
                     }
                     // probabilities of this token for the chunk's rows -> its row of P^T, eight rows per 16-byte store
-                    uint32_t pk[CH / 2];
+                    uint32_t pk[CH / 2], pl[CH / 2];
 #pragma unroll
                     for (int c = 0; c < CH; c += 2) {
                         const int rl = ch * CH + c;
@@ -367,11 +414,18 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                         l[rl] += e0;
                         l[rl + 1] += e1;
                         pk[c / 2] = pack_bf16(e0, e1);
+                        if constexpr (L::kPTerms == 2) pl[c / 2] = pack_bf16_rest(e0, e1, pk[c / 2]);
                     }
 #pragma unroll
                     for (int i = 0; i < CH / 8; ++i)
                         *reinterpret_cast<uint4*>(prow + ((((uint32_t)((r0 + ch * CH) / 8 + i)) ^ pswz) << 4)) =
                             make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
+                    if constexpr (L::kPTerms == 2) {
+#pragma unroll
+                        for (int i = 0; i < CH / 8; ++i)
+                            *reinterpret_cast<uint4*>(prow + L::kPTerm + ((((uint32_t)((r0 + ch * CH) / 8 + i)) ^ pswz) << 4)) =
+                                make_uint4(pl[4 * i], pl[4 * i + 1], pl[4 * i + 2], pl[4 * i + 3]);
+                    }
                 }
                 if (!ok) break;
                 fence_proxy_async_smem();  // generic-proxy writes of P^T -> visible to the tensor core

@@ -108,6 +108,17 @@ inline bool absorb_prefers_tokens(const gqla_dims& d, int32_t s_q) {
     return rows_t <= GQLA_ABSORB_TOKENS_MAX_ROWS;
 }
 
+// Rows per box of a paged decode call on the tensor-core kernels: 0 = the boxes of the packed form (whole tiles, which
+// need pages of a multiple of 128 rows and pieces that start on tile boundaries), 64 / 32 / 16 = the small-page form (the
+// largest that divides the page; the fixed plan's pieces start on multiples of 64 rows), -1 = neither, the generic kernels
+// serve the call.  Shuffled pages, 32 sequences of 300-8000 rows, 128 heads, whole step: 14.0 ms with pages of 64 rows on the
+// generic kernels; here 91 us on the absorb path and 119 us on the GQA path (pages of 16 rows: 94 and 150 us; of 128 rows,
+// which keep one bf16 term of a probability: 73 and 109 us).
+inline int page_box_rows(const RowMap& rows, bool on_tile_boundaries) {
+    if (!rows.paged() || (rows.page_size % kTileRows == 0 && on_tile_boundaries)) return 0;
+    return rows.page_size % 64 == 0 ? 64 : (rows.page_size % 32 == 0 ? 32 : (rows.page_size % 16 == 0 ? 16 : -1));
+}
+
 // Workers of the balanced plan on the absorb path's CTA-pair kernels (bf16 and E4M3): pairs resident at once per
 // block of 128 query rows.
 inline int32_t pair_balanced_workers(const gqla_dims& d, int32_t s_q) {
@@ -333,13 +344,24 @@ inline gqla_status tc_combine_up_proj(const gqla_dims& d, gqla_dtype dtype, int3
                : GQLA_ERR_CUDA;
 }
 
-template <int R>
+template <int R, int PG = 0>
 inline cudaError_t absorb_t_launch(const tc::AbsorbParams& p, const CUtensorMap& q, const CUtensorMap& c, unsigned grid,
                                    cudaStream_t st) {
-    auto kern = tc::decode_absorb_t_kernel<R>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::AbsorbTSmem<R>::kTotal);
+    using L = tc::AbsorbTSmem<R, PG>;
+    auto kern = tc::decode_absorb_t_kernel<R, PG>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
     if (e != cudaSuccess) return e;
-    return tc::launch_pdl(kern, dim3(grid), dim3(tc::AbsorbTSmem<R>::kThreads), tc::AbsorbTSmem<R>::kTotal, st, p, q, c);
+    return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, c);
+}
+
+template <int PG>
+inline cudaError_t absorb_pair_launch(const tc::AbsorbParams& p, const CUtensorMap& q, const CUtensorMap& c, unsigned grid,
+                                      cudaStream_t st) {
+    using L = tc::AbsorbSmemT<PG>;
+    auto kern = tc::decode_absorb_tc_kernel<PG>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
+    if (e != cudaSuccess) return e;
+    return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, c);
 }
 
 inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, float scale, int32_t S,
@@ -350,19 +372,20 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
     if (!tc_covers(d, GQLA_BF16, s_q, 0) || !stride_ok(cache_row_stride) || cache_rows > 0x7fffffffLL ||
         cache_rows < 1)
         return GQLA_ERR_UNSUPPORTED;
-    if (rows.paged() && rows.page_size % kTileRows != 0) return GQLA_ERR_UNSUPPORTED;  // a tile must not straddle pages
     const int rows_total = s_q * d.h_q;
     const int row_blocks = (rows_total + 127) / 128;
-    // S < 0: balanced plan with -S slots per sequence, W persistent pairs per row block
-    const int32_t workers = S < 0 ? tc_balanced_workers(d, s_q, 0) : 0;
+    const int rows_t = absorb_rows_t(d, s_q);
+    const bool small_pages = page_box_rows(rows, S <= 1) != 0;  // S < 0: the balanced plan's pieces start on tile boundaries
+    // two-term probabilities of 64 query rows do not fit the tokens-on-M kernel: small pages take the pair kernel there
+    const bool tokens_on_m = absorb_prefers_tokens(d, s_q) && !(small_pages && rows_t > 32);
+    // S < 0: balanced plan with -S slots per sequence, W persistent CTAs (tokens-on-M) or pairs per row block
+    const int32_t workers = S >= 0 ? 0 : (tokens_on_m ? sm_count() : pair_balanced_workers(d, s_q));
     const bool balanced = S < 0 && workers > 0;
     if (S < 0) S = -S;
-    // paged: pieces must start on tile boundaries, which the fixed plan's 64-row granule does not give for S > 1
-    if (rows.paged() && !balanced && S != 1) return GQLA_ERR_UNSUPPORTED;
+    const int pg = page_box_rows(rows, balanced || S == 1);
+    if (pg < 0 || (pg > 0 && tokens_on_m && rows_t > 32)) return GQLA_ERR_UNSUPPORTED;
     const int64_t pairs = balanced ? (int64_t)workers * row_blocks : (int64_t)B * S * row_blocks;
     if (2 * pairs > 0x7fffffffLL) return GQLA_ERR_UNSUPPORTED;
-    const bool tokens_on_m = absorb_prefers_tokens(d, s_q);
-    const int rows_t = absorb_rows_t(d, s_q);
     CUtensorMap tmQ, tmC;
     {
         const uint64_t dims[2] = {(uint64_t)(d.r_kv + d.d_r), (uint64_t)B * rows_total};
@@ -373,7 +396,7 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
     {
         const uint64_t dims[2] = {(uint64_t)(d.r_kv + d.d_r), (uint64_t)cache_rows};
         const uint64_t str[1] = {(uint64_t)cache_row_stride * 2};
-        const uint32_t box[2] = {64, 64};
+        const uint32_t box[2] = {64, pg != 0 ? (uint32_t)pg : 64u};
         if (!tc::make_tmap_bf16(&tmC, cache, 2, dims, str, box)) return GQLA_ERR_CUDA;
     }
     tc::AbsorbParams p{};
@@ -381,22 +404,27 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
     p.balanced = balanced ? 1 : 0; p.W = workers;
     p.scale_log2 = scale * 1.4426950408889634f;
     p.rows = rows; p.seqlens = seqlens; p.o_part = o_part; p.lse_part = lse_part; p.status = status;
-    p.o_final = (__nv_bfloat16*)o_final;
+    p.o_final = (__nv_bfloat16*)o_final; p.n_rows = (int32_t)cache_rows;
     if (o_final != nullptr && (balanced || S != 1)) return GQLA_ERR_UNSUPPORTED;
-    if (tokens_on_m) {
-        const unsigned grid = (unsigned)(balanced ? workers : B * S);  // single CTAs: W of them, or one per piece
-        const cudaError_t e = rows_t == 16   ? absorb_t_launch<16>(p, tmQ, tmC, grid, st)
-                              : rows_t == 32 ? absorb_t_launch<32>(p, tmQ, tmC, grid, st)
-                                             : absorb_t_launch<64>(p, tmQ, tmC, grid, st);
-        return e == cudaSuccess ? GQLA_OK : GQLA_ERR_CUDA;
-    }
-    auto kern = tc::decode_absorb_tc_kernel<0>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::AbsorbSmem::kTotal) != cudaSuccess)
-        return GQLA_ERR_CUDA;
-    return tc::launch_pdl(kern, dim3((unsigned)(2 * pairs)), dim3(tc::AbsorbSmem::kThreads), tc::AbsorbSmem::kTotal, st, p,
-                          tmQ, tmC) == cudaSuccess
-               ? GQLA_OK
-               : GQLA_ERR_CUDA;
+    const unsigned grid = (unsigned)(!tokens_on_m ? 2 * pairs : (balanced ? workers : B * S));  // pairs, or single CTAs
+    cudaError_t e;
+    if (tokens_on_m && pg != 0)
+        e = rows_t == 16 ? (pg == 64   ? absorb_t_launch<16, 64>(p, tmQ, tmC, grid, st)
+                            : pg == 32 ? absorb_t_launch<16, 32>(p, tmQ, tmC, grid, st)
+                                       : absorb_t_launch<16, 16>(p, tmQ, tmC, grid, st))
+                         : (pg == 64   ? absorb_t_launch<32, 64>(p, tmQ, tmC, grid, st)
+                            : pg == 32 ? absorb_t_launch<32, 32>(p, tmQ, tmC, grid, st)
+                                       : absorb_t_launch<32, 16>(p, tmQ, tmC, grid, st));
+    else if (tokens_on_m)
+        e = rows_t == 16   ? absorb_t_launch<16>(p, tmQ, tmC, grid, st)
+            : rows_t == 32 ? absorb_t_launch<32>(p, tmQ, tmC, grid, st)
+                           : absorb_t_launch<64>(p, tmQ, tmC, grid, st);
+    else
+        e = pg == 0    ? absorb_pair_launch<0>(p, tmQ, tmC, grid, st)
+            : pg == 64 ? absorb_pair_launch<64>(p, tmQ, tmC, grid, st)
+            : pg == 32 ? absorb_pair_launch<32>(p, tmQ, tmC, grid, st)
+                       : absorb_pair_launch<16>(p, tmQ, tmC, grid, st);
+    return e == cudaSuccess ? GQLA_OK : GQLA_ERR_CUDA;
 }
 
 // CTA pairs of the absorb kernel that can be resident at once on the current device (cached).
@@ -457,13 +485,14 @@ inline bool gqa_prefers_tokens(int rows_t) {
     return rows_t <= GQLA_GQA_TOKENS_MAX_ROWS;
 }
 
-template <int R>
+template <int R, int PG = 0>
 inline cudaError_t gqa_t_launch(const tc::GqaParams& p, const CUtensorMap& q, const CUtensorMap& k, const CUtensorMap& r,
                                 const CUtensorMap& v, unsigned grid, cudaStream_t st) {
-    auto kern = tc::decode_gqa_t_kernel<R>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::GqaTSmem<R>::kTotal);
+    using L = tc::GqaTSmem<R, PG>;
+    auto kern = tc::decode_gqa_t_kernel<R, PG>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
     if (e != cudaSuccess) return e;
-    return tc::launch_pdl(kern, dim3(grid), dim3(tc::GqaTSmem<R>::kThreads), tc::GqaTSmem<R>::kTotal, st, p, q, k, r, v);
+    return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, k, r, v);
 }
 
 template <int R>
@@ -486,18 +515,19 @@ inline gqla_status tc_decode_gqa(const gqla_dims& d, int32_t B, int32_t s_q, flo
         d_v % 128 != 0 || d_v < 128 || d_v > 512)
         return GQLA_ERR_UNSUPPORTED;
     const int v_blocks = d_v / 128;
-    if (rows.paged() && rows.page_size % kTileRows != 0) return GQLA_ERR_UNSUPPORTED;  // a tile must not straddle pages
     // S < 0: balanced plan with -S slots per sequence, W persistent CTAs per (group, value block)
     const int32_t workers = S < 0 ? tc_balanced_workers(d, s_q, 1) / v_blocks : 0;
     const bool balanced = S < 0 && workers > 0;
     if (S < 0) S = -S;
-    if (rows.paged() && !balanced && S != 1) return GQLA_ERR_UNSUPPORTED;  // see tc_decode_absorb
+    const int rows_t = gqa_rows_t(d, s_q, nullptr, nullptr);
+    const int pg = page_box_rows(rows, balanced || S == 1);
+    if (pg < 0 || (pg > 0 && rows_t > 32)) return GQLA_ERR_UNSUPPORTED;  // small pages: the tokens-on-M kernel only
     const int64_t units = (balanced ? (int64_t)workers * d.g : (int64_t)B * S * d.g) * v_blocks;
     if (units > 0x7fffffffLL) return GQLA_ERR_UNSUPPORTED;
     const int hpg = d.h_q / d.g;
     int hpg_box = 0, sq_box = 0;
     int R = gqa_rows(d, s_q, &hpg_box, &sq_box);
-    const bool tokens_on_m = gqa_prefers_tokens(gqa_rows_t(d, s_q, nullptr, nullptr));
+    const bool tokens_on_m = pg != 0 || gqa_prefers_tokens(rows_t);
     if (tokens_on_m) R = gqa_rows_t(d, s_q, &hpg_box, &sq_box);
     CUtensorMap tmQ, tmK, tmR, tmV;
     {
@@ -512,23 +542,33 @@ inline gqla_status tc_decode_gqa(const gqla_dims& d, int32_t B, int32_t s_q, flo
         const uint64_t str[2] = {(uint64_t)d.d_h * 2, (uint64_t)d.g * d.d_h * 2};
         const uint64_t vdims[3] = {(uint64_t)d_v, (uint64_t)d.g, (uint64_t)n_rows};
         const uint64_t vstr[2] = {(uint64_t)d_v * 2, (uint64_t)d.g * d_v * 2};
-        const uint32_t box[3] = {64, 1, 128};
+        const uint32_t box[3] = {64, 1, pg != 0 ? (uint32_t)pg : 128u};
         if (!tc::make_tmap_bf16(&tmK, k_c, 3, dims, str, box)) return GQLA_ERR_CUDA;
         if (!tc::make_tmap_bf16(&tmV, v, 3, vdims, vstr, box)) return GQLA_ERR_CUDA;
     }
     {
         const uint64_t dims[2] = {(uint64_t)d.d_r, (uint64_t)n_rows};
         const uint64_t str[1] = {(uint64_t)k_r_row_stride * 2};
-        const uint32_t box[2] = {64, 128};
+        const uint32_t box[2] = {64, pg != 0 ? (uint32_t)pg : 128u};
         if (!tc::make_tmap_bf16(&tmR, k_r, 2, dims, str, box)) return GQLA_ERR_CUDA;
     }
     tc::GqaParams p{};
+    p.n_rows = (int32_t)n_rows;
     p.v_blocks = v_blocks; p.d_v = d_v;
     p.B = B; p.S = S; p.s_q = s_q; p.h_q = d.h_q; p.g = d.g; p.hpg = hpg; p.hpg_box = hpg_box;
     p.balanced = balanced ? 1 : 0; p.W = workers;
     p.scale_log2 = scale * 1.4426950408889634f;
     p.rows = rows; p.seqlens = seqlens; p.o_part = o_part; p.lse_part = lse_part; p.status = status;
     cudaError_t e;
+    if (pg != 0) {
+        e = R == 16 ? (pg == 64   ? gqa_t_launch<16, 64>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st)
+                       : pg == 32 ? gqa_t_launch<16, 32>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st)
+                                  : gqa_t_launch<16, 16>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st))
+                    : (pg == 64   ? gqa_t_launch<32, 64>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st)
+                       : pg == 32 ? gqa_t_launch<32, 32>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st)
+                                  : gqa_t_launch<32, 16>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st));
+        return e == cudaSuccess ? GQLA_OK : GQLA_ERR_CUDA;
+    }
     if (tokens_on_m) {
         switch (R) {
             case 16: e = gqa_t_launch<16>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st); break;

@@ -813,3 +813,51 @@ def test_fused_merge_up_projection_over_slots(h_q, g, Bn, s_q, S):
     ref = O.up_proj(O.Dims(h_q, g, 128, 512, 64), oh, synth.to_f64(w_uv))
     assert_close(o.float().cpu().numpy(), ref, "combine_up_proj")
     assert_close(lse_out.cpu().numpy(), l_ref, "lse", rel=1e-5, abs_=1e-5)
+
+
+@pytest.mark.parametrize("dims", [CANON, LLAMA, dict(CANON, h_q=64), dict(h_q=28, g=4, d_h=128, r_kv=512, d_r=64), dict(LLAMA, h_q=16)])
+@pytest.mark.parametrize("page_size,S,s_q", [(16, 1, 1), (16, -9, 2), (32, -3, 1), (48, 5, 2), (64, 1, 2), (64, 3, 1), (64, -7, 1), (192, -3, 2),
+                                             (128, 3, 1), (256, 6, 2)])
+def test_small_pages_on_the_tensor_cores(dims, page_size, S, s_q):
+    """Pages that are no multiple of the 128-row tile (and pieces that start inside one): boxes of 64, 32 or 16 rows, lengths at
+    the edges of boxes, pages and tiles, against the oracle in fp32.  These calls keep probabilities to 16 bits (two bf16
+    terms): |do| <= 2 (2^-17 + dx) max|v| with dx <= 2^-13 for the fp32 scores (|x| up to about 30, 576 products),
+    a sixth of what one bf16 term would give at its worst (2^-9 max|v|)."""
+    from tests.parity_util import dims_of, round_to
+    from oracle import gqla_oracle as O
+    seqlens = np.array([1, 15, 16, 17, 31, 33, 47, 48, 49, 63, 64, 65, 127, 128, 129, 0, 191, 192, 193, 333, 1031], dtype=np.int32)
+    w = _wl("pages", len(seqlens), s_q, 260, **dims)
+    x = synth.make_inputs(w, seqlens=seqlens, q_gain=4.0)
+    od, bd = dims_of(w)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    cache_p, table = synth.to_paged(x["cache"], x["seq_start"], seqlens, page_size, seed=261)
+    f = {k: synth.to_f64(x[k]) for k in ("q_c", "q_r", "cache", "w_uk", "w_uv")}
+    qh = round_to(w, O.absorb_q(od, f["q_c"], f["q_r"], f["w_uk"])).cuda()
+    cache_d, table_d, sl = cache_p.cuda(), table.cuda(), x["seqlens"].cuda()
+
+    def check(call, D, ref, l_ref, vmax):
+        o_p = torch.full((w.batch, abs(S), s_q, w.h_q, D), float("nan"), device="cuda")
+        l_p = torch.full((w.batch, abs(S), s_q, w.h_q), float("nan"), device="cuda")
+        call(o_p, l_p)
+        o = torch.empty((w.batch, s_q, w.h_q, D), device="cuda")
+        lse = torch.empty((w.batch, s_q, w.h_q), device="cuda")
+        B.gqla_combine_splits(o_p, l_p, o, lse)
+        assert int(status.item()) == 0
+        err = np.abs(o.double().cpu().numpy() - ref).max()
+        assert err <= 2 * (2.0 ** -17 + 2.0 ** -13) * vmax, err
+        l_got = lse.double().cpu().numpy()
+        live = np.isfinite(l_ref)
+        assert np.array_equal(np.isneginf(l_got), ~live) and np.abs(l_got[live] - l_ref[live]).max() <= 2.0 ** -12
+
+    ss, sn = x["seq_start"].numpy(), seqlens
+    ref, l_ref = O.decode_absorb(od, synth.to_f64(qh), f["cache"], ss, sn, s_q, w.scale)
+    check(lambda o_p, l_p: B.gqla_decode_absorb_paged(bd, qh, cache_d, table_d, page_size, sl, w.scale, S, o_p, l_p, status),
+          w.r_kv, ref, l_ref, np.abs(f["cache"][:, :w.r_kv]).max())
+    kc, v = (torch.empty((cache_p.shape[0], w.g, w.d_h), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    B.gqla_expand_cache(bd, cache_d, x["w_uk"].cuda(), x["w_uv"].cuda(), kc, v, None)
+    q = torch.cat([x["q_c"], x["q_r"]], -1).contiguous()
+    planes = [O.unpage(synth.to_f64(t), table.numpy(), page_size, seqlens)[0] for t in (kc, v)]
+    ref, l_ref = O.decode_gqa(od, synth.to_f64(q), *planes, f["cache"][:, w.r_kv:], ss, sn, s_q, w.scale)
+    q_d = q.cuda()
+    check(lambda o_p, l_p: B.gqla_decode_gqa_paged(bd, q_d, kc, v, cache_d[:, w.r_kv:], table_d, page_size, sl, w.scale, S, o_p, l_p,
+                                                   status), w.d_h, ref, l_ref, np.abs(planes[1]).max())
