@@ -861,3 +861,25 @@ def test_small_pages_on_the_tensor_cores(dims, page_size, S, s_q):
     q_d = q.cuda()
     check(lambda o_p, l_p: B.gqla_decode_gqa_paged(bd, q_d, kc, v, cache_d[:, w.r_kv:], table_d, page_size, sl, w.scale, S, o_p, l_p,
                                                    status), w.d_h, ref, l_ref, np.abs(planes[1]).max())
+
+
+@pytest.mark.parametrize("N", [1, 127, 128, 129, 256, 257, 2049, 9473, 18944, 18945, 40000])
+@pytest.mark.parametrize("g", [2, 8, 12])
+def test_expansion_units_over_row_counts(N, g):
+    """The expansion's units (row blocks x column tiles) and the turns its CTA pairs take over them change with N and g: row
+    counts at the edges of blocks and of whole turns, k_R copied, nothing written outside.  fp32 accumulation of 512 products,
+    then one rounding to bf16: |err| <= 2^-8 |ref| + 512 * 2^-23 * max|c| max|w|."""
+    from tests.parity_util import Canaried
+    gen = torch.Generator(device="cuda").manual_seed(N + g)
+    cache = torch.randn((N, 576), generator=gen, device="cuda").bfloat16()
+    w = [(torch.randn((g, 512, 128), generator=gen, device="cuda") / 512 ** 0.5).bfloat16() for _ in range(2)]
+    bd = B.make_dims(2 * g, g, 128, 512, 64)
+    k_c, v, k_r = Canaried((N, g, 128), torch.bfloat16), Canaried((N, g, 128), torch.bfloat16), Canaried((N, 64), torch.bfloat16)
+    B.gqla_expand_cache(bd, cache, w[0], w[1], k_c.t, v.t, k_r.t)
+    assert torch.equal(k_r.t, cache[:, 512:])
+    for got, wt, what in ((k_c, w[0], "k_c"), (v, w[1], "v")):
+        ref = torch.einsum("nr,grd->ngd", cache[:, :512].double(), wt.double())
+        bound = ref.abs() * 2.0 ** -8 + 512 * 2.0 ** -23 * float(cache.abs().max()) * float(wt.abs().max())
+        assert bool(((got.t.double() - ref).abs() <= bound).all()), what
+        got.check(what)
+    k_r.check("k_r")
