@@ -34,7 +34,11 @@ struct BalancedStart {
     int32_t share, my_begin, my_end, b0, off_b0, total;
 };
 
-__host__ __device__ inline int32_t ceil_div_i32(int64_t a, int64_t b) { return (int32_t)((a + b - 1) / b); }
+__host__ __device__ inline int32_t ceil_div_i32(int64_t a, int64_t b) {
+    // tile counts nearly always fit 32 bits, and a 64-bit division is a call of some hundred cycles on the device
+    if (a + b <= 0x7fffffffLL) return (int32_t)(((uint32_t)a + (uint32_t)b - 1u) / (uint32_t)b);
+    return (int32_t)((a + b - 1) / b);
+}
 __host__ __device__ inline int32_t tiles_of(int32_t T) { return T > 0 ? (T + kTileRows - 1) / kTileRows : 0; }
 
 // share from the batch totals (see the header comment).
@@ -54,16 +58,18 @@ struct Walker {
     bool fixed_done;
     // balanced plan
     int32_t w, W, share, my_begin, my_end, b, off, total;
+    int32_t ahead;  // length of sequence b, loaded when its predecessor was walked (a piece starts with its length)
 
     __host__ __device__ void init_fixed(const int32_t* sl, int32_t B_, int32_t S_, int32_t b_, int32_t k_) {
         seqlens = sl; B = B_; S = S_; balanced = false; fb = b_; fk = k_; fixed_done = false;
-        w = W = share = my_begin = my_end = b = off = total = 0;
+        w = W = share = my_begin = my_end = b = off = total = ahead = 0;
     }
     __host__ __device__ void init_balanced(const int32_t* sl, int32_t B_, int32_t S_, int32_t w_, int32_t W_,
                                           const BalancedStart& st) {
         seqlens = sl; B = B_; S = S_; balanced = true; fb = fk = 0; fixed_done = true;
         w = w_; W = W_; share = st.share; my_begin = st.my_begin; my_end = st.my_end;
         b = st.b0; off = st.off_b0; total = st.total;
+        ahead = b < B ? seqlens[b] : 0;
     }
 
     __host__ __device__ bool next(Piece& pc) {
@@ -81,11 +87,12 @@ struct Walker {
             // past this worker's share (an empty sequence exactly on the boundary belongs to w + 1);
             // the last worker walks on to pick up empty sequences behind the last tile
             if (off >= my_end && w != W - 1) return false;
-            const int32_t T = seqlens[b];
+            const int32_t T = ahead;
             const int32_t tiles = tiles_of(T);
             const int32_t cur_b = b, cur_off = off;
             ++b;
             off += tiles;
+            if (b < B) ahead = seqlens[b];
             if (tiles == 0) {
                 const int32_t owner = cur_off >= total ? W - 1 : cur_off / share;
                 if (owner != w) continue;
@@ -148,12 +155,56 @@ __host__ __device__ inline BalancedStart balanced_start_serial(const int32_t* se
 }
 
 #ifdef __CUDACC__
+constexpr int kWarpPlan = 128;  // sequences up to which a warp evaluates the plan alone (four lengths per lane)
 // Cooperative evaluation by all `nthreads` threads of a CTA (a multiple of 32, at most 1024).  `scratch` is
 // shared memory of at least 3 * 32 + 4 int32.  Same result as balanced_start_serial.  Contains __syncthreads.
 // Thread t owns the contiguous chunk [t * chunk, (t + 1) * chunk) of the sequences; chunk sums are scanned
 // with warp shuffles and one shared-memory hop across warps.
 __device__ inline BalancedStart balanced_prepass(const int32_t* seqlens, int32_t B, int32_t S, int32_t w, int32_t W,
                                                  int32_t* scratch, int nthreads) {
+    // Batches of up to kWarpPlan sequences: every warp evaluates the plan by itself, a contiguous chunk of the sequences
+    // per lane, without the shared-memory hops and block barriers of the general form (about 3000 cycles at any size).
+    if (B <= kWarpPlan) {
+        const int lane = threadIdx.x & 31;
+        const int32_t chunk = (B + 31) >> 5;
+        const int32_t lo = lane * chunk < B ? lane * chunk : B, hi = lo + chunk < B ? lo + chunk : B;
+        int32_t tl[kWarpPlan / 32], sum = 0, mx = 0;
+#pragma unroll
+        for (int i = 0; i < kWarpPlan / 32; ++i) {
+            tl[i] = lo + i < hi ? tiles_of(seqlens[lo + i]) : 0;
+            sum += tl[i];
+            mx = max(mx, tl[i]);
+        }
+        int32_t incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t up = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += up;
+        }
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        const int32_t total = __shfl_sync(0xffffffffu, incl, 31);
+        BalancedStart st;
+        st.share = balanced_share(total, mx, S, W);
+        const int64_t mb = (int64_t)w * st.share;
+        st.my_begin = (int32_t)(mb < total ? mb : total);
+        const int64_t me = (int64_t)st.my_begin + st.share;
+        st.my_end = (int32_t)(me < total ? me : total);
+        st.total = total;
+        int32_t off = incl - sum, found = B, found_off = total;
+#pragma unroll
+        for (int i = 0; i < kWarpPlan / 32; ++i) {
+            if (lo + i < hi && found == B && off + (tl[i] > 0 ? tl[i] : 1) > st.my_begin) {
+                found = lo + i;
+                found_off = off;
+            }
+            off += tl[i];
+        }
+        const uint32_t who = __ballot_sync(0xffffffffu, found < B);  // lanes hold the sequences in order
+        const int src = who != 0 ? __ffs(who) - 1 : 0;
+        st.b0 = __shfl_sync(0xffffffffu, found, src);
+        st.off_b0 = __shfl_sync(0xffffffffu, found_off, src);
+        return st;
+    }
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarps = nthreads >> 5;
     const int32_t chunk = (B + nthreads - 1) / nthreads;
     const int32_t lo = tid * chunk < B ? tid * chunk : B, hi = lo + chunk < B ? lo + chunk : B;

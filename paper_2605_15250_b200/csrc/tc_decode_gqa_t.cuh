@@ -83,6 +83,23 @@ __device__ __forceinline__ float warp_max_redux(float x) {
     i ^= (i >> 31) & 0x7fffffff;
     return __int_as_float(i);
 }
+// Sums of N values over the warp, N = 8 or 16: halving exchanges leave the sum of value i in x[0] of the 32 / N lanes
+// [i * 32 / N, ..) -- N + log2(32 / N) - 1 shuffles instead of 5 N.
+template <int N>
+__device__ __forceinline__ void warp_sums_scatter(float* x, int lane) {
+    int o = 16;
+#pragma unroll
+    for (int n = N / 2; n > 0; n /= 2, o /= 2) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const float mine = up ? x[n + i] : x[i], theirs = up ? x[i] : x[n + i];
+            x[i] = mine + __shfl_xor_sync(0xffffffffu, theirs, o);
+        }
+    }
+#pragma unroll
+    for (; o > 0; o /= 2) x[0] += __shfl_xor_sync(0xffffffffu, x[0], o);
+}
 __device__ __forceinline__ void tmem_ld_n(uint32_t taddr, uint32_t* r, int n) {  // n in {8, 16}
     if (n == 8) tmem_ld8(taddr, r);
     else tmem_ld16(taddr, r);
@@ -164,6 +181,13 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
+        auto load_q = [&](int kb, int32_t b) {  // one k-block of the query rows of sequence b
+            asm volatile(
+                "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
+                "[%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(q_smem + kb * L::kQBlock)),
+                "l"(reinterpret_cast<uint64_t>(&tmQ)), "r"(smem_u32(q_full)), "r"(kb * 64), "r"(0), "r"(j), "r"(b * p.s_q)
+                : "memory");
+        };
         if constexpr (PG != 0) {
             constexpr int NB = 128 / PG;  // boxes per column block of a tile; one lane of the warp each
             const int run = lane % NB, blk = lane / NB;
@@ -171,16 +195,6 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
             while (ok && walk.next(pc)) {
                 if (pc.n_tiles == 0) continue;
                 const int32_t T = p.seqlens[pc.b], tok = pc.tok_begin + run * PG;
-                if (pi > 0 && !(ok = __all_sync(0xffffffffu, mbar_wait(q_empty, (pi - 1) & 1, ab, 13)))) break;
-                if (lane == 0) mbar_expect_tx(q_full, L::kQBytes);
-                __syncwarp();
-                if (lane < 3)
-                    asm volatile(
-                        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
-                        "[%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(q_smem + lane * L::kQBlock)),
-                        "l"(reinterpret_cast<uint64_t>(&tmQ)), "r"(smem_u32(q_full)), "r"(lane * 64), "r"(0), "r"(j),
-                        "r"(pc.b * p.s_q)
-                        : "memory");
                 int32_t next_row = p.rows.run_row(pc.b, tok, T, p.n_rows);
                 for (int t = 0; t < pc.n_tiles; ++t, ++gt) {
                     const int s = gt & 1;
@@ -193,6 +207,12 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                     __syncwarp();
                     if (blk < 2) tma_load_3d(st, &tmK, blk * 64, j, row, &kfull[s]);
                     else if (blk == 2) tma_load_2d(st, &tmR, 0, row, &kfull[s]);
+                    if (t == 0) {  // Q behind the piece's first K tile, as below
+                        if (pi > 0 && !(ok = __all_sync(0xffffffffu, mbar_wait(q_empty, (pi - 1) & 1, ab, 13)))) break;
+                        if (lane == 0) mbar_expect_tx(q_full, L::kQBytes);
+                        __syncwarp();
+                        if (lane < 3) load_q(lane, pc.b);
+                    }
                     if (!(ok = __all_sync(0xffffffffu, mbar_wait(&vempty[s], ph ^ 1, ab, 2)))) break;
                     if (lane == 0) mbar_expect_tx(&vfull[s], L::kVBytes);
                     __syncwarp();
@@ -209,15 +229,6 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
             bool ok = true;
             while (ok && walk.next(pc)) {
                 if (pc.n_tiles == 0) continue;
-                if (pi > 0 && !(ok = mbar_wait(q_empty, (pi - 1) & 1, ab, 13))) break;
-                mbar_expect_tx(q_full, L::kQBytes);
-                for (int kb = 0; kb < 3; ++kb)
-                    asm volatile(
-                        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
-                        "[%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(q_smem + kb * L::kQBlock)),
-                        "l"(reinterpret_cast<uint64_t>(&tmQ)), "r"(smem_u32(q_full)), "r"(kb * 64), "r"(0), "r"(j),
-                        "r"(pc.b * p.s_q)
-                        : "memory");
                 int64_t tile_row = p.rows.row(pc.b, pc.tok_begin);
                 for (int t = 0; t < pc.n_tiles; ++t, ++gt) {
                     const int s = gt & 1;
@@ -231,6 +242,13 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                     tma_load_3d(st, &tmK, 0, j, row, &kfull[s]);
                     tma_load_3d(st + 16384, &tmK, 64, j, row, &kfull[s]);
                     tma_load_2d(st + L::kKcBytes, &tmR, 0, row, &kfull[s]);
+                    // Q of the piece goes out behind its first K tile: that one only needs a free slot, Q needs every
+                    // Q K^T of the previous piece to have completed
+                    if (t == 0) {
+                        if (pi > 0 && !(ok = mbar_wait(q_empty, (pi - 1) & 1, ab, 13))) break;
+                        mbar_expect_tx(q_full, L::kQBytes);
+                        for (int kb = 0; kb < 3; ++kb) load_q(kb, pc.b);
+                    }
                     if (!(ok = mbar_wait(&vempty[s], ph ^ 1, ab, 2))) break;
                     mbar_expect_tx(&vfull[s], L::kVBytes);
                     tma_load_3d(st + L::kKcBytes + L::kKrBytes, &tmV, vb * 128, j, row, &vfull[s]);
@@ -435,39 +453,52 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
             }
 
             // -------------------------------------------------------------- row sums across the 128 tokens, then the output
+            // (the sums do not need the last P.V, so they are exchanged while it runs; red holds [row][4 quadrants] here)
+#pragma unroll
+            for (int ch = 0; ch < NCH; ++ch) {
+                float ws[CH];
+#pragma unroll
+                for (int c = 0; c < CH; ++c) ws[c] = l[ch * CH + c];
+                warp_sums_scatter<CH>(ws, lane);
+                if (lane % (32 / CH) == 0) red[4 * (r0 + ch * CH + lane / (32 / CH)) + q] = ws[0];
+            }
             const int n_last = gt + pc.n_tiles - 1;
             if (pc.n_tiles > 0 && ok)
-                ok = __all_sync(0xffffffffu, mbar_wait(&pv_done[n_last & 1], (n_last >> 1) & 1, ab, 9));
+                ok = __all_sync(0xffffffffu, mbar_wait_fast(&pv_done[n_last & 1], (n_last >> 1) & 1, ab, 9));
             tc_fence_after();
+            named_bar_sync(1, kSmT);
             const int64_t out_row0 = ((slot0 + pc.k) * p.s_q) * p.h_q + (int64_t)j * p.hpg;
+            float* o_base = p.o_part + out_row0 * p.d_v + vb * 128 + tl;
 #pragma unroll
             for (int ch = 0; ch < NCH; ++ch) {  // unrolled: l and m_ref must stay in registers
-                float* redw = red + q * R + r0 + ch * CH;
-#pragma unroll
-                for (int c = 0; c < CH; ++c) {
-                    const float ws = warp_sum(l[ch * CH + c]);
-                    if (lane == 0) redw[c] = ws;
-                }
-                named_bar_sync(1, kSmT);
                 uint32_t o[CH];
                 if (pc.n_tiles > 0 && ok) {  // warp-uniform
                     tmem_ld_n(lane_base + kColO + r0 + ch * CH, o, CH);
                     tmem_wait_ld();
                 }
+                // lane c finishes row c of the chunk (one division and one logarithm per warp side by side, not CH in a
+                // row: done by every thread for every row they took 5700 cycles of a piece), the others get its factor
+                const int rl = ch * CH + (lane & (CH - 1)), r = r0 + rl;
+                float mr = m_ref[ch * CH];
+#pragma unroll
+                for (int c = 1; c < CH; ++c) mr = (lane & (CH - 1)) == c ? m_ref[ch * CH + c] : mr;
+                const float4 part = *reinterpret_cast<const float4*>(red + 4 * r);
+                const float Lt = (part.x + part.y) + (part.z + part.w);
+                const bool live = ok && pc.n_tiles > 0 && Lt > 0.f && mr > -INFINITY;
+                const float inv = 1.f / (live ? Lt : INFINITY);
+                if (vb == 0 && q == 0 && lane < CH && (r & (p.hpg_box - 1)) < p.hpg && (r >> hshift) < p.s_q)
+                    p.lse_part[out_row0 + (r >> hshift) * p.h_q + (r & (p.hpg_box - 1))] =
+                        live ? (mr + log2f(Lt)) * 0.6931471805599453f : -INFINITY;
 #pragma unroll
                 for (int c = 0; c < CH; ++c) {
-                    const int rl = ch * CH + c, r = r0 + rl;
-                    const int pq = r / p.hpg_box, il = r % p.hpg_box;
-                    if (il >= p.hpg || pq >= p.s_q) continue;  // padding rows are computed and dropped
-                    const float Lt = (red[r] + red[R + r]) + (red[2 * R + r] + red[3 * R + r]);
-                    const bool live = ok && pc.n_tiles > 0 && Lt > 0.f && m_ref[rl] > -INFINITY;
-                    const int64_t orow = out_row0 + (int64_t)pq * p.h_q + il;
+                    const int rc = r0 + ch * CH + c, pq = rc >> hshift, il = rc & (p.hpg_box - 1);
+                    const float f = __shfl_sync(0xffffffffu, inv, c);
                     // lane tl holds value column tl of every row: 128 consecutive floats per row
-                    p.o_part[orow * p.d_v + vb * 128 + tl] = live ? __uint_as_float(o[c]) / Lt : 0.f;
-                    if (vb == 0 && tl == 0) p.lse_part[orow] = live ? (m_ref[rl] + log2f(Lt)) * 0.6931471805599453f : -INFINITY;
+                    if (il < p.hpg && pq < p.s_q)  // padding rows are computed and dropped
+                        o_base[(int64_t)(pq * p.h_q + il) * p.d_v] = f > 0.f ? __uint_as_float(o[c]) * f : 0.f;
                 }
-                named_bar_sync(1, kSmT);
             }
+            named_bar_sync(1, kSmT);  // red may be rewritten by the next piece
             // O^T has been read: the next piece's first P.V may overwrite it
             tc_fence_before();
             __syncwarp();

@@ -883,3 +883,43 @@ def test_expansion_units_over_row_counts(N, g):
         assert bool(((got.t.double() - ref).abs() <= bound).all()), what
         got.check(what)
     k_r.check("k_r")
+
+
+@pytest.mark.parametrize("Bn", [1, 31, 32, 33, 64, 97, 128, 129, 200])
+@pytest.mark.parametrize("path", ["absorb", "gqa"])
+def test_balanced_plan_of_the_kernels_is_the_host_plan(Bn, path):
+    """Up to 128 sequences every warp works the plan out by itself, beyond that the CTA does together: the slots that the
+    kernels fill (finite lse) are the host plan's, with empty sequences at both ends and in runs, and the merged lse is the
+    one-piece call's (fp32 statistics of the same scores: within 1e-5)."""
+    rng = np.random.default_rng(Bn)
+    seqlens = rng.integers(0, 700, size=Bn).astype(np.int32)
+    seqlens[rng.random(Bn) < 0.2] = 0
+    seqlens[0] = seqlens[-1] = 0 if Bn > 1 else 700
+    w = _wl("plan", Bn, 1, 500 + Bn, **CANON)
+    x = {k: t.cuda() for k, t in synth.make_inputs(w, seqlens=seqlens).items()}
+    bd = B.make_dims(w.h_q, w.g, w.d_h, w.r_kv, w.d_r)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    cache = torch.cat([x["cache"], x["cache"].new_zeros(1, 576)])  # all sequences may be empty
+    W = B.gqla_balanced_workers(bd, torch.bfloat16, 1, path)
+    merged = []
+    for S in (-4, 1):
+        D = w.r_kv if path == "absorb" else w.d_h
+        o_p = torch.empty((Bn, abs(S), 1, w.h_q, D), device="cuda")
+        l_p = torch.full((Bn, abs(S), 1, w.h_q), float("nan"), device="cuda")
+        if path == "absorb":
+            q_hat = torch.randn((Bn, 1, w.h_q, w.d_abs), generator=torch.Generator().manual_seed(1)).bfloat16().cuda()
+            B.gqla_decode_absorb(bd, q_hat, cache, x["seq_start"], x["seqlens"], w.scale, S, o_p, l_p, status)
+        else:
+            kc = cache[:, :128].repeat(1, w.g).view(-1, w.g, 128).contiguous()
+            q = torch.cat([x["q_c"], x["q_r"]], -1).contiguous()
+            B.gqla_decode_gqa(bd, q, kc, kc, cache[:, w.r_kv:], x["seq_start"], x["seqlens"], w.scale, S, o_p, l_p, status)
+        if S < 0:
+            plan, _ = B.gqla_balanced_plan(seqlens, -S, W)
+            filled = np.array([[hi > lo for lo, hi in pl] for pl in plan])
+            got = l_p.cpu().numpy()
+            assert not np.isnan(got).any() and np.array_equal(np.isfinite(got).all(axis=(2, 3)), filled)
+            assert np.array_equal(np.isneginf(got).all(axis=(2, 3)), ~filled)
+        merged.append(torch.logsumexp(l_p.double(), 1).cpu().numpy())
+    assert int(status.item()) == 0
+    live = np.isfinite(merged[1])
+    assert np.array_equal(live, np.isfinite(merged[0])) and np.abs(merged[0][live] - merged[1][live]).max(initial=0.0) <= 1e-5
