@@ -173,7 +173,7 @@ __device__ __forceinline__ float4 ld_stream4(const float* p) {  // read once: do
     return v;
 }
 template <typename TO, int V, int G>
-__global__ void __launch_bounds__(kCombineThreads, V == 4 ? 2 : 4) combine_vec_kernel(int64_t rows, int32_t rows_per_seq, int32_t S,
+__global__ void __launch_bounds__(kCombineThreads, 4) combine_vec_kernel(int64_t rows, int32_t rows_per_seq, int32_t S,
                                                                       int32_t d_out, const float* __restrict__ o_part,
                                                                       const float* __restrict__ lse_part,
                                                                       TO* __restrict__ out, float* __restrict__ lse) {
