@@ -332,8 +332,13 @@ inline gqla_status tc_combine_up_proj(const gqla_dims& d, gqla_dtype dtype, int3
         d.r_kv > tc::CombineUpSmem::kMaxChunks * tc::CombineUpSmem::kChunkK)
         return GQLA_ERR_UNSUPPORTED;
     const int64_t positions = (int64_t)B * s_q;
-    const int64_t m_tiles = (positions + 64 / hpb - 1) / (64 / hpb);
-    if (m_tiles > 0x7fffffffLL) return GQLA_ERR_UNSUPPORTED;
+    // a group's rows in as many runs as there are SMs for a group, at least four rows each (one per builder warp of a quarter)
+    const int64_t group_rows = positions * hpb;
+    int64_t runs = sm_count() / d.g > 0 ? sm_count() / d.g : 1;
+    if (runs > (group_rows + 3) / 4) runs = (group_rows + 3) / 4;
+    const int64_t run = (group_rows + runs - 1) / runs;
+    runs = (group_rows + run - 1) / run;
+    if (run > 0x7fffffffLL) return GQLA_ERR_UNSUPPORTED;
     CUtensorMap tmB;
     {
         const uint64_t dims[2] = {(uint64_t)d.d_h, (uint64_t)d.g * d.r_kv};
@@ -343,7 +348,7 @@ inline gqla_status tc_combine_up_proj(const gqla_dims& d, gqla_dtype dtype, int3
     }
     tc::CombineUpParams p{};
     p.S = S; p.s_q = s_q; p.h_q = d.h_q; p.g = d.g; p.hpg = hpg; p.hpb = hpb; p.r_kv = d.r_kv;
-    p.positions = positions; p.o_part = o_part; p.lse_part = lse_part; p.out = o; p.lse = lse; p.status = projection_status_word();
+    p.positions = positions; p.run = (int32_t)run; p.o_part = o_part; p.lse_part = lse_part; p.out = o; p.lse = lse; p.status = projection_status_word();
     auto kern = tc::combine_up_tc_kernel;
     static bool attr_set[64] = {};
     int dev = 0;
@@ -353,7 +358,7 @@ inline gqla_status tc_combine_up_proj(const gqla_dims& d, gqla_dtype dtype, int3
             return GQLA_ERR_CUDA;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
-    return tc::launch_pdl(kern, dim3((unsigned)m_tiles, (unsigned)d.g, 1), dim3(tc::CombineUpSmem::kThreads),
+    return tc::launch_pdl(kern, dim3((unsigned)runs, (unsigned)d.g, 1), dim3(tc::CombineUpSmem::kThreads),
                           tc::CombineUpSmem::kTotal, st, p, tmB) == cudaSuccess
                ? GQLA_OK
                : GQLA_ERR_CUDA;
