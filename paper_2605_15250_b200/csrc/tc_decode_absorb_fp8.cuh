@@ -141,7 +141,18 @@ decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUt
     }
 
     pdl_launch_dependents();
-    pdl_wait();  // barriers and TMEM are set up; everything below reads the caller's tensors
+    if (warp == 0 && elect_one()) {
+        tma_prefetch_desc(&tmQ);
+        tma_prefetch_desc(&tmQr);
+        tma_prefetch_desc(&tmC);
+        tma_prefetch_desc(&tmCr);
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();  // both CTAs' barriers exist before any remote arrival
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();  // set-up is done (behind the preceding kernel's tail); everything below reads the caller's tensors
     // the plan of this pair: row block rb, and either one (sequence, split) piece or worker w's share
     const int pair = blockIdx.x >> 1;
     const int rb = pair % p.row_blocks;
@@ -155,11 +166,6 @@ decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUt
         walk.init_fixed(p.seqlens, p.B, p.S, unit / p.S, unit % p.S);
     }
     const int rho0 = rb * 128 + (int)cta * 64;  // first (query, head) row of this CTA
-    tc_fence_before();
-    __syncthreads();
-    cluster_sync();  // both CTAs' barriers exist before any remote arrival
-    tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
     Piece pc;
     int pi = 0;  // non-empty pieces walked so far (phase of the per-piece barriers)
 
@@ -167,10 +173,6 @@ decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUt
         // ------------------------------------------------------------------ TMA producer of Q and the K ring
         // (both CTAs).  Every "full" barrier lives in the leader and counts the bytes of BOTH CTAs.
         if (elect_one()) {
-            tma_prefetch_desc(&tmQ);
-            tma_prefetch_desc(&tmQr);
-            tma_prefetch_desc(&tmC);
-            tma_prefetch_desc(&tmCr);
             const uint32_t q_full_l = mapa(smem_u32(q_full), 0);
             int ks = 0;
             uint32_t kph = 1;  // parity that means "slot is free"

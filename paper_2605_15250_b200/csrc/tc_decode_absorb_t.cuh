@@ -124,7 +124,15 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
     }
 
     pdl_launch_dependents();
-    pdl_wait();
+    if (warp == 0 && elect_one()) {
+        tma_prefetch_desc(&tmQ);
+        tma_prefetch_desc(&tmC);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();  // set-up is done (behind the preceding kernel's tail); everything below reads the caller's tensors
     const int unit = blockIdx.x;
     Walker walk;
     if (p.balanced) {
@@ -133,10 +141,6 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
     } else {
         walk.init_fixed(p.seqlens, p.B, p.S, unit / p.S, unit % p.S);
     }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
     Piece pc;
     int gt = 0;  // 64-token tiles walked so far: stage = gt & 1, barrier phase = (gt >> 1) & 1
     int pi = 0;  // non-empty pieces walked so far
@@ -179,8 +183,6 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                 ++pi;
             }
         } else if (elect_one()) {
-            tma_prefetch_desc(&tmQ);
-            tma_prefetch_desc(&tmC);
             bool ok = true;
             while (ok && walk.next(pc)) {
                 if (pc.n_tiles == 0) continue;

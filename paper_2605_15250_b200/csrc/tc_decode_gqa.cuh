@@ -118,7 +118,17 @@ decode_gqa_tc_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ,
     }
 
     pdl_launch_dependents();
-    pdl_wait();  // barriers and TMEM are set up; everything below reads the caller's tensors
+    if (warp == 0 && elect_one()) {
+        tma_prefetch_desc(&tmQ);
+        tma_prefetch_desc(&tmK);
+        tma_prefetch_desc(&tmR);
+        tma_prefetch_desc(&tmV);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();  // set-up is done (behind the preceding kernel's tail); everything below reads the caller's tensors
     // the plan of this CTA: group j, and either one (sequence, split) piece or worker w's share
     // consecutive CTAs: the value blocks of a group, then the groups of the same rows (they share k_R and K_C tiles
     // through L2)
@@ -132,10 +142,6 @@ decode_gqa_tc_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ,
     } else {
         walk.init_fixed(p.seqlens, p.B, p.S, unit / p.S, unit % p.S);
     }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
     Piece pc;
     int gt = 0;  // tiles walked so far: ring slot = gt & 1, barrier phase = (gt >> 1) & 1
     int pi = 0;  // non-empty pieces walked so far
@@ -143,10 +149,6 @@ decode_gqa_tc_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ,
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         if (elect_one()) {
-            tma_prefetch_desc(&tmQ);
-            tma_prefetch_desc(&tmK);
-            tma_prefetch_desc(&tmR);
-            tma_prefetch_desc(&tmV);
             bool ok = true;
             while (ok && walk.next(pc)) {
                 if (pc.n_tiles == 0) continue;

@@ -146,7 +146,18 @@ decode_gqa_fp8_tc_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorM
     }
 
     pdl_launch_dependents();
-    pdl_wait();
+    if (warp == 0 && elect_one()) {
+        tma_prefetch_desc(&tmQc);
+        tma_prefetch_desc(&tmQr);
+        tma_prefetch_desc(&tmK);
+        tma_prefetch_desc(&tmR);
+        tma_prefetch_desc(&tmV);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();  // set-up is done (behind the preceding kernel's tail); everything below reads the caller's tensors
     const int j = blockIdx.x % p.g;
     Walker walk;
     if (p.balanced) {
@@ -157,10 +168,6 @@ decode_gqa_fp8_tc_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorM
         const int unit = blockIdx.x / p.g;
         walk.init_fixed(p.seqlens, p.B, p.S, unit / p.S, unit % p.S);
     }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
     Piece pc;
     int gt = 0;  // tiles walked so far: ring slot = gt % NS, ring phase = (gt / NS) & 1; S/P buffer = gt & 1
     int pi = 0;  // non-empty pieces walked so far
@@ -168,11 +175,6 @@ decode_gqa_fp8_tc_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorM
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         if (elect_one()) {
-            tma_prefetch_desc(&tmQc);
-            tma_prefetch_desc(&tmQr);
-            tma_prefetch_desc(&tmK);
-            tma_prefetch_desc(&tmR);
-            tma_prefetch_desc(&tmV);
             bool ok = true;
             while (ok && walk.next(pc)) {
                 if (pc.n_tiles == 0) continue;

@@ -160,7 +160,17 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
     }
 
     pdl_launch_dependents();
-    pdl_wait();
+    if (warp == 0 && elect_one()) {
+        tma_prefetch_desc(&tmQ);
+        tma_prefetch_desc(&tmK);
+        tma_prefetch_desc(&tmR);
+        tma_prefetch_desc(&tmV);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();  // set-up is done (behind the preceding kernel's tail); everything below reads the caller's tensors
     const int vb = blockIdx.x % p.v_blocks;
     const int j = (blockIdx.x / p.v_blocks) % p.g;
     const int unit = blockIdx.x / (p.v_blocks * p.g);
@@ -171,10 +181,6 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
     } else {
         walk.init_fixed(p.seqlens, p.B, p.S, unit / p.S, unit % p.S);
     }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
     Piece pc;
     int gt = 0;  // tiles walked so far: ring slot = gt & 1, barrier phase = (gt >> 1) & 1
     int pi = 0;  // non-empty pieces walked so far
@@ -222,10 +228,6 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                 ++pi;
             }
         } else if (elect_one()) {
-            tma_prefetch_desc(&tmQ);
-            tma_prefetch_desc(&tmK);
-            tma_prefetch_desc(&tmR);
-            tma_prefetch_desc(&tmV);
             bool ok = true;
             while (ok && walk.next(pc)) {
                 if (pc.n_tiles == 0) continue;
