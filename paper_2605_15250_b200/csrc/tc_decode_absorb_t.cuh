@@ -454,37 +454,42 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
             }
 
             // -------------------------------------------------------------- row sums across the tokens, then the output
-            const int n_last = gt + nt - 1;
-            if (nt > 0 && ok) ok = __all_sync(0xffffffffu, mbar_wait(&pv_done[n_last & 1], (n_last >> 1) & 1, ab, 9));
-            tc_fence_after();
+            // (the sums do not need the last P.V, so they are exchanged while it runs; red holds [row][4 quadrants] here)
 #pragma unroll
             for (int j = 0; j < NJ; ++j) {  // the row's sum over the warp's tokens: lanes with equal t % 4
                 float ws = l[j];
                 ws += __shfl_xor_sync(0xffffffffu, ws, 4);
                 ws += __shfl_xor_sync(0xffffffffu, ws, 8);
                 ws += __shfl_xor_sync(0xffffffffu, ws, 16);
-                if (lane < 4) red[q * R + r0 + rj(j)] = ws;
+                if (lane < 4) red[4 * (r0 + rj(j)) + q] = ws;
             }
+            const int n_last = gt + nt - 1;
+            if (nt > 0 && ok) ok = __all_sync(0xffffffffu, mbar_wait_fast(&pv_done[n_last & 1], (n_last >> 1) & 1, ab, 9));
+            tc_fence_after();
             named_bar_sync(1, kSmT);
             const int64_t out_row0 = (p.o_final != nullptr ? (int64_t)pc.b : slot0 + pc.k) * p.rows_total;
+            auto row_sum = [&](int r) -> float {
+                const float4 part = *reinterpret_cast<const float4*>(red + 4 * r);
+                return (part.x + part.y) + (part.z + part.w);
+            };
             if (q == 0 && lane < 4 && p.lse_part != nullptr) {
 #pragma unroll
                 for (int j = 0; j < NJ; ++j) {
                     const int r = r0 + rj(j);
-                    const float Lt = (red[r] + red[R + r]) + (red[2 * R + r] + red[3 * R + r]);
+                    const float Lt = row_sum(r);
                     const bool live = ok && nt > 0 && Lt > 0.f && m_ref[j] > -INFINITY;
                     if (r < p.rows_total) p.lse_part[out_row0 + r] = live ? (m_ref[j] + log2f(Lt)) * 0.6931471805599453f : -INFINITY;
                 }
             }
 #pragma unroll
             for (int cc = 0; cc < RW; cc += 8) {  // eight rows at a time (a lane is a latent column of all of them)
-                float inv[8];
+                // lane c divides for row c, the others get its factor (every thread dividing for every row, one after the
+                // other, was most of the 5500 cycles a piece's output took)
+                const float Lc = row_sum(r0 + cc + (lane & 7));
+                const float inv = 1.f / (ok && nt > 0 && Lc > 0.f ? Lc : INFINITY);
+                float f[8];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const int r = r0 + cc + c;
-                    const float Lt = (red[r] + red[R + r]) + (red[2 * R + r] + red[3 * R + r]);
-                    inv[c] = (ok && nt > 0 && Lt > 0.f) ? 1.f / Lt : 0.f;
-                }
+                for (int c = 0; c < 8; ++c) f[c] = __shfl_sync(0xffffffffu, inv, c);
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
                     uint32_t o[8];
@@ -496,7 +501,7 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                     for (int c = 0; c < 8; ++c) {
                         const int r = r0 + cc + c;
                         if (r >= p.rows_total) continue;  // padding rows are computed and dropped
-                        const float val = inv[c] > 0.f ? __uint_as_float(o[c]) * inv[c] : 0.f;
+                        const float val = f[c] > 0.f ? __uint_as_float(o[c]) * f[c] : 0.f;
                         // lane tl holds latent column 128 m + tl of every row: 128 consecutive values per row and block
                         if (p.o_final != nullptr) p.o_final[(out_row0 + r) * 512 + m * 128 + tl] = __float2bfloat16(val);
                         else p.o_part[(out_row0 + r) * 512 + m * 128 + tl] = val;
