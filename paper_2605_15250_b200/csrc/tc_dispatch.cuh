@@ -173,12 +173,12 @@ inline gqla_status tc_expand_cache(const gqla_dims& d, gqla_dtype dtype, int64_t
                 return GQLA_ERR_CUDA;
             if (dev >= 0 && dev < 64) attr_set[dev] = true;
         }
-        // output planes as [N, g * 128] matrices; stores of 64 columns x 128 rows, clipped at row N
+        // output planes as [N, g * 128] matrices; stores of 64 columns x 32 rows, clipped at row N
         CUtensorMap tmOK, tmOV;
         {
             const uint64_t odims[2] = {(uint64_t)d.g * 128, (uint64_t)N};
             const uint64_t ostr[1] = {(uint64_t)d.g * 128 * 2};
-            const uint32_t obox[2] = {64, 128};
+            const uint32_t obox[2] = {64, 32};
             if (!tc::make_tmap_bf16(&tmOK, k_c, 2, odims, ostr, obox)) return GQLA_ERR_CUDA;
             if (!tc::make_tmap_bf16(&tmOV, v, 2, odims, ostr, obox)) return GQLA_ERR_CUDA;
         }

@@ -8,9 +8,11 @@
 // rows are loaded into it right away: with two 256-column accumulators in TMEM the epilogue warps store tile t while
 // the MMAs of tile t + 1 run, across units too, and the tensor core only waits at the very first unit of a pair.
 // (One pair per 256 rows and launch slot, as this kernel was before, paid set-up, the load of the rows and the last
-// tile's store once per unit: 443 us against 402 us on 224 672 rows, 61 against 48 us on 20 000.)  The output leaves through a
-// swizzled shared-memory staging box and TMA stores (64 columns x 128 rows at a time): one thread per row
-// writing its row straight to global memory costs more store instructions than the MMAs give it time for.
+// tile's store once per unit: 443 us against 402 us on 224 672 rows, 61 against 48 us on 20 000.)  The output leaves through
+// swizzled shared-memory staging boxes and TMA stores, 64 columns x 32 rows at a time: one thread per row
+// writing its row straight to global memory costs more store instructions than the MMAs give it time for.  Every
+// epilogue warp has a box of its own: with one box of 128 rows the four warps met at two barriers per 64 columns and
+// waited together for its store (224 672 rows: 430 against 428 us, 20 000 rows 49.1 against 48.3).
 // Warp roles per CTA: warp 0 TMA producer, warp 1 TMEM owner (+ MMA issuer in the leader), warps 2-5
 // epilogue (TMEM lane = row).
 #pragma once
@@ -40,8 +42,8 @@ struct ExpandSmem {
     // ring of B stages: measured on the C2 cache, 4 stages 0.498 ms, 5 stages 0.464 ms (the weights come out of
     // L2 and every k-block is only 512 cycles of tensor work)
     static constexpr int kStages = 5;
-    static constexpr int kOutBytes = 16384;              // output staging box: 128 rows x 64 bf16, 128-byte swizzle
-    static constexpr int kTileBytes = kABytes + kStages * kBStage + kOutBytes;  // one staging box (a second one measured slower: 0.524 vs 0.498 ms)
+    static constexpr int kOutBytes = 16384;              // output staging: a box of 32 rows x 64 bf16 per epilogue warp, 128-byte swizzle
+    static constexpr int kTileBytes = kABytes + kStages * kBStage + kOutBytes;
     // a_full[kKBlocks], a_empty[kKBlocks], b_full[], b_empty[], acc_full[2], acc_empty[2]
     static constexpr int kNumBars = 2 * kKBlocks + 2 * kStages + 4;
     static constexpr int kThreads = 192;
@@ -169,10 +171,11 @@ expand_tc_kernel(const ExpandParams p, const __grid_constant__ CUtensorMap tmA, 
         // ------------------------------------------------------------------ epilogue: TMEM lane = row
         const int q = warp & 3;
         const uint32_t acc_empty_l[2] = {mapa(smem_u32(&acc_empty[0]), 0), mapa(smem_u32(&acc_empty[1]), 0)};
+        uint8_t* box = out_smem + q * 4096;  // this warp's 32 rows x 64 columns
         bool ok = true;
         int at = 0;
         for (int u = pair; u < n_units && ok; u += n_pairs) {
-            const int64_t row_base = row_of(u), n = row_base + q * 32 + lane;
+            const int64_t warp_row = row_of(u) + q * 32, n = warp_row + lane;
             const int t0 = (u % col_units) * p.unit_tiles;
             if (t0 == 0 && n < p.n_rows && p.k_r != nullptr) {  // k^R is carried over unchanged
                 const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.cache) +
@@ -187,17 +190,15 @@ expand_tc_kernel(const ExpandParams p, const __grid_constant__ CUtensorMap tmA, 
                 tc_fence_after();
                 const CUtensorMap* tmO = 2 * t >= p.g ? &tmOV : &tmOK;
                 const int col_base = ((2 * t) % p.g) * 128;  // first column of the tile in its plane's [N, g * 128] rows
-                const int r = q * 32 + lane;                 // row of this thread within the CTA's 128
 #pragma unroll 1
                 for (int cb = 0; cb < 4; ++cb) {
                     uint32_t v[64];
                     tmem_ld32(tmem_addr(tmem_base, q * 32, buf * 256 + cb * 64), v);
                     tmem_ld32(tmem_addr(tmem_base, q * 32, buf * 256 + cb * 64 + 32), v + 32);
                     tmem_wait_ld();
-                    // the staging box is rewritten: the store that last read it must have finished reading
-                    uint8_t* box = out_smem;
-                    if (threadIdx.x == 64) bulk_wait_read();
-                    named_bar_sync(1, 128);
+                    // the warp's staging box is rewritten: its last store must have finished reading
+                    if (lane == 0) bulk_wait_read();
+                    __syncwarp();
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {  // 8 chunks of 8 bf16; chunk index XORed with (row & 7)
                         uint4 o;
@@ -205,12 +206,12 @@ expand_tc_kernel(const ExpandParams p, const __grid_constant__ CUtensorMap tmA, 
                         o.y = pack_bf16(__uint_as_float(v[8 * c + 2]), __uint_as_float(v[8 * c + 3]));
                         o.z = pack_bf16(__uint_as_float(v[8 * c + 4]), __uint_as_float(v[8 * c + 5]));
                         o.w = pack_bf16(__uint_as_float(v[8 * c + 6]), __uint_as_float(v[8 * c + 7]));
-                        *reinterpret_cast<uint4*>(box + r * 128 + ((c ^ (r & 7)) << 4)) = o;
+                        *reinterpret_cast<uint4*>(box + lane * 128 + ((c ^ (lane & 7)) << 4)) = o;
                     }
                     fence_proxy_async_smem();
-                    named_bar_sync(1, 128);
-                    if (threadIdx.x == 64 && row_base < p.n_rows) {  // a CTA wholly behind the last row stores nothing
-                        tma_store_2d(tmO, box, col_base + cb * 64, (int32_t)row_base);
+                    __syncwarp();
+                    if (lane == 0 && warp_row < p.n_rows) {  // a warp wholly behind the last row stores nothing
+                        tma_store_2d(tmO, box, col_base + cb * 64, (int32_t)warp_row);
                         bulk_commit();
                     }
                 }
@@ -219,7 +220,7 @@ expand_tc_kernel(const ExpandParams p, const __grid_constant__ CUtensorMap tmA, 
                 if (lane == 0) mbar_arrive_cluster(acc_empty_l[buf]);
             }
         }
-        if (threadIdx.x == 64) bulk_wait_read();  // the last store still reads the staging box
+        if (lane == 0) bulk_wait_read();  // the last store still reads the staging box
     }
     tc_fence_before();
     __syncthreads();
