@@ -64,6 +64,8 @@ struct AbsorbFp8Smem {
     static constexpr int kThreads = 96 + 32 * kSoftmaxWarps;
     static constexpr int kOutPitch = 256 * 4 + 16;
     static_assert(64 * kOutPitch <= kPBytes + kNV * kVGroup, "output staging must fit in P + V ring");
+    static constexpr int kWarpPitch = 64 * 4 + 16;  // fp32 partials: a softmax warp's 32 rows x 64 columns
+    static_assert(8 * 32 * kWarpPitch <= kPBytes + kNV * kVGroup, "output staging must fit in P + V ring");
     static_assert(kKGroup % 1024 == 0 && kOffP % 1024 == 0, "swizzled tiles need 1 KB alignment");
     static constexpr int kTotal = kTileBytes + kNumBars * 8 + 16 + 2 * 4 * 64 * 4;
     static_assert(2 * 4 * 64 >= kThreads + 4, "plan scratch must fit in sm_max");
@@ -87,7 +89,9 @@ __device__ __forceinline__ void umma_f8_ss2_lo(uint32_t d_tmem, uint32_t a_lo, u
         : "memory");
 }
 
-template <int DUMMY>
+// FINAL: the whole-sequence call (o_final set); a form of its own, because the registers of the partials' output cost the
+// softmax loop 1 % of it.
+template <bool FINAL>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(AbsorbFp8Smem::kThreads, 1)
 decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUtensorMap tmQ,
                             const __grid_constant__ CUtensorMap tmQr, const __grid_constant__ CUtensorMap tmC,
@@ -484,10 +488,10 @@ decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUt
             const bool live = ok && pc.n_tiles > 0 && Lt > 0.f && m_used > -INFINITY;
             const float inv = live ? p.v_scale / Lt : 0.f;
             // The CTA's 64 output rows leave through shared memory (P and the V ring are idle now: the last
-            // P.V has completed) as 1 KB bulk stores, the 256 columns of MMA m = 0 first, then those of m = 1.
-            // The padded pitch keeps the 16-byte stores of a quarter warp on distinct banks.
+            // P.V has completed) as bulk stores.  The padded pitches keep the 16-byte stores of a quarter warp on
+            // distinct banks.
             uint8_t* stage = tiles + L::kOffP;
-            if (p.o_final != nullptr) {
+            if constexpr (FINAL) {
                 // whole-sequence call: the final bf16 rows (1 KB each) fit the staging at once -- one pass
                 uint4* dst = reinterpret_cast<uint4*>(stage + r * L::kOutPitch + (128 * hf + 64 * ch) * 2);
 #pragma unroll 1
@@ -522,10 +526,12 @@ decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUt
                     }
                 }
             } else {
-                float* gbase = p.o_part + ((slot0 + pc.k) * p.rows_total + rho0) * 512;
+                // fp32 partials: every warp stages and ships 32 rows x 64 columns of MMA m's block by itself (256-byte bulk
+                // stores), as in the bf16 kernel (14 sequences of 19-1229 rows: 38.9 -> 36.9 us a step)
+                uint8_t* own = stage + ((int)threadIdx.x - 64) * L::kWarpPitch;
 #pragma unroll 1
                 for (int m = 0; m < 2; ++m) {
-                    float4* dst = reinterpret_cast<float4*>(stage + r * L::kOutPitch + (128 * hf + 64 * ch) * 4);
+                    if (m == 1) bulk_wait_read();  // this lane's row of m = 0 has left the staging
 #pragma unroll 1
                     for (int c = 0; c < 64; c += 32) {
                         uint32_t o[32];
@@ -535,36 +541,23 @@ decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUt
                         }
 #pragma unroll
                         for (int i = 0; i < 8; ++i)
-                            dst[c / 4 + i] =
+                            reinterpret_cast<float4*>(own)[c / 4 + i] =
                                 live ? make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv,
                                                    __uint_as_float(o[4 * i + 2]) * inv, __uint_as_float(o[4 * i + 3]) * inv)
                                      : make_float4(0.f, 0.f, 0.f, 0.f);
                     }
-                    fence_proxy_async_smem();  // staged rows -> visible to the bulk-copy engine
-                    if (m == 1) {              // O has been read: the next piece's first P.V may overwrite it
+                    if (m == 1) {  // O has been read: the next piece's first P.V may overwrite it
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive_cluster(o_free_l);
                     }
+                    fence_proxy_async_smem();  // staged row -> visible to the bulk-copy engine
+                    if (row_valid && ok)
+                        bulk_store(p.o_part + ((slot0 + pc.k) * p.rows_total + rho) * 512 + 256 * m + 128 * hf + 64 * ch, own, 256);
+                    bulk_commit();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(epi);
-                    if (!__all_sync(0xffffffffu, mbar_wait(epi, ec & 1, ab, 12))) ok = false;
-                    ++ec;
-                    if (ok && lane < 8) {
-                        const int rr = (warp - 2) * 8 + lane;  // each softmax warp ships eight rows
-                        if (rho0 + rr < p.rows_total) {
-                            bulk_store(gbase + (int64_t)rr * 512 + 256 * m, stage + rr * L::kOutPitch, 256 * 4);
-                            bulk_commit();
-                            bulk_wait_read();
-                        }
-                    }
-                    if (m == 0) {  // the staging is rewritten next: every warp's stores must have read it
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(epi);
-                        if (!__all_sync(0xffffffffu, mbar_wait(epi, ec & 1, ab, 12))) ok = false;
-                        ++ec;
-                    }
                 }
+                bulk_wait_read();
             }
             // staging (and with it P and the V ring) is free again once every warp's stores have read it
             __syncwarp();

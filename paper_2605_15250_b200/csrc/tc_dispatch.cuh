@@ -646,7 +646,7 @@ inline gqla_status tc_decode_absorb_fp8(const gqla_dims& d, int32_t B, int32_t s
     p.rows = rows; p.seqlens = seqlens; p.o_part = o_part; p.lse_part = lse_part; p.status = status;
     p.o_final = (__nv_bfloat16*)o_final;
     if (o_final != nullptr && (balanced || S != 1)) return GQLA_ERR_UNSUPPORTED;
-    auto kern = tc::decode_absorb_fp8_tc_kernel<0>;
+    auto kern = o_final != nullptr ? tc::decode_absorb_fp8_tc_kernel<true> : tc::decode_absorb_fp8_tc_kernel<false>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::AbsorbFp8Smem::kTotal) != cudaSuccess)
         return GQLA_ERR_CUDA;
     return tc::launch_pdl(kern, dim3((unsigned)(2 * pairs)), dim3(tc::AbsorbFp8Smem::kThreads), tc::AbsorbFp8Smem::kTotal, st,
