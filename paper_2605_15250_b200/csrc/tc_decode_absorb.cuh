@@ -97,7 +97,9 @@ using AbsorbSmem = AbsorbSmemT<0>;
 constexpr uint32_t kAColO = 0;    // O: MMA m (latent columns [256m, 256m+256)) at TMEM columns [128m, 128m+128)
 constexpr uint32_t kAColS = 256;  // two 64-column score buffers
 
-template <int PG>
+// FINAL: the whole-sequence call (o_final set); a form of its own, so that neither output's registers weigh on the softmax
+// loop of the other.
+template <int PG, bool FINAL = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(AbsorbSmemT<PG>::kThreads, 1)
 decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap tmQ,
                         const __grid_constant__ CUtensorMap tmC) {
@@ -540,7 +542,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
             // P.V has completed) as bulk stores.  The padded pitches keep the 16-byte stores of a quarter warp on
             // distinct banks.
             uint8_t* stage = tiles + L::kOffP;
-            if (p.o_final != nullptr) {
+            if constexpr (FINAL) {
                 // whole-sequence call: the final bf16 rows (1 KB each) fit the staging at once -- one pass
                 uint4* dst = reinterpret_cast<uint4*>(stage + r * L::kOutPitch + (128 * hf + 64 * ch) * 2);
 #pragma unroll 1

@@ -374,11 +374,11 @@ inline cudaError_t absorb_t_launch(const tc::AbsorbParams& p, const CUtensorMap&
     return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, c);
 }
 
-template <int PG>
+template <int PG, bool FINAL = false>
 inline cudaError_t absorb_pair_launch(const tc::AbsorbParams& p, const CUtensorMap& q, const CUtensorMap& c, unsigned grid,
                                       cudaStream_t st) {
     using L = tc::AbsorbSmemT<PG>;
-    auto kern = tc::decode_absorb_tc_kernel<PG>;
+    auto kern = tc::decode_absorb_tc_kernel<PG, FINAL>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
     if (e != cudaSuccess) return e;
     return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, c);
@@ -440,7 +440,8 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
             : rows_t == 32 ? absorb_t_launch<32>(p, tmQ, tmC, grid, st)
                            : absorb_t_launch<64>(p, tmQ, tmC, grid, st);
     else
-        e = pg == 0    ? absorb_pair_launch<0>(p, tmQ, tmC, grid, st)
+        e = pg == 0    ? (o_final != nullptr ? absorb_pair_launch<0, true>(p, tmQ, tmC, grid, st)
+                                             : absorb_pair_launch<0>(p, tmQ, tmC, grid, st))
             : pg == 64 ? absorb_pair_launch<64>(p, tmQ, tmC, grid, st)
             : pg == 32 ? absorb_pair_launch<32>(p, tmQ, tmC, grid, st)
                        : absorb_pair_launch<16>(p, tmQ, tmC, grid, st);
