@@ -198,10 +198,11 @@ gqla_status gqla_decode_gqa_noalloc(const gqla_dims* dims, gqla_dtype dtype, int
  * with block_table an int32 [B, max_pages] device array whose entries below ceil(seqlens[b] / page_size)
  * must name pages inside the cache (page * page_size + page_size <= cache_rows / n_rows); later entries
  * are never read.  Everything else is as for gqla_decode_absorb / gqla_decode_gqa, and the outputs are
- * the same as for the packed cache holding the same rows (rows of a sequence's last page behind its end
- * must hold finite values, as rows outside a sequence do there).  With a page size that is a multiple of
+ * the same as for the packed cache holding the same rows.  With a page size that is a multiple of
  * 128 rows and num_splits == 1 or the balanced plan (num_splits <= -2) the tensor-core kernels run as over
- * a packed cache.  Other page sizes that are a multiple of 16, and num_splits >= 2, run on forms of them
+ * a packed cache (so rows of a sequence's last page behind its end must hold finite values, as rows outside a
+ * sequence do there; the other forms accept anything in them).  Other page sizes that are a multiple of 16,
+ * and num_splits >= 2, run on forms of them
  * that fetch by pages and keep the probabilities to 16 bits (on the absorb path with 33 to 64 query rows
  * the balanced plan is then cut for half the SMs per 128 query rows, as in gqla_decode_absorb_fp8; on the
  * GQA path up to 32 padded query rows per group); everything else runs on the generic kernels. */

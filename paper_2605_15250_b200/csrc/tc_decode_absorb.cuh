@@ -31,7 +31,8 @@
 // Small pages (template parameter PG = rows of a box: 64, 32 or 16; 0 = the form above).  A paged cache whose pages are
 // no multiple of the 128-row tile is fetched in boxes of PG rows that no page boundary cuts (PG divides the page size
 // and the tile's halves): the boxes of a group go out together, one lane of the producer warp each, after every lane has
-// looked its page up; boxes behind the sequence's end start behind the cache's last row and are filled with zeros.  Such
+// looked its page up; boxes behind the sequence's end start behind the cache's last row and are filled with zeros, and of the
+// box that the end cuts V gets zeros behind it (load_cut_run): rows outside a sequence may hold anything.  Such
 // calls keep 32-bit probabilities: P is split into two bf16 terms (hi + lo, 16 bits) and P V is issued for both, the
 // second P buffer taking the place of one K group.  These calls ran one warp per query row on the SIMT kernel before,
 // which read every cache row h_q times from L2: 13.7 ms for 32 sequences of 300-8000 rows in pages of 64 rows.
@@ -102,7 +103,7 @@ constexpr uint32_t kAColS = 256;  // two 64-column score buffers
 template <int PG, bool FINAL = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(AbsorbSmemT<PG>::kThreads, 1)
 decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap tmQ,
-                        const __grid_constant__ CUtensorMap tmC) {
+                        const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CutMaps<PG> cut_maps) {
     using L = AbsorbSmemT<PG>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* tiles = smem_raw;
@@ -266,13 +267,23 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 int32_t next_row = p.rows.run_row(pc.b, tok, T, p.n_rows);
                 for (int vg = 0; vg < 2 * pc.n_tiles; ++vg) {  // (tile, token half)
                     const int32_t row = next_row;
+                    const int32_t left = T - (pc.tok_begin + vg * 64);
+                    const int cut = cut_run<PG>(left, 64);
                     if (vg + 1 < 2 * pc.n_tiles) next_row = p.rows.run_row(pc.b, tok + (vg + 1) * 64, T, p.n_rows);
                     if (!(ok = __all_sync(0xffffffffu, mbar_wait(&vempty[vs], vph, ab, 2)))) break;
                     if (cta == 0 && lane == 0) mbar_expect_tx(&vfull[vs], 2 * L::kVGroup);
                     __syncwarp();
-                    if (mi < 4)
-                        tma_load_2d_pair(tiles + L::kOffV + vs * L::kVGroup + mi * L::kBox + run * PG * 128, &tmC,
-                                         256 * (mi >> 1) + 128 * (int)cta + 64 * (mi & 1), row, mapa(smem_u32(&vfull[vs]), 0));
+                    uint8_t* dst = tiles + L::kOffV + vs * L::kVGroup;
+                    const uint32_t bar = mapa(smem_u32(&vfull[vs]), 0);
+                    if (mi < 4 && run != cut)
+                        tma_load_2d_pair(dst + mi * L::kBox + run * PG * 128, &tmC,
+                                         256 * (mi >> 1) + 128 * (int)cta + 64 * (mi & 1), row, bar);
+                    if (cut >= 0)
+                        load_cut_run<PG, 4>(cut_maps, lane, left % PG, __shfl_sync(0xffffffffu, row, cut), p.n_rows,
+                                            [&](const CUtensorMap* m, int b, int r, int32_t y) {
+                                                tma_load_2d_pair(dst + b * L::kBox + (cut * PG + r) * 128, m,
+                                                                 256 * (b >> 1) + 128 * (int)cta + 64 * (b & 1), y, bar);
+                                            });
                     if (++vs == L::kNV) { vs = 0; vph ^= 1; }
                 }
                 ++pi;

@@ -78,7 +78,8 @@ constexpr uint32_t kPollSpins = 1u << 25;  // polls of the MMA issuer without pr
 
 template <int R, int PG = 0>
 __global__ void __launch_bounds__(AbsorbTSmem<R, PG>::kThreads, 1)
-decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmC) {
+decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmC,
+                       const __grid_constant__ CutMaps<PG> cut_maps) {
     using L = AbsorbTSmem<R, PG>;
     constexpr int RW = L::kRowsPerWarp;
     constexpr int NJ = RW / 4;  // query rows per softmax thread
@@ -163,15 +164,23 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                 int32_t row = p.rows.run_row(pc.b, tok, T, p.n_rows), row1 = p.rows.run_row(pc.b, tok + TK, T, p.n_rows);
                 for (int t = 0; t < nt; ++t, ++gt) {
                     const int s = gt & 1;
+                    const int32_t left = T - (pc.tok_begin + t * TK);
+                    const int cut = cut_run<PG>(left, TK);
                     const int32_t row2 = p.rows.run_row(pc.b, tok + (t + 2) * TK, T, p.n_rows);
                     if (!(ok = __all_sync(0xffffffffu, mbar_wait(&empty[s], ((gt >> 1) & 1) ^ 1, ab, 1)))) break;
 #pragma unroll
                     for (int g = 0; g < 3; ++g) {
                         if (lane == 0) mbar_expect_tx(&full[s * 3 + g], L::kGroup);
                         __syncwarp();
-                        if (blk < 3)
-                            tma_load_2d(stage0 + s * L::kStageBytes + (3 * g + blk) * L::kBox + run * PG * 128, &tmC,
-                                        (3 * g + blk) * 64, row, &full[s * 3 + g]);
+                        uint8_t* dst = stage0 + s * L::kStageBytes + 3 * g * L::kBox;
+                        if (blk < 3 && run != cut)
+                            tma_load_2d(dst + blk * L::kBox + run * PG * 128, &tmC, (3 * g + blk) * 64, row, &full[s * 3 + g]);
+                        if (cut >= 0)
+                            load_cut_run<PG, 3>(cut_maps, lane, left % PG, __shfl_sync(0xffffffffu, row, cut), p.n_rows,
+                                                [&](const CUtensorMap* m, int b, int r, int32_t y) {
+                                                    tma_load_2d(dst + b * L::kBox + (cut * PG + r) * 128, m, (3 * g + b) * 64, y,
+                                                                &full[s * 3 + g]);
+                                                });
                     }
                     if (blk < 3 && t + 2 < nt && row2 != p.n_rows) {
 #pragma unroll

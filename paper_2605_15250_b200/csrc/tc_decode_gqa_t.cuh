@@ -112,7 +112,8 @@ __device__ __forceinline__ void tmem_st_n(uint32_t taddr, const uint32_t* r, int
 template <int R, int PG = 0>
 __global__ void __launch_bounds__(GqaTSmem<R, PG>::kThreads, 1)
 decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                    const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmV) {
+                    const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmV,
+                    const __grid_constant__ CutMaps<PG> cut_maps) {
     using L = GqaTSmem<R, PG>;
     constexpr int RW = L::kRowsPerThread;    // query rows per softmax thread (the others belong to its partner warps)
     constexpr int CH = RW;                   // rows handled per pass (TMEM columns per load)
@@ -207,6 +208,8 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                     const uint32_t ph = (gt >> 1) & 1;
                     uint8_t* st = stage0 + s * L::kStageBytes + blk * 16384 + run * PG * 128;
                     const int32_t row = next_row;
+                    const int32_t left = T - (pc.tok_begin + t * 128);
+                    const int cut = cut_run<PG>(left, 128);
                     if (t + 1 < pc.n_tiles) next_row = p.rows.run_row(pc.b, tok + (t + 1) * 128, T, p.n_rows);
                     if (!(ok = __all_sync(0xffffffffu, mbar_wait(&kempty[s], ph ^ 1, ab, 1)))) break;
                     if (lane == 0) mbar_expect_tx(&kfull[s], L::kKcBytes + L::kKrBytes);
@@ -222,8 +225,15 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                     if (!(ok = __all_sync(0xffffffffu, mbar_wait(&vempty[s], ph ^ 1, ab, 2)))) break;
                     if (lane == 0) mbar_expect_tx(&vfull[s], L::kVBytes);
                     __syncwarp();
-                    if (blk < 2)
+                    if (blk < 2 && run != cut)
                         tma_load_3d(st + L::kKcBytes + L::kKrBytes, &tmV, vb * 128 + blk * 64, j, row, &vfull[s]);
+                    if (cut >= 0) {
+                        uint8_t* dst = stage0 + s * L::kStageBytes + L::kKcBytes + L::kKrBytes + cut * PG * 128;
+                        load_cut_run<PG, 2>(cut_maps, lane, left % PG, __shfl_sync(0xffffffffu, row, cut), p.n_rows,
+                                            [&](const CUtensorMap* m, int b, int r, int32_t y) {
+                                                tma_load_3d(dst + b * 16384 + r * 128, m, vb * 128 + b * 64, j, y, &vfull[s]);
+                                            });
+                    }
                 }
                 ++pi;
             }

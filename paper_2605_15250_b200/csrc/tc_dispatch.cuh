@@ -4,6 +4,8 @@
 #pragma once
 #include <stdlib.h>
 
+#include <type_traits>
+
 #include "../../include/gqla.h"
 #include "common.cuh"
 #include "tc_decode_absorb.cuh"
@@ -364,24 +366,40 @@ inline gqla_status tc_combine_up_proj(const gqla_dims& d, gqla_dtype dtype, int3
                : GQLA_ERR_CUDA;
 }
 
+// The box heights of a small-page form as a compile-time constant: f(std::integral_constant<int, PG>).
+template <typename F>
+inline cudaError_t with_page_box(int pg, F f) {
+    if (pg == 64) return f(std::integral_constant<int, 64>());
+    if (pg == 32) return f(std::integral_constant<int, 32>());
+    return f(std::integral_constant<int, 16>());
+}
+// Maps of the boxes that a sequence's end cuts (tc_common.cuh), of a plane whose tensor map has these dims and strides.
+template <int PG>
+inline bool make_cut_maps(tc::CutMaps<PG>* out, const void* base, int rank, const uint64_t* dims, const uint64_t* strides) {
+    uint32_t box[3] = {64, 1, 1};
+    if (!tc::make_tmap_bf16(&out->row1, base, rank, dims, strides, box)) return false;
+    box[rank - 1] = 8;
+    return tc::make_tmap_bf16(&out->rows8, base, rank, dims, strides, box);
+}
+
 template <int R, int PG = 0>
 inline cudaError_t absorb_t_launch(const tc::AbsorbParams& p, const CUtensorMap& q, const CUtensorMap& c, unsigned grid,
-                                   cudaStream_t st) {
+                                   cudaStream_t st, const tc::CutMaps<PG>& cut = {}) {
     using L = tc::AbsorbTSmem<R, PG>;
     auto kern = tc::decode_absorb_t_kernel<R, PG>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
     if (e != cudaSuccess) return e;
-    return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, c);
+    return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, c, cut);
 }
 
 template <int PG, bool FINAL = false>
 inline cudaError_t absorb_pair_launch(const tc::AbsorbParams& p, const CUtensorMap& q, const CUtensorMap& c, unsigned grid,
-                                      cudaStream_t st) {
+                                      cudaStream_t st, const tc::CutMaps<PG>& cut = {}) {
     using L = tc::AbsorbSmemT<PG>;
     auto kern = tc::decode_absorb_tc_kernel<PG, FINAL>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
     if (e != cudaSuccess) return e;
-    return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, c);
+    return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, c, cut);
 }
 
 inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, float scale, int32_t S,
@@ -413,11 +431,11 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
         const uint32_t box[2] = {64, tokens_on_m ? (uint32_t)rows_t : 64u};  // beyond the last row: zero fill
         if (!tc::make_tmap_bf16(&tmQ, q_hat, 2, dims, str, box)) return GQLA_ERR_CUDA;
     }
+    const uint64_t cdims[2] = {(uint64_t)(d.r_kv + d.d_r), (uint64_t)cache_rows};
+    const uint64_t cstr[1] = {(uint64_t)cache_row_stride * 2};
     {
-        const uint64_t dims[2] = {(uint64_t)(d.r_kv + d.d_r), (uint64_t)cache_rows};
-        const uint64_t str[1] = {(uint64_t)cache_row_stride * 2};
         const uint32_t box[2] = {64, pg != 0 ? (uint32_t)pg : 64u};
-        if (!tc::make_tmap_bf16(&tmC, cache, 2, dims, str, box)) return GQLA_ERR_CUDA;
+        if (!tc::make_tmap_bf16(&tmC, cache, 2, cdims, cstr, box)) return GQLA_ERR_CUDA;
     }
     tc::AbsorbParams p{};
     p.B = B; p.S = S; p.s_q = s_q; p.h_q = d.h_q; p.rows_total = rows_total; p.row_blocks = row_blocks;
@@ -428,23 +446,21 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
     if (o_final != nullptr && (balanced || S != 1)) return GQLA_ERR_UNSUPPORTED;
     const unsigned grid = (unsigned)(!tokens_on_m ? 2 * pairs : (balanced ? workers : B * S));  // pairs, or single CTAs
     cudaError_t e;
-    if (tokens_on_m && pg != 0)
-        e = rows_t == 16 ? (pg == 64   ? absorb_t_launch<16, 64>(p, tmQ, tmC, grid, st)
-                            : pg == 32 ? absorb_t_launch<16, 32>(p, tmQ, tmC, grid, st)
-                                       : absorb_t_launch<16, 16>(p, tmQ, tmC, grid, st))
-                         : (pg == 64   ? absorb_t_launch<32, 64>(p, tmQ, tmC, grid, st)
-                            : pg == 32 ? absorb_t_launch<32, 32>(p, tmQ, tmC, grid, st)
-                                       : absorb_t_launch<32, 16>(p, tmQ, tmC, grid, st));
+    if (pg != 0)
+        e = with_page_box(pg, [&](auto box_rows) {
+            constexpr int PG = decltype(box_rows)::value;
+            tc::CutMaps<PG> cut;
+            if (!make_cut_maps(&cut, cache, 2, cdims, cstr)) return cudaErrorInvalidValue;
+            if (!tokens_on_m) return absorb_pair_launch<PG>(p, tmQ, tmC, grid, st, cut);
+            return rows_t == 16 ? absorb_t_launch<16, PG>(p, tmQ, tmC, grid, st, cut)
+                                : absorb_t_launch<32, PG>(p, tmQ, tmC, grid, st, cut);
+        });
     else if (tokens_on_m)
         e = rows_t == 16   ? absorb_t_launch<16>(p, tmQ, tmC, grid, st)
             : rows_t == 32 ? absorb_t_launch<32>(p, tmQ, tmC, grid, st)
                            : absorb_t_launch<64>(p, tmQ, tmC, grid, st);
     else
-        e = pg == 0    ? (o_final != nullptr ? absorb_pair_launch<0, true>(p, tmQ, tmC, grid, st)
-                                             : absorb_pair_launch<0>(p, tmQ, tmC, grid, st))
-            : pg == 64 ? absorb_pair_launch<64>(p, tmQ, tmC, grid, st)
-            : pg == 32 ? absorb_pair_launch<32>(p, tmQ, tmC, grid, st)
-                       : absorb_pair_launch<16>(p, tmQ, tmC, grid, st);
+        e = o_final != nullptr ? absorb_pair_launch<0, true>(p, tmQ, tmC, grid, st) : absorb_pair_launch<0>(p, tmQ, tmC, grid, st);
     return e == cudaSuccess ? GQLA_OK : GQLA_ERR_CUDA;
 }
 
@@ -508,12 +524,12 @@ inline bool gqa_prefers_tokens(int rows_t) {
 
 template <int R, int PG = 0>
 inline cudaError_t gqa_t_launch(const tc::GqaParams& p, const CUtensorMap& q, const CUtensorMap& k, const CUtensorMap& r,
-                                const CUtensorMap& v, unsigned grid, cudaStream_t st) {
+                                const CUtensorMap& v, unsigned grid, cudaStream_t st, const tc::CutMaps<PG>& cut = {}) {
     using L = tc::GqaTSmem<R, PG>;
     auto kern = tc::decode_gqa_t_kernel<R, PG>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
     if (e != cudaSuccess) return e;
-    return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, k, r, v);
+    return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, k, r, v, cut);
 }
 
 template <int R>
@@ -551,6 +567,8 @@ inline gqla_status tc_decode_gqa(const gqla_dims& d, int32_t B, int32_t s_q, flo
     const bool tokens_on_m = pg != 0 || gqa_prefers_tokens(rows_t);
     if (tokens_on_m) R = gqa_rows_t(d, s_q, &hpg_box, &sq_box);
     CUtensorMap tmQ, tmK, tmR, tmV;
+    const uint64_t vdims[3] = {(uint64_t)d_v, (uint64_t)d.g, (uint64_t)n_rows};
+    const uint64_t vstr[2] = {(uint64_t)d_v * 2, (uint64_t)d.g * d_v * 2};
     {
         const int feat = d.d_h + d.d_r;
         const uint64_t dims[4] = {(uint64_t)feat, (uint64_t)hpg, (uint64_t)d.g, (uint64_t)B * s_q};
@@ -561,8 +579,6 @@ inline gqla_status tc_decode_gqa(const gqla_dims& d, int32_t B, int32_t s_q, flo
     {
         const uint64_t dims[3] = {(uint64_t)d.d_h, (uint64_t)d.g, (uint64_t)n_rows};
         const uint64_t str[2] = {(uint64_t)d.d_h * 2, (uint64_t)d.g * d.d_h * 2};
-        const uint64_t vdims[3] = {(uint64_t)d_v, (uint64_t)d.g, (uint64_t)n_rows};
-        const uint64_t vstr[2] = {(uint64_t)d_v * 2, (uint64_t)d.g * d_v * 2};
         const uint32_t box[3] = {64, 1, pg != 0 ? (uint32_t)pg : 128u};
         if (!tc::make_tmap_bf16(&tmK, k_c, 3, dims, str, box)) return GQLA_ERR_CUDA;
         if (!tc::make_tmap_bf16(&tmV, v, 3, vdims, vstr, box)) return GQLA_ERR_CUDA;
@@ -582,12 +598,13 @@ inline gqla_status tc_decode_gqa(const gqla_dims& d, int32_t B, int32_t s_q, flo
     p.rows = rows; p.seqlens = seqlens; p.o_part = o_part; p.lse_part = lse_part; p.status = status;
     cudaError_t e;
     if (pg != 0) {
-        e = R == 16 ? (pg == 64   ? gqa_t_launch<16, 64>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st)
-                       : pg == 32 ? gqa_t_launch<16, 32>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st)
-                                  : gqa_t_launch<16, 16>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st))
-                    : (pg == 64   ? gqa_t_launch<32, 64>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st)
-                       : pg == 32 ? gqa_t_launch<32, 32>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st)
-                                  : gqa_t_launch<32, 16>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st));
+        e = with_page_box(pg, [&](auto box_rows) {
+            constexpr int PG = decltype(box_rows)::value;
+            tc::CutMaps<PG> cut;
+            if (!make_cut_maps(&cut, v, 3, vdims, vstr)) return cudaErrorInvalidValue;
+            return R == 16 ? gqa_t_launch<16, PG>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st, cut)
+                           : gqa_t_launch<32, PG>(p, tmQ, tmK, tmR, tmV, (unsigned)units, st, cut);
+        });
         return e == cudaSuccess ? GQLA_OK : GQLA_ERR_CUDA;
     }
     if (tokens_on_m) {

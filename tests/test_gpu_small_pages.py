@@ -1,0 +1,71 @@
+"""Paged decode calls that the tensor-core kernels fetch in boxes within a page: pages of a multiple of 16 rows that are no
+multiple of the 128-row tile, and pieces that start inside a tile."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2605_15250_b200 import binding as B
+from paper_2605_15250_b200 import build as gbuild
+from paper_2605_15250_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+CANON = dict(h_q=128, g=8, d_h=128, r_kv=512, d_r=64)
+LLAMA = dict(CANON, h_q=32)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    gbuild.build()
+    assert torch.cuda.is_available()
+    B.lib()
+    B.set_policy(B.POLICY_AUTO)
+    yield
+    B.set_policy(B.POLICY_AUTO)
+
+
+def _absorb(bd, w, q_hat, cache, table, page, sl, S, status, scale=None):
+    o = torch.zeros((w.batch, abs(S), w.s_q, w.h_q, w.r_kv), device="cuda")
+    lse = torch.full((w.batch, abs(S), w.s_q, w.h_q), float("nan"), device="cuda")
+    B.gqla_decode_absorb_paged(bd, q_hat, cache, table, page, sl, w.scale if scale is None else scale, S, o, lse, status)
+    return o, lse
+
+
+def _gqa(bd, w, q, k_c, v, k_r, table, page, sl, S, status, scale=None):
+    o = torch.zeros((w.batch, abs(S), w.s_q, w.h_q, w.d_h), device="cuda")
+    lse = torch.full((w.batch, abs(S), w.s_q, w.h_q), float("nan"), device="cuda")
+    B.gqla_decode_gqa_paged(bd, q, k_c, v, k_r, table, page, sl, w.scale if scale is None else scale, S, o, lse, status)
+    return o, lse
+
+
+@pytest.mark.parametrize("dims", [CANON, LLAMA, dict(LLAMA, h_q=16)])
+@pytest.mark.parametrize("page,S,s_q", [(16, 1, 1), (16, -3, 2), (32, -3, 1), (48, 2, 1), (64, 1, 2), (64, -4, 1), (192, 3, 1), (128, 2, 1)])
+@pytest.mark.parametrize("fill", [float("nan"), float("inf")])
+def test_rows_that_no_sequence_owns_may_hold_anything(dims, page, S, s_q, fill):
+    """NaN or infinity in every row of the pool behind a sequence's end and in the spare pages: bit for bit what a pool
+    of zeros gives.  Ends at every remainder of eight rows, at the edges of boxes, tiles and pages."""
+    seqlens = np.array([*range(1, 18), 0, 31, 33, 62, 63, 64, 65, 71, 100, 127, 128, 129, 190, 193, 257, 300], dtype=np.int32)
+    w = synth.Workload("tails", batch=len(seqlens), s_q=s_q, dtype="bf16", seed=301, **dims)
+    x = synth.make_inputs(w, seqlens=seqlens, q_gain=4.0)
+    bd = B.make_dims(w.h_q, w.g, w.d_h, w.r_kv, w.d_r)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    sl = x["seqlens"].cuda()
+    zero, table = synth.to_paged(x["cache"], x["seq_start"], seqlens, page, seed=302, fill=0.0)
+    owned, _ = synth.to_paged(torch.ones(x["cache"].shape[0], 1), x["seq_start"], seqlens, page, seed=302, fill=0.0)
+    zero, table, free = zero.cuda(), table.cuda(), (owned[:, 0] == 0).cuda()
+    q = torch.cat([x["q_c"], x["q_r"]], -1).contiguous().cuda()
+    q_hat = torch.empty((w.batch, s_q, w.h_q, w.d_abs), dtype=torch.bfloat16, device="cuda")
+    B.gqla_absorb_q(bd, x["q_c"].cuda(), x["q_r"].cuda(), x["w_uk"].cuda(), q_hat)
+    k_c, v = (torch.empty((zero.shape[0], w.g, w.d_h), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    B.gqla_expand_cache(bd, zero, x["w_uk"].cuda(), x["w_uv"].cuda(), k_c, v, None)
+    got = []
+    for value in (0.0, fill):
+        cache, k, vv = zero.clone(), k_c.clone(), v.clone()
+        for plane in (cache, k, vv):
+            plane[free] = value
+        got.append((*_absorb(bd, w, q_hat, cache, table, page, sl, S, status),
+                    *_gqa(bd, w, q, k, vv, cache[:, w.r_kv:], table, page, sl, S, status)))
+    assert int(status.item()) == 0
+    for a, b, what in zip(*got, ("absorb o", "absorb lse", "gqa o", "gqa lse")):
+        assert not torch.isnan(b).any(), what
+        assert torch.equal(a, b), what
