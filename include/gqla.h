@@ -203,7 +203,7 @@ gqla_status gqla_decode_gqa_noalloc(const gqla_dims* dims, gqla_dtype dtype, int
  * a packed cache (so rows of a sequence's last page behind its end must hold finite values, as rows outside a
  * sequence do there; the other forms accept anything in them).  Other page sizes that are a multiple of 16,
  * and num_splits >= 2, run on forms of them
- * that fetch by pages and keep the probabilities to 16 bits (on the absorb path with 33 to 64 query rows
+ * that fetch by pages and keep the probabilities in fp32 precision (on the absorb path with 33 to 64 query rows
  * the balanced plan is then cut for half the SMs per 128 query rows, as in gqla_decode_absorb_fp8; on the
  * GQA path up to 32 padded query rows per group); everything else runs on the generic kernels. */
 gqla_status gqla_decode_absorb_paged(const gqla_dims* dims, gqla_dtype dtype, int32_t B, int32_t s_q, float scale,

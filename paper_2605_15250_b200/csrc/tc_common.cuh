@@ -477,9 +477,17 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&v);
 }
-// What the bf16 pair `hi` of (lo, hi) values left over, as a second bf16 pair: value = hi term + rest to 16 bits.
-__device__ __forceinline__ uint32_t pack_bf16_rest(float x0, float x1, uint32_t hi) {
-    return pack_bf16(x0 - __uint_as_float(hi << 16), x1 - __uint_as_float(hi & 0xffff0000u));
+// A pair of fp32 values as N bf16 terms each, out[n * stride] the pair of terms n.  Three terms are the value itself: every
+// term takes eight bits and the differences are exact, so nothing is left of the 24 bits (short of bf16's smallest number).
+template <int N>
+__device__ __forceinline__ void split_bf16(float x0, float x1, uint32_t* out, int stride) {
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+        const uint32_t t = pack_bf16(x0, x1);
+        out[n * stride] = t;
+        x0 -= __uint_as_float(t << 16);
+        x1 -= __uint_as_float(t & 0xffff0000u);
+    }
 }
 
 // ----------------------------------------------------------------------------- host: tensor maps

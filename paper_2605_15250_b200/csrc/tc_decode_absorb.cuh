@@ -33,8 +33,14 @@
 // and the tile's halves): the boxes of a group go out together, one lane of the producer warp each, after every lane has
 // looked its page up; boxes behind the sequence's end start behind the cache's last row and are filled with zeros, and of the
 // box that the end cuts V gets zeros behind it (load_cut_run): rows outside a sequence may hold anything.  Such
-// calls keep 32-bit probabilities: P is split into two bf16 terms (hi + lo, 16 bits) and P V is issued for both, the
-// second P buffer taking the place of one K group.  These calls ran one warp per query row on the SIMT kernel before,
+// calls keep 32-bit probabilities: P is split into three bf16 terms, which hold all of its 24 bits, and P V is issued for each of
+// them.  The two further P buffers are paid for by a K ring of five single column blocks in place of three groups of three, and
+// the products of the second and third term go to accumulators of their own where tensor memory has room for them (half of O
+// here, all of it in the tokens-on-M kernels): the tensor core truncates its running sums, so every further addition into one of
+// them costs bits (relative to O about 1.7e-8 per 16 rows and term).  What bounds it: the chain P V (3072 cycles a tile) -> P
+// written -> P V; 105 us a step on 32 sequences of 300-8000 rows in pages of 64 rows, 128 heads, where two terms took 88.
+// Errors of the merged partials there, against 64 bits: 3.6e-6 of the 2-norm (two terms 3.8e-6, SIMT kernel 3.4e-7); of the step:
+// 2.79e-3 with each of the three, from the roundings to bf16.  These calls ran one warp per query row on the SIMT kernel before,
 // which read every cache row h_q times from L2: 13.7 ms for 32 sequences of 300-8000 rows in pages of 64 rows.
 #pragma once
 #include "common.cuh"
@@ -62,12 +68,13 @@ template <int PG>
 struct AbsorbSmemT {
     static constexpr int kBox = 8192;              // 64 rows x 64 bf16, 128-byte swizzle
     static constexpr int kQBytes = 9 * kBox;       // 64 query rows x 576
-    static constexpr int kPTerms = PG != 0 ? 2 : 1;  // bf16 terms of a probability
+    static constexpr int kPTerms = PG != 0 ? 3 : 1;  // bf16 terms of a probability
     static constexpr int kPTerm = 2 * kBox;        // 64 rows x 128 tokens (two 64-token k-blocks)
     static constexpr int kPBytes = kPTerms * kPTerm;
-    static constexpr int kKGroup = 3 * kBox;       // three column blocks of this CTA's 64 rows of a tile
+    static constexpr int kKBlocks = PG != 0 ? 1 : 3;  // column blocks of a K group
+    static constexpr int kKGroup = kKBlocks * kBox;   // of this CTA's 64 rows of a tile
     static constexpr int kVGroup = 4 * kBox;       // 64 tokens x this CTA's 2 x 128 latent columns
-    static constexpr int kNK = PG != 0 ? 2 : 3;    // ring of K groups (Qh Kh^T operand): one tile
+    static constexpr int kNK = PG != 0 ? 5 : 3;    // ring of K groups (Qh Kh^T operand)
     static constexpr int kNV = 2;                  // ring of V groups (P V operand): one tile
     static constexpr int kOffK = kQBytes;
     static constexpr int kOffP = kOffK + kNK * kKGroup;
@@ -97,6 +104,7 @@ using AbsorbSmem = AbsorbSmemT<0>;
 
 constexpr uint32_t kAColO = 0;    // O: MMA m (latent columns [256m, 256m+256)) at TMEM columns [128m, 128m+128)
 constexpr uint32_t kAColS = 256;  // two 64-column score buffers
+constexpr uint32_t kAColRest = 384;  // small pages: the part of O's MMA 0 that the second and third terms of P give
 
 // FINAL: the whole-sequence call (o_final set); a form of its own, so that neither output's registers weigh on the softmax
 // loop of the other.
@@ -184,7 +192,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
         // (both CTAs).  Every "full" barrier lives in the leader and counts the bytes of BOTH CTAs.
         if constexpr (PG != 0) {
             constexpr int NB = 64 / PG;  // boxes per column block of this CTA's 64 rows
-            const int run = lane % NB, blk = lane / NB;
+            const int run = lane % NB;
             const uint32_t q_full_l = mapa(smem_u32(q_full), 0);
             int ks = 0;
             uint32_t kph = 1;
@@ -202,13 +210,13 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                     const int32_t row = next_row;
                     if (kt + 1 < pc.n_tiles) next_row = p.rows.run_row(pc.b, tok + (kt + 1) * 128, T, p.n_rows);
 #pragma unroll 1
-                    for (int kg = 0; kg < 3; ++kg) {
+                    for (int kg = 0; kg < 9; ++kg) {
                         if (!(ok = __all_sync(0xffffffffu, mbar_wait(&kempty[ks], kph, ab, 1)))) break;
                         if (cta == 0 && lane == 0) mbar_expect_tx(&kfull[ks], 2 * L::kKGroup);
                         __syncwarp();
-                        if (blk < 3)
-                            tma_load_2d_pair(tiles + L::kOffK + ks * L::kKGroup + blk * L::kBox + run * PG * 128, &tmC,
-                                             (3 * kg + blk) * 64, row, mapa(smem_u32(&kfull[ks]), 0));
+                        if (lane < NB)
+                            tma_load_2d_pair(tiles + L::kOffK + ks * L::kKGroup + run * PG * 128, &tmC, kg * 64, row,
+                                             mapa(smem_u32(&kfull[ks]), 0));
                         if (++ks == L::kNK) { ks = 0; kph ^= 1; }
                     }
                 }
@@ -332,18 +340,18 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
             auto issue_qk = [&](int n) -> bool {
                 const uint32_t d = tmem_base + kAColS + (uint32_t)(n & 1) * 64;
 #pragma unroll 1
-                for (int g3 = 0; g3 < 3; ++g3) {
+                for (int g = 0; g < 9 / L::kKBlocks; ++g) {
                     if (!mbar_wait_fast(&kfull[ks], kph, ab, 3)) return false;
                     tc_fence_after();
                     // descriptors as low words: the high word is a constant, stepping is one 32-bit add
                     const uint32_t kd = desc_lo(desc_kmajor_sw128(smem_u32(tiles + L::kOffK + ks * L::kKGroup)));
-                    const uint32_t qd = desc_lo(q_desc) + ((g3 * 3 * L::kBox) >> 4);
-                    if (g3 == 0)
+                    const uint32_t qd = desc_lo(q_desc) + ((g * L::kKBlocks * L::kBox) >> 4);
+                    if (g == 0)
                         umma_ss2_lo<false>(d, qd, kd, idesc_qk);  // the tile's first MMA overwrites S
                     else
                         umma_ss2_lo<true>(d, qd, kd, idesc_qk);
 #pragma unroll
-                    for (int i = 0; i < 3; ++i)
+                    for (int i = 0; i < L::kKBlocks; ++i)
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk)
                             if ((i | kk) != 0)
@@ -388,11 +396,15 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
 #pragma unroll
                             for (int kk = 1; kk < 4; ++kk)
                                 umma_ss2_lo<true>(dm, pd + ((kk * 32) >> 4), vd + ((m * 2 * L::kBox + kk * 2048) >> 4), idesc_pv);
-                            if constexpr (L::kPTerms == 2) {
 #pragma unroll
-                                for (int kk = 0; kk < 4; ++kk)
-                                    umma_ss2_lo<true>(dm, pd + ((L::kPTerm + kk * 32) >> 4),
-                                                      vd + ((m * 2 * L::kBox + kk * 2048) >> 4), idesc_pv);
+                            for (int kk = 4; kk < 4 * L::kPTerms; ++kk) {  // the other terms of P
+                                const uint32_t d = m == 0 ? tmem_base + kAColRest : dm;
+                                const uint32_t a = pd + (((kk >> 2) * L::kPTerm + (kk & 3) * 32) >> 4);
+                                const uint32_t b = vd + ((m * 2 * L::kBox + (kk & 3) * 2048) >> 4);
+                                if (m == 0 && kk == 4 && (t | h) == 0)
+                                    umma_ss2_lo<false>(d, a, b, idesc_pv);
+                                else
+                                    umma_ss2_lo<true>(d, a, b, idesc_pv);
                             }
                         }
                         umma_commit2(&vempty[vs], 3);
@@ -478,15 +490,14 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                     m_used = m_t;
                 }
                 const float m_sub = m_used == -INFINITY ? 0.f : m_used;
-                uint32_t pk[16], pl[L::kPTerms == 2 ? 16 : 1];
+                uint32_t pk[16 * L::kPTerms];  // [term][pair of columns]
                 if (full) {
 #pragma unroll
                     for (int c = 0; c < 32; c += 2) {
                         const float e0 = ex2(fmaf(__uint_as_float(x[c]), p.scale_log2, -m_sub));
                         const float e1 = ex2(fmaf(__uint_as_float(x[c + 1]), p.scale_log2, -m_sub));
                         l += e0 + e1;
-                        pk[c / 2] = pack_bf16(e0, e1);
-                        if constexpr (L::kPTerms == 2) pl[c / 2] = pack_bf16_rest(e0, e1, pk[c / 2]);
+                        split_bf16<L::kPTerms>(e0, e1, pk + c / 2, 16);
                     }
                 } else {
 #pragma unroll
@@ -495,8 +506,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                         const float e1 =
                             tok0 + c + 1 < lim ? ex2(fmaf(__uint_as_float(x[c + 1]), p.scale_log2, -m_sub)) : 0.f;
                         l += e0 + e1;
-                        pk[c / 2] = pack_bf16(e0, e1);
-                        if constexpr (L::kPTerms == 2) pl[c / 2] = pack_bf16_rest(e0, e1, pk[c / 2]);
+                        split_bf16<L::kPTerms>(e0, e1, pk + c / 2, 16);
                     }
                 }
                 // O may be rescaled, and the P buffer rewritten, only once P.V(n-1) has completed
@@ -508,8 +518,8 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 if (__any_sync(0xffffffffu, need) && t > 0) {
                     // this thread's share of the lane's O: columns [128m + 64ch, +64) for m = 0, 1
 #pragma unroll 1
-                    for (int c = 0; c < 4; ++c) {
-                        const uint32_t col = kAColO + (uint32_t)(c >> 1) * 128 + ch * 64 + (c & 1) * 32;
+                    for (int c = 0; c < (L::kPTerms > 1 ? 6 : 4); ++c) {
+                        const uint32_t col = (c < 4 ? kAColO + (uint32_t)(c >> 1) * 128 : kAColRest) + ch * 64 + (c & 1) * 32;
                         uint32_t o[32];
                         tmem_ld32(lane_base + col, o);
                         tmem_wait_ld();
@@ -522,15 +532,9 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 // P row r, k-block hf: 128 bytes = 8 chunks of 8 bf16, chunk index XORed with (r & 7)
                 uint8_t* prow = tiles + L::kOffP + hf * L::kBox + r * 128;
 #pragma unroll
-                for (int c4 = 0; c4 < 4; ++c4)
-                    *reinterpret_cast<uint4*>(prow + (((ch * 4 + c4) ^ (r & 7)) << 4)) =
+                for (int c4 = 0; c4 < 4 * L::kPTerms; ++c4)
+                    *reinterpret_cast<uint4*>(prow + (c4 >> 2) * L::kPTerm + (((ch * 4 + (c4 & 3)) ^ (r & 7)) << 4)) =
                         make_uint4(pk[4 * c4], pk[4 * c4 + 1], pk[4 * c4 + 2], pk[4 * c4 + 3]);
-                if constexpr (L::kPTerms == 2) {
-#pragma unroll
-                    for (int c4 = 0; c4 < 4; ++c4)
-                        *reinterpret_cast<uint4*>(prow + L::kPTerm + (((ch * 4 + c4) ^ (r & 7)) << 4)) =
-                            make_uint4(pl[4 * c4], pl[4 * c4 + 1], pl[4 * c4 + 2], pl[4 * c4 + 3]);
-                }
                 fence_proxy_async_smem();  // generic-proxy writes of P -> visible to the tensor core
                 tc_fence_before();
                 __syncwarp();
@@ -603,6 +607,13 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                         if (pc.n_tiles > 0 && ok) {  // warp-uniform
                             tmem_ld32(lane_base + kAColO + m * 128 + ch * 64 + c, o);
                             tmem_wait_ld();
+                            if (L::kPTerms > 1 && m == 0) {
+                                uint32_t rest[32];
+                                tmem_ld32(lane_base + kAColRest + ch * 64 + c, rest);
+                                tmem_wait_ld();
+#pragma unroll
+                                for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) + __uint_as_float(rest[i]));
+                            }
                         }
 #pragma unroll
                         for (int i = 0; i < 8; ++i)

@@ -37,7 +37,7 @@ namespace gqla {
 namespace tc {
 
 // PG: rows of a box for caches in small pages, 0 otherwise (see tc_decode_absorb.cuh: boxes within pages, probabilities in
-// two bf16 terms).  With 64 query rows the second term does not fit; the pair kernel serves those calls.
+// three bf16 terms).  With 64 query rows the further terms do not fit; the pair kernel serves those calls.
 template <int R, int PG = 0>
 struct AbsorbTSmem {
     static constexpr int kTile = 64;                          // tokens per tile
@@ -48,7 +48,8 @@ struct AbsorbTSmem {
     static constexpr int kStages = 2;
     static constexpr int kPRow = 2 * R;                       // one token's R probabilities (bf16)
     static constexpr int kPSwzBits = R == 64 ? 3 : (R == 32 ? 2 : 1);  // swizzle span = row length (128 / 64 / 32 bytes)
-    static constexpr int kPTerms = PG != 0 ? 2 : 1;           // bf16 terms of a probability
+    static constexpr int kPTerms = PG != 0 ? 3 : 1;           // bf16 terms of a probability
+    static constexpr int kAcc = PG != 0 ? 2 : 1;              // accumulators: the first terms' products, the other terms'
     static constexpr int kPTerm = (kTile * kPRow + 1023) / 1024 * 1024;
     static constexpr int kPBuf = kPTerms * kPTerm;
     static constexpr int kPBufs = R == 64 ? 1 : 2;            // P^T buffers (one where Qh takes 72 KB: P(n) waits for P.V(n-1))
@@ -107,9 +108,9 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + L::kNumBars);
     volatile int32_t* abort_flag = reinterpret_cast<volatile int32_t*>(tmem_slot + 1);
 
-    // TMEM columns: two score buffers of R columns, then four output blocks of R columns
-    constexpr uint32_t kColS = 0, kColO = 2 * R;
-    constexpr uint32_t kTmemCols = 6 * R <= 128 ? 128 : (6 * R <= 256 ? 256 : 512);
+    // TMEM columns: two score buffers of R columns, then four output blocks of R columns per accumulator
+    constexpr uint32_t kColS = 0, kColO = 2 * R, kColsUsed = (2 + 4 * L::kAcc) * R;
+    constexpr uint32_t kTmemCols = kColsUsed <= 128 ? 128 : (kColsUsed <= 256 ? 256 : 512);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const Abort ab{abort_flag, p.status};
@@ -262,13 +263,15 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                                     for (int ks = 0; ks < 4; ++ks)  // 16 tokens per step
                                         umma_ss_lo(tmem_base + kColO + m * R, v_lo + ((2 * m * L::kBox + ks * 2048) >> 4), v_hi,
                                                    p_lo + ((ks * 16 * L::kPRow) >> 4), p_hi, idesc_pv, (pv_tile | ks) != 0);
-                                if constexpr (L::kPTerms == 2) {
+                                if constexpr (L::kPTerms > 1) {
 #pragma unroll
                                     for (int m = 0; m < 4; ++m)
 #pragma unroll
-                                        for (int ks = 0; ks < 4; ++ks)
-                                            umma_ss_lo(tmem_base + kColO + m * R, v_lo + ((2 * m * L::kBox + ks * 2048) >> 4),
-                                                       v_hi, p_lo + ((L::kPTerm + ks * 16 * L::kPRow) >> 4), p_hi, idesc_pv, 1);
+                                        for (int ks = 4; ks < 4 * L::kPTerms; ++ks)  // the other terms of P
+                                            umma_ss_lo(tmem_base + kColO + (4 + m) * R,
+                                                       v_lo + ((2 * m * L::kBox + (ks & 3) * 2048) >> 4), v_hi,
+                                                       p_lo + (((ks >> 2) * L::kPTerm + (ks & 3) * 16 * L::kPRow) >> 4), p_hi,
+                                                       idesc_pv, pv_tile != 0 || ks != 4);
                                 }
                                 umma_commit(&empty[s]);
                                 umma_commit(&pv_done[s]);
@@ -410,7 +413,7 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
 #pragma unroll
                                 for (int c = 0; c < 8; ++c) f8[c] = __shfl_sync(0xffffffffu, factor[(c & 1) + 2 * (cc >> 3)], c >> 1);
 #pragma unroll
-                                for (int m = 0; m < 4; ++m) {
+                                for (int m = 0; m < 4 * L::kAcc; ++m) {
                                     uint32_t o[8];
                                     tmem_ld8(lane_base + kColO + m * R + r0 + cc, o);
                                     tmem_wait_ld();
@@ -425,8 +428,7 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                 }
                 // probabilities: a bf16 pair (the thread's two rows) into each of its two tokens' rows of P^T
                 const int pbi = n % L::kPBufs;
-                uint32_t pk[NJ];  // [2 h + pair]: the bf16 pair of token h for the thread's row pair
-                uint32_t pl[NJ];  // (small pages) the pair's second term
+                uint32_t pk[L::kPTerms * NJ];  // [term][2 h + pair]: the bf16 pair of token h for the thread's row pair
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -436,9 +438,7 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                         const float e1 = xs[i + 1] > -INFINITY ? ex2(xs[i + 1] - m_ref[jp + 1]) : 0.f;
                         l[jp] += e0;
                         l[jp + 1] += e1;
-                        pk[(NJ / 2) * h + (jp >> 1)] = pack_bf16(e0, e1);
-                        if constexpr (L::kPTerms == 2)
-                            pl[(NJ / 2) * h + (jp >> 1)] = pack_bf16_rest(e0, e1, pk[(NJ / 2) * h + (jp >> 1)]);
+                        split_bf16<L::kPTerms>(e0, e1, pk + (NJ / 2) * h + (jp >> 1), NJ);
                     }
                 // a single P^T buffer is still being read by P.V(n-1)
                 if (L::kPBufs == 1 && t > 0 && okl)
@@ -451,9 +451,9 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                     for (int jp = 0; jp < NJ; jp += 2) {
                         const uint32_t col = (uint32_t)(r0 + rj(jp)) * 2;                      // byte of that row pair in it
                         uint8_t* dst = p_smem + pbi * L::kPBuf + off + (((col >> 4) ^ pswz) << 4) + (col & 15);
-                        *reinterpret_cast<uint32_t*>(dst) = pk[(NJ / 2) * h + (jp >> 1)];
-                        if constexpr (L::kPTerms == 2)
-                            *reinterpret_cast<uint32_t*>(dst + L::kPTerm) = pl[(NJ / 2) * h + (jp >> 1)];
+#pragma unroll
+                        for (int n = 0; n < L::kPTerms; ++n)
+                            *reinterpret_cast<uint32_t*>(dst + n * L::kPTerm) = pk[n * NJ + (NJ / 2) * h + (jp >> 1)];
                     }
                 }
                 fence_proxy_async_smem();  // generic-proxy writes of P^T -> visible to the tensor core
@@ -504,7 +504,13 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                     uint32_t o[8];
                     if (nt > 0 && ok) {  // warp-uniform
                         tmem_ld8(lane_base + kColO + m * R + r0 + cc, o);
+                        uint32_t rest[8];
+                        if constexpr (L::kAcc == 2) tmem_ld8(lane_base + kColO + (4 + m) * R + r0 + cc, rest);
                         tmem_wait_ld();
+                        if constexpr (L::kAcc == 2) {
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) + __uint_as_float(rest[c]));
+                        }
                     }
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {

@@ -414,7 +414,7 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
     const int row_blocks = (rows_total + 127) / 128;
     const int rows_t = absorb_rows_t(d, s_q);
     const bool small_pages = page_box_rows(rows, S <= 1) != 0;  // S < 0: the balanced plan's pieces start on tile boundaries
-    // two-term probabilities of 64 query rows do not fit the tokens-on-M kernel: small pages take the pair kernel there
+    // the terms of 64 query rows' probabilities do not fit the tokens-on-M kernel: small pages take the pair kernel there
     const bool tokens_on_m = absorb_prefers_tokens(d, s_q) && !(small_pages && rows_t > 32);
     // S < 0: balanced plan with -S slots per sequence, W persistent CTAs (tokens-on-M) or pairs per row block
     const int32_t workers = S >= 0 ? 0 : (tokens_on_m ? sm_count() : pair_balanced_workers(d, s_q));

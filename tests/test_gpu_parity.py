@@ -820,9 +820,9 @@ def test_fused_merge_up_projection_over_slots(h_q, g, Bn, s_q, S):
                                              (128, 3, 1), (256, 6, 2)])
 def test_small_pages_on_the_tensor_cores(dims, page_size, S, s_q):
     """Pages that are no multiple of the 128-row tile (and pieces that start inside one): boxes of 64, 32 or 16 rows, lengths at
-    the edges of boxes, pages and tiles, against the oracle in fp32.  These calls keep probabilities to 16 bits (two bf16
-    terms): |do| <= 2 (2^-17 + dx) max|v| with dx <= 2^-13 for the fp32 scores (|x| up to about 30, 576 products),
-    a sixth of what one bf16 term would give at its worst (2^-9 max|v|)."""
+    the edges of boxes, pages and tiles, against the oracle in fp32.  The bound is
+    |do| <= 2 (2^-17 + dx) max|v| with dx <= 2^-13 for the fp32 scores (|x| up to about 30, 576 products),
+    a sixth of what probabilities of one bf16 term would give at their worst (2^-9 max|v|)."""
     from tests.parity_util import dims_of, round_to
     from oracle import gqla_oracle as O
     seqlens = np.array([1, 15, 16, 17, 31, 33, 47, 48, 49, 63, 64, 65, 127, 128, 129, 0, 191, 192, 193, 333, 1031], dtype=np.int32)

@@ -69,3 +69,41 @@ def test_rows_that_no_sequence_owns_may_hold_anything(dims, page, S, s_q, fill):
     for a, b, what in zip(*got, ("absorb o", "absorb lse", "gqa o", "gqa lse")):
         assert not torch.isnan(b).any(), what
         assert torch.equal(a, b), what
+
+
+@pytest.mark.parametrize("dims", [CANON, LLAMA, dict(LLAMA, h_q=16)])
+@pytest.mark.parametrize("page,S,s_q", [(16, 1, 1), (32, -3, 2), (64, 1, 2), (64, 3, 1), (192, -2, 1), (128, 2, 1)])
+def test_probabilities_keep_their_24_bits(dims, page, S, s_q):
+    """Value rows are unit vectors, so every output element is one probability, and the keys are too, so every score is one
+    query element, exactly.  What is left are the roundings of x = s log2(e) (|s| <= 1/2: 3 * 2^-25), ex2 (2^-22) in the
+    probability and in the sum, and a few of 2^-24 in the normalisation and the merge: below 2^-20 in all.  Probabilities cut to
+    16 bits miss by up to 2^-17."""
+    seqlens = np.array([1, 2, 5, 16, 63, 64, 65, 100, 127, 128], dtype=np.int32)
+    w = synth.Workload("onehot", batch=len(seqlens), s_q=s_q, dtype="bf16", seed=303, **dims)
+    gen = torch.Generator().manual_seed(304)
+    scale = 0.25
+    rows = torch.cat([torch.eye(128)[:n] for n in seqlens]).bfloat16()
+    starts = np.concatenate([[0], np.cumsum(seqlens)[:-1]])
+    pool, table = synth.to_paged(rows, starts, seqlens, page, seed=305, fill=0.0)
+    pool, table, sl = pool.cuda(), table.cuda(), torch.from_numpy(seqlens).cuda()
+    cache = torch.zeros((pool.shape[0], w.r_kv + w.d_r), dtype=torch.bfloat16, device="cuda")
+    cache[:, :128] = pool
+    k_c = pool[:, None, :].expand(-1, w.g, -1).contiguous()
+    x = (4 * torch.rand((w.batch, s_q, w.h_q, 128), generator=gen) - 2).bfloat16()
+    zeros = torch.zeros((w.batch, s_q, w.h_q, w.r_kv - 128 + w.d_r), dtype=torch.bfloat16)
+    q_hat, q = torch.cat([x, zeros], -1).cuda(), torch.cat([x, zeros[..., :w.d_r]], -1).cuda()
+    bd = B.make_dims(w.h_q, w.g, w.d_h, w.r_kv, w.d_r)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    s = scale * x.double()
+    for b, n in enumerate(seqlens):
+        for p in range(s_q):
+            s[b, p, :, max(0, int(n) - (s_q - 1 - p)):] = -np.inf
+    ref = torch.nan_to_num(torch.softmax(s, -1))  # a query that sees nothing gives 0
+    for o, lse, what in ((*_absorb(bd, w, q_hat, cache, table, page, sl, S, status, scale), "absorb"),
+                         (*_gqa(bd, w, q, k_c, k_c, cache[:, w.r_kv:], table, page, sl, S, status, scale), "gqa")):
+        out = torch.empty((w.batch, s_q, w.h_q, o.shape[-1]), device="cuda")
+        B.gqla_combine_splits(o, lse, out)
+        got = out.double().cpu()
+        assert int(status.item()) == 0 and not got[..., 128:].any()
+        err = ((got[..., :128] - ref).abs() / torch.where(ref > 0, ref, torch.ones(()).double())).max()
+        assert err <= 2.0 ** -20, (what, float(err))
