@@ -6,6 +6,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <float.h>
 #include <stdint.h>
 
 namespace gqla {
@@ -476,6 +477,14 @@ __device__ __forceinline__ float ex2(float x) {
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&v);
+}
+// x / y from x, y and the rounded reciprocal of y: the product, corrected once by its exact remainder (P. Markstein, Computation of
+// elementary functions on the IBM RISC System/6000 processor, IBM J. Res. Dev. 34, 1990).  For where many x share one y: with a
+// division per x a step took 14.0 us instead of 12.7 (one sequence of 3001 rows, GQA path), like this 12.4, uncorrected 12.6.
+// The remainder of an infinite x is NaN, for which fminf gives a finite number: infinity stays what it is.
+__device__ __forceinline__ float div_by(float x, float y, float recip) {
+    const float q = x * recip;
+    return fmaf(fminf(fmaf(-q, y, x), FLT_MAX), recip, q);
 }
 // A pair of fp32 values as N bf16 terms each, out[n * stride] the pair of terms n.  Three terms are the value itself: every
 // term takes eight bits and the differences are exact, so nothing is left of the 24 bits (short of bf16's smallest number).

@@ -497,8 +497,8 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                         for (int c = 0; c < CH; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) + __uint_as_float(rest[c]));
                     }
                 }
-                // lane c finishes row c of the chunk (one division and one logarithm per warp side by side, not CH in a
-                // row: done by every thread for every row they took 5700 cycles of a piece), the others get its factor
+                // lane c finishes row c of the chunk (one reciprocal and one logarithm per warp side by side, not CH in a
+                // row: done by every thread for every row they took 5700 cycles of a piece), the others get its sum and factor
                 const int rl = ch * CH + (lane & (CH - 1)), r = r0 + rl;
                 float mr = m_ref[ch * CH];
 #pragma unroll
@@ -513,10 +513,10 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
 #pragma unroll
                 for (int c = 0; c < CH; ++c) {
                     const int rc = r0 + ch * CH + c, pq = rc >> hshift, il = rc & (p.hpg_box - 1);
-                    const float f = __shfl_sync(0xffffffffu, inv, c);
+                    const float f = __shfl_sync(0xffffffffu, inv, c), sum = __shfl_sync(0xffffffffu, Lt, c);
                     // lane tl holds value column tl of every row: 128 consecutive floats per row
                     if (il < p.hpg && pq < p.s_q)  // padding rows are computed and dropped
-                        o_base[(int64_t)(pq * p.h_q + il) * p.d_v] = f > 0.f ? __uint_as_float(o[c]) * f : 0.f;
+                        o_base[(int64_t)(pq * p.h_q + il) * p.d_v] = f > 0.f ? div_by(__uint_as_float(o[c]), sum, f) : 0.f;
                 }
             }
             named_bar_sync(1, kSmT);  // red may be rewritten by the next piece

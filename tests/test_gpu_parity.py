@@ -923,3 +923,31 @@ def test_balanced_plan_of_the_kernels_is_the_host_plan(Bn, path):
     assert int(status.item()) == 0
     live = np.isfinite(merged[1])
     assert np.array_equal(live, np.isfinite(merged[0])) and np.abs(merged[0][live] - merged[1][live]).max(initial=0.0) <= 1e-5
+
+
+@pytest.mark.parametrize("dims", [CANON, LLAMA])
+@pytest.mark.parametrize("s_q", [1, 2])
+def test_gqa_partials_are_divided_by_their_sum(dims, s_q):
+    """Zero queries and whole-number values: every probability is 1, the sums are exact, and a partial is the fp32 quotient of
+    two whole numbers, bit for bit, or an infinity that the values hold (a multiplication by the rounded reciprocal misses it at 49 equal values, for one)."""
+    seqlens = np.array([*range(1, 131), 301, 777, 1031], dtype=np.int32)
+    w = _wl("quotients", len(seqlens), s_q, 306, **dims)
+    gen = torch.Generator().manual_seed(307)
+    starts = np.concatenate([[0], np.cumsum(seqlens)[:-1]])
+    N = int(seqlens.sum())
+    v = torch.randint(-200, 201, (N, w.g, w.d_h), generator=gen).bfloat16()
+    v[0, :, :4], v[0, :, 4:9] = np.inf, -np.inf  # the only row of sequence 0, in front of all others
+    q = torch.zeros((w.batch, s_q, w.h_q, w.d_h + w.d_r), dtype=torch.bfloat16, device="cuda")
+    k_c, k_r = (torch.randn(shape, generator=gen).bfloat16().cuda() for shape in ((N, w.g, w.d_h), (N, w.d_r)))
+    o = torch.empty((w.batch, 1, s_q, w.h_q, w.d_h), device="cuda")
+    lse = torch.empty((w.batch, 1, s_q, w.h_q), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.gqla_decode_gqa(B.make_dims(w.h_q, w.g, w.d_h, w.r_kv, w.d_r), q, k_c, v.cuda(), k_r, torch.from_numpy(starts).cuda(),
+                      torch.from_numpy(seqlens).cuda(), w.scale, 1, o, lse, status)
+    assert int(status.item()) == 0
+    got = o.cpu().view(w.batch, s_q, w.g, w.h_q // w.g, w.d_h)
+    for b, (lo, n) in enumerate(zip(starts, seqlens)):
+        for p in range(s_q):
+            t = int(n) - (s_q - 1 - p)
+            ref = v[lo:lo + t].float().sum(0) / max(t, 1)  # whole numbers below 2^24: exact in any order
+            assert torch.equal(got[b, p], ref[:, None].expand(-1, w.h_q // w.g, -1)), (int(n), p)
