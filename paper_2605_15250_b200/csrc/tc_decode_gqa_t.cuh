@@ -493,8 +493,11 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                     if constexpr (L::kAcc == 2) tmem_ld_n(lane_base + kColO + R + r0 + ch * CH, rest, CH);
                     tmem_wait_ld();
                     if constexpr (L::kAcc == 2) {
+                        // an infinite value makes the first accumulator infinite and leaves infinities of either sign, or NaN
+                        // from a zero term, in the other: the first one decides
 #pragma unroll
-                        for (int c = 0; c < CH; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) + __uint_as_float(rest[c]));
+                        for (int c = 0; c < CH; ++c)
+                            o[c] = __float_as_uint(__uint_as_float(o[c]) + fmaxf(fminf(__uint_as_float(rest[c]), FLT_MAX), -FLT_MAX));
                     }
                 }
                 // lane c finishes row c of the chunk (one reciprocal and one logarithm per warp side by side, not CH in a

@@ -107,3 +107,35 @@ def test_probabilities_keep_their_24_bits(dims, page, S, s_q):
         assert int(status.item()) == 0 and not got[..., 128:].any()
         err = ((got[..., :128] - ref).abs() / torch.where(ref > 0, ref, torch.ones(()).double())).max()
         assert err <= 2.0 ** -20, (what, float(err))
+
+
+@pytest.mark.parametrize("h_q,s_q", [(128, 1), (128, 2), (32, 1)])
+@pytest.mark.parametrize("page,S", [(16, 1), (64, -2), (128, 2)])
+def test_infinite_values_stay_infinite_on_the_gqa_path(h_q, s_q, page, S):
+    """An infinity among the values of a sequence reaches the output as itself (it is a sum with positive weights), also where the
+    second and third term of a probability are zero or negative; the sequences beside it are untouched."""
+    seqlens = np.array([2, 40, 70, 200], dtype=np.int32)
+    w = synth.Workload("inf", batch=len(seqlens), s_q=s_q, dtype="bf16", seed=308, **dict(CANON, h_q=h_q))
+    x = synth.make_inputs(w, seqlens=seqlens)
+    table = synth.to_paged(x["cache"], x["seq_start"], seqlens, page, seed=309)[1].cuda()
+    n = 1 + int(table.max()) + 3
+    gen = torch.Generator().manual_seed(310)
+    k_c, v = (torch.randn((n * page, w.g, w.d_h), generator=gen).bfloat16().cuda() for _ in range(2))
+    k_r = torch.randn((n * page, w.d_r), generator=gen).bfloat16().cuda()
+    q = torch.cat([x["q_c"], x["q_r"]], -1).contiguous()
+    q[0] = 0  # equal probabilities: their further terms are zero
+    bd = B.make_dims(w.h_q, w.g, w.d_h, w.r_kv, w.d_r)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def step():
+        o, lse = _gqa(bd, w, q.cuda(), k_c, v, k_r, table, page, x["seqlens"].cuda(), S, status)
+        out = torch.empty((w.batch, s_q, w.h_q, w.d_h), device="cuda")
+        B.gqla_combine_splits(o, lse, out)
+        return out
+
+    ref = step()
+    for b in (0, 2):
+        row = int(table[b, 0]) * page  # the sequence's first row, which every query sees
+        v[row, :, :3], v[row, :, 3:7] = np.inf, -np.inf
+        ref[b, ..., :3], ref[b, ..., 3:7] = np.inf, -np.inf
+    assert torch.equal(step(), ref) and int(status.item()) == 0
