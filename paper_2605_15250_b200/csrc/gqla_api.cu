@@ -141,6 +141,7 @@ const char* gqla_kernel_for(const gqla_dims* d, gqla_dtype dtype, int32_t s_q, i
     if (check_dims(d) != GQLA_OK) return "invalid";
     if (g_policy.load() != GQLA_POLICY_AUTO) return "generic";
     if (path == 2) return tc_gemm_covers(*d, dtype) ? "tcgen05" : "generic";
+    if (path == 3) return tc_combine_up_covers(*d, dtype) ? "tcgen05" : "generic";
     return tc_covers(*d, dtype, s_q, path) ? "tcgen05" : "generic";
 }
 

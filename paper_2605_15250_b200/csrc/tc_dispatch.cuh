@@ -326,13 +326,17 @@ inline gqla_status tc_append_expand(const gqla_dims& d, gqla_dtype dtype, int32_
 }
 
 // Fused split merge + up-projection; covers what tc_up_proj covers with d_h = 128 and r_kv % 128 == 0.
+// Shapes the fused merge + up-projection covers: those of the projections with at most 64 head slots per group (a tile's rows)
+// and r_kv <= 512 (both operands resident), up to CombineUpSmem::kMaxS slots.
+inline bool tc_combine_up_covers(const gqla_dims& d, gqla_dtype dtype) {
+    return tc_gemm_covers(d, dtype) && next_pow2(d.h_q / d.g) <= tc::CombineUpSmem::kRows &&
+           d.r_kv <= tc::CombineUpSmem::kMaxChunks * tc::CombineUpSmem::kChunkK;
+}
 inline gqla_status tc_combine_up_proj(const gqla_dims& d, gqla_dtype dtype, int32_t B, int32_t s_q, int32_t S,
                                       const float* o_part, const float* lse_part, const void* w_uv, void* o, float* lse,
                                       cudaStream_t st) {
     const int hpg = d.h_q / d.g, hpb = next_pow2(hpg);
-    if (!tc_gemm_covers(d, dtype) || S > tc::CombineUpSmem::kMaxS || hpb > 64 ||
-        d.r_kv > tc::CombineUpSmem::kMaxChunks * tc::CombineUpSmem::kChunkK)
-        return GQLA_ERR_UNSUPPORTED;
+    if (!tc_combine_up_covers(d, dtype) || S > tc::CombineUpSmem::kMaxS) return GQLA_ERR_UNSUPPORTED;
     const int64_t positions = (int64_t)B * s_q;
     // a group's rows in as many runs as there are SMs for a group, at least four rows each (one per builder warp of a quarter)
     const int64_t group_rows = positions * hpb;

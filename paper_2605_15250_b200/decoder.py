@@ -91,9 +91,13 @@ class GqlaDecoder:
         else:
             B.gqla_decode_absorb_paged(self.dims, q_hat, self.cache, self.block_table, self.page_size, self.seqlens,
                                        self.scale, num_splits, o_part, lse_part, self.status)
-        # with many slots per sequence the fused kernel (a warp walks the slots of a row) falls behind the separate merge,
-        # which spreads them over thread groups: 9.4 against 10.0 us at 11 slots, 10.7 against 9.9 us at 20
-        if fused_tail and slots <= 12:
+        # With many slots per sequence the fused tensor-core kernel (a warp walks the slots of a row) falls behind the separate
+        # merge, which spreads them over thread groups: 9.4 against 10.0 us at 11 slots, 10.7 against 9.9 us at 20.  Where the
+        # generic fused kernel (a block per row, which reads all of W^UV) would take the place of a tensor-core or faster
+        # up-projection, few slots only: 34 against 8.4 us (4 sequences, one group of 128 heads), 69 against 12 (8, 128 heads,
+        # r_kv = 1024) and 60 against 49 (32, 64 heads, r_kv = 384) at eight slots.  In fp32 it has no such rival: 32 against 68.
+        if fused_tail and (slots <= 4 or slots <= 12 and (self.dtype == torch.float32 or B.kernel_for(
+                self.dims, self.dtype, s_q, "fused_tail") == "tcgen05")):
             B.gqla_combine_up_proj(self.dims, o_part, lse_part, self.w_uv, o, lse)
         else:
             B.gqla_combine_splits(o_part, lse_part, o_hat, lse)
