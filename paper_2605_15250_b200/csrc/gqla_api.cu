@@ -24,10 +24,6 @@ gqla_status check_dims(const gqla_dims* d) {
 }
 gqla_status check_dtype(gqla_dtype t) { return (t == GQLA_BF16 || t == GQLA_F32) ? GQLA_OK : GQLA_ERR_DTYPE; }
 
-// gqla_combine_splits: grids of up to this many threads get narrower items and split slots
-constexpr int64_t kCombineFewThreads = 65536;
-constexpr int64_t kCombineWave = 148 * 4 * kCombineThreads;  // threads of it that are resident at once
-
 gqla_status launch_status() { return cudaGetLastError() == cudaSuccess ? GQLA_OK : GQLA_ERR_CUDA; }
 
 gqla_status launch_decode_generic(gqla_dtype dtype, const DecodeArgs& a, cudaStream_t st) {
@@ -479,15 +475,17 @@ gqla_status gqla_combine_splits(int32_t B, int32_t rows_per_seq, int32_t num_spl
     if (rows > 0x7fffffffLL) return GQLA_ERR_SHAPE;
     cudaStream_t st = (cudaStream_t)stream;
     if (d_out % 4 == 0) {
-        // Columns per thread (V) and thread groups that share a row's slots (G): the widest item while it still gives
-        // half of the threads that fit beside a decode kernel's CTAs (such a grid is resident as one wave while it
-        // waits for them), narrower ones and split slots below that, where the chain of loads is what takes the time -- as
-        // long as the grid is still resident as one wave (512 rows x 512 columns x 20 slots: 5.5 us with two groups,
+        // Columns per thread (V) and thread groups that share a row's slots (G).  `wave`: threads that are resident at once,
+        // four blocks per SM (148 where the device cannot be asked).  The widest item while it still gives 65536 threads on 148
+        // SMs, two fifths of a wave; narrower ones and split slots below that, where the chain of loads is what takes the time
+        // -- as long as the grid is still one wave (512 rows x 512 columns x 20 slots: 5.5 us with two groups,
         // 9.7 with four, whose blocks took two and a half waves; 128 rows x 8 slots: 3.2 against 5.3 us).
+        const int64_t sms = sm_count() > 0 ? sm_count() : 148;
+        const int64_t wave = sms * 4 * kCombineThreads, few = 65536 * sms / 148;
         int vec = d_out % 16 == 0 ? 16 : (d_out % 8 == 0 ? 8 : 4);
-        while (vec > 4 && rows * (d_out / vec) <= kCombineFewThreads) vec /= 2;
+        while (vec > 4 && rows * (d_out / vec) <= few) vec /= 2;
         int groups = 1;
-        while (vec == 4 && groups < 8 && 2 * groups <= num_splits && 2 * rows * (d_out / 4) * groups <= kCombineWave) groups *= 2;
+        while (vec == 4 && groups < 8 && 2 * groups <= num_splits && 2 * rows * (d_out / 4) * groups <= wave) groups *= 2;
         const int64_t items = rows * (d_out / vec);
         const int64_t nblk = (items * groups + kCombineThreads - 1) / kCombineThreads;
         if (nblk > 0x7fffffffLL) return GQLA_ERR_SHAPE;
