@@ -37,9 +37,10 @@ struct RowMap {
         return (int64_t)block_table[(int64_t)b * max_pages + t / page_size] * page_size + t % page_size;
     }
     // First cache row of a run of rows t.. that lies within one page; `beyond` where the sequence (T rows) has ended:
-    // the block table says nothing about pages behind it.
-    __device__ __forceinline__ int32_t run_row(int32_t b, int32_t t, int32_t T, int32_t beyond) const {
-        return t < T ? (int32_t)row(b, t) : beyond;
+    // the block table says nothing about pages behind it.  Unsigned, because a run is looked up ahead of the tile that needs
+    // it: behind an end close to 2^31 its row number would wrap to a negative one, in front of the table.
+    __device__ __forceinline__ int32_t run_row(int32_t b, uint32_t t, int32_t T, int32_t beyond) const {
+        return t < (uint32_t)T ? (int32_t)row(b, (int32_t)t) : beyond;
     }
 };
 

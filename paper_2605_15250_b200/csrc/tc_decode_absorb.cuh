@@ -204,7 +204,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 if (cta == 0 && lane == 0) mbar_expect_tx(q_full, 2 * L::kQBytes);
                 __syncwarp();
                 if (lane < 9) tma_load_2d_pair(tiles + lane * L::kBox, &tmQ, lane * 64, pc.b * p.rows_total + rho0, q_full_l);
-                const int32_t tok = pc.tok_begin + (int)cta * 64 + run * PG;  // this lane's run of rows in the first tile
+                const uint32_t tok = pc.tok_begin + (int)cta * 64 + run * PG;  // this lane's run of rows in the first tile
                 int32_t next_row = p.rows.run_row(pc.b, tok, T, p.n_rows);
                 for (int kt = 0; kt < pc.n_tiles && ok; ++kt) {
                     const int32_t row = next_row;
@@ -271,7 +271,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 if (pc.n_tiles == 0) continue;
                 const int32_t T = p.seqlens[pc.b];
                 if (pi > 0 && !(ok = __all_sync(0xffffffffu, mbar_wait(epi_done, (pi - 1) & 1, ab, 16)))) break;
-                const int32_t tok = pc.tok_begin + run * PG;
+                const uint32_t tok = pc.tok_begin + run * PG;
                 int32_t next_row = p.rows.run_row(pc.b, tok, T, p.n_rows);
                 for (int vg = 0; vg < 2 * pc.n_tiles; ++vg) {  // (tile, token half)
                     const int32_t row = next_row;

@@ -156,7 +156,8 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
             while (ok && walk.next(pc)) {
                 if (pc.n_tiles == 0) continue;
                 const int nt = (pc.tok_end - pc.tok_begin + TK - 1) / TK;
-                const int32_t T = p.seqlens[pc.b], tok = pc.tok_begin + run * PG;
+                const int32_t T = p.seqlens[pc.b];
+                const uint32_t tok = pc.tok_begin + run * PG;
                 if (pi > 0 && !(ok = __all_sync(0xffffffffu, mbar_wait(q_empty, (pi - 1) & 1, ab, 13)))) break;
                 if (lane == 0) mbar_expect_tx(q_full, L::kQBytes);
                 __syncwarp();

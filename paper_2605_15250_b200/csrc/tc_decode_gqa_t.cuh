@@ -203,7 +203,8 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
             bool ok = true;
             while (ok && walk.next(pc)) {
                 if (pc.n_tiles == 0) continue;
-                const int32_t T = p.seqlens[pc.b], tok = pc.tok_begin + run * PG;
+                const int32_t T = p.seqlens[pc.b];
+                const uint32_t tok = pc.tok_begin + run * PG;
                 int32_t next_row = p.rows.run_row(pc.b, tok, T, p.n_rows);
                 for (int t = 0; t < pc.n_tiles; ++t, ++gt) {
                     const int s = gt & 1;
