@@ -47,11 +47,14 @@ struct CombineUpSmem {
     static_assert(OneCtaPerSM<kTotal>::value, "");
 };
 
-__device__ __forceinline__ float4 ld_partial4(const float* p) {  // read once: do not keep in L1
+// Read once: do not keep in L1.  A coherent load, not the read-only one: the kernel in front still writes the partials when this
+// one has been launched (6.9 us at five slots of 8 sequences with either).
+__device__ __forceinline__ float4 ld_partial4(const float* p) {
     float4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "l"(p));
+                 : "l"(p)
+                 : "memory");
     return v;
 }
 
