@@ -762,7 +762,7 @@ def test_c4_long_context_split_sweep(s_q):
 
 
 @pytest.mark.parametrize("rows,S,d_out", [(1, 1, 4), (3, 2, 4), (131, 13, 128), (128, 8, 512), (2050, 5, 128), (300, 20, 512), (37, 70, 24),
-                                          (7, 1100, 16), (300, 40, 4), (8200, 2, 128), (16500, 3, 128)])
+                                          (7, 1100, 16), (300, 40, 4), (8200, 2, 128), (16500, 3, 128), (8200, 20, 24), (5000, 70, 24)])
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 def test_split_merge_over_the_ways_it_is_cut(rows, S, d_out, dtype):
     """Column widths, slot groups and weight staging of the merge change with rows x d_out and the slot count; rows that
