@@ -220,8 +220,8 @@ def test_shape_variants_of_the_paper(h_q, g, s_q):
 def test_paged_cache_gives_what_the_packed_cache_gives(dims, s_q, page_size, S):
     """Paging is storage only (the paper's model leaves it out, Sec. 5.1): both decode calls over a pool of
     shuffled pages must return what they return over the packed cache that holds the same rows -- bit for
-    bit where both runs use the same kernel and the same pieces (tensor-core kernels: pages of a multiple
-    of 128 rows with one split or the balanced plan; generic kernels: any page size) -- and match the oracle
+    bit where both runs use the same kernel and the same pieces (pages of a multiple of 128 rows with one split or
+    the balanced plan; other page sizes run on forms of the kernels that fetch by pages) -- and match the oracle
     fed with the rows gathered back."""
     from tests.parity_util import assert_close, dims_of, round_to
     from oracle import gqla_oracle as O
@@ -252,7 +252,7 @@ def test_paged_cache_gives_what_the_packed_cache_gives(dims, s_q, page_size, S):
     B.gqla_decode_absorb_paged(bd, qh_in, cache_p.cuda(), table_d, page_size, sl, w.scale, S, o_b, l_b, status)
     torch.cuda.synchronize()
     assert int(status.item()) == 0
-    same_kernel = page_size % 128 == 0 and (S == 1 or S < 0)  # else the paged call runs on the generic kernel
+    same_kernel = page_size % 128 == 0 and (S == 1 or S < 0)  # else another form, which fetches by pages
     live = ~torch.isneginf(l_a)  # partial outputs of empty slots are not written under the balanced plan
     if same_kernel:  # same pieces too; otherwise only the merged result is comparable (below)
         assert torch.equal(l_a, l_b) and torch.equal(o_a[live], o_b[live])

@@ -139,3 +139,37 @@ def test_infinite_values_stay_infinite_on_the_gqa_path(h_q, s_q, page, S):
         v[row, :, :3], v[row, :, 3:7] = np.inf, -np.inf
         ref[b, ..., :3], ref[b, ..., 3:7] = np.inf, -np.inf
     assert torch.equal(step(), ref) and int(status.item()) == 0
+
+
+@pytest.mark.parametrize("dims", [CANON, LLAMA, dict(CANON, h_q=64), dict(CANON, h_q=28, g=4), dict(LLAMA, h_q=16)])
+@pytest.mark.parametrize("page,S,s_q,tensor_cores", [
+    (16, 1, 1, True), (16, -9, 2, True), (32, -3, 1, True), (48, 5, 2, True), (64, 1, 2, True), (64, -7, 1, True), (192, -3, 2, True),
+    (128, 3, 1, True), (256, 6, 2, True), (128, -3, 1, True), (64, 2, 3, True), (24, 1, 1, False), (8, -3, 2, False)])
+def test_which_kernels_serve_a_page_size(dims, page, S, s_q, tensor_cores):
+    """The generic kernels give the same bits under either policy; the tensor-core kernels sum in another order and do not.
+    GQA calls over small pages leave the tensor cores beyond 32 padded query rows per group."""
+    seqlens = np.array([700, 129, 333], dtype=np.int32)
+    w = synth.Workload("route", batch=len(seqlens), s_q=s_q, dtype="bf16", seed=311, **dims)
+    x = synth.make_inputs(w, seqlens=seqlens, q_gain=2.0)
+    pool, table = synth.to_paged(x["cache"], x["seq_start"], seqlens, page, seed=312)
+    pool, table, sl = pool.cuda(), table.cuda(), x["seqlens"].cuda()
+    bd = B.make_dims(w.h_q, w.g, w.d_h, w.r_kv, w.d_r)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    q = torch.cat([x["q_c"], x["q_r"]], -1).contiguous().cuda()
+    q_hat = torch.empty((w.batch, s_q, w.h_q, w.d_abs), dtype=torch.bfloat16, device="cuda")
+    k_c, v = (torch.empty((pool.shape[0], w.g, w.d_h), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    B.gqla_absorb_q(bd, x["q_c"].cuda(), x["q_r"].cuda(), x["w_uk"].cuda(), q_hat)
+    B.gqla_expand_cache(bd, pool, x["w_uk"].cuda(), x["w_uv"].cuda(), k_c, v, None)
+    runs = []
+    for policy in (B.POLICY_AUTO, B.POLICY_GENERIC):
+        B.set_policy(policy)
+        try:
+            runs.append((_absorb(bd, w, q_hat, pool, table, page, sl, S, status)[0],
+                         _gqa(bd, w, q, k_c, v, pool[:, w.r_kv:], table, page, sl, S, status)[0]))
+        finally:
+            B.set_policy(B.POLICY_AUTO)
+    assert int(status.item()) == 0
+    rows = (1 << (w.h_q // w.g - 1).bit_length()) * (1 << (s_q - 1).bit_length())
+    small = page % 128 != 0 or S > 1
+    assert torch.equal(runs[0][0], runs[1][0]) == (not tensor_cores)
+    assert torch.equal(runs[0][1], runs[1][1]) == (not tensor_cores or (small and rows > 32))
