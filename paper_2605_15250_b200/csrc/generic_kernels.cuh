@@ -151,10 +151,11 @@ __global__ void __launch_bounds__(128) combine_generic_kernel(int32_t B, int32_t
 // S slots of an item over G thread groups, whose sums meet in shared memory.  The weights of the block's rows are
 // computed once, with a row's slots over adjacent lanes, and staged in shared memory, so the loads of the
 // partials depend on nothing but them: those of 16 / V slots are in flight per thread.
-// What bounds it: the latency of that chain (lse -> weights -> partials) at small row counts, HBM at large ones.  The
-// form it replaces (every thread walked all S slots, one load round trip per slot, 16 columns per thread whatever the
-// size) took 14 us on 128 rows x 128 columns x 13 slots (4 blocks) and 20 us on 512 x 512 x 20; whole steps around
-// such merges went from 22.5 to 16.4 us and from 198 to 175 us.
+// What bounds it: the latency of that chain (lse -> weights -> partials) at small row counts, HBM at large ones.  Back to
+// back with the partials in L2, this form against the one it replaces (every thread walked all S slots, one load round trip
+// per slot, 16 columns per thread whatever the size): 256 rows x 128 columns x 13 slots 3.1 against 8.5 us, 1024 x 512 x 20
+// 6.9 against 17.8, 16384 x 512 x 20 105 against 116; whole steps around such merges went from 22.5 to 16.4 us and from 198
+// to 175 us.
 constexpr int kCombineThreads = 256;
 constexpr int kCombineWeights = 1024;  // staged weights of a block: rows x slots at a time
 __device__ __forceinline__ void store4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }

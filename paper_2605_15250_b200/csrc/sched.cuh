@@ -157,7 +157,8 @@ __host__ __device__ inline BalancedStart balanced_start_serial(const int32_t* se
 #ifdef __CUDACC__
 constexpr int kWarpPlan = 128;  // sequences up to which a warp evaluates the plan alone (four lengths per lane)
 // Cooperative evaluation by all `nthreads` threads of a CTA (a multiple of 32, at most 1024).  `scratch` is
-// shared memory of at least 3 * 32 + 4 int32.  Same result as balanced_start_serial.  Contains __syncthreads.
+// shared memory of at least 3 * 32 + 4 int32.  Same result as balanced_start_serial.  Only batches of more than
+// kWarpPlan sequences meet __syncthreads and touch `scratch`: no caller may count on this as a barrier of the block.
 // Thread t owns the contiguous chunk [t * chunk, (t + 1) * chunk) of the sequences; chunk sums are scanned
 // with warp shuffles and one shared-memory hop across warps.
 __device__ inline BalancedStart balanced_prepass(const int32_t* seqlens, int32_t B, int32_t S, int32_t w, int32_t W,

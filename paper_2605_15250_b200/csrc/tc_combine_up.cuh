@@ -13,7 +13,8 @@
 // rows are dealt to the sixteen builder warps one by one, the weights of all slots are known (eight lanes per row)
 // before the first load, empty slots are passed over, and three live slots of a row are in flight together.
 // Partials from HBM, kernel alone: 4 sequences of 128 heads in four slots 6.2 us (9.0 with one CTA per 64 rows and two rows
-// of a warp at a time), 48 x 2 positions in three slots 21.4 (25.1), 128 sequences of 32 heads 10.1 (11.7).
+// of a warp at a time), 48 x 2 positions in three slots 21.4 (25.1), 128 sequences of 32 heads 10.1 (11.7).  The 18 warps leave
+// 96 registers a thread, into which three slots of a row just fit (16 bytes of spills).
 #pragma once
 #include "tc_common.cuh"
 

@@ -37,8 +37,10 @@
 // them.  The two further P buffers are paid for by a K ring of five single column blocks in place of three groups of three, and
 // the products of the second and third term go to accumulators of their own where tensor memory has room for them (half of O
 // here, all of it in the tokens-on-M kernels): the tensor core truncates its running sums, so every further addition into one of
-// them costs bits (relative to O about 1.7e-8 per 16 rows and term).  What bounds it: the chain P V (3072 cycles a tile) -> P
-// written -> P V; 105 us a step on 32 sequences of 300-8000 rows in pages of 64 rows, 128 heads, where two terms took 88.
+// them costs bits (relative to O about 1.7e-8 per 16 rows and term).  What bounds it: what the MMAs read through shared memory
+// (with the loads 616 KB a tile and CTA; 504 with two terms, 392 in the form above); 105 us a step on 32 sequences of 300-8000
+// rows in pages of 64 rows, 128 heads, where two terms took 88.  Neither an issuer that polls for K groups and P alike nor P
+// written by token halves while P V of the other half runs made it faster (101-110 and 104 us).
 // Errors of the merged partials there, against 64 bits: 3.6e-6 of the 2-norm (two terms 3.8e-6, SIMT kernel 3.4e-7); of the step:
 // 2.79e-3 with each of the three, from the roundings to bf16.  These calls ran one warp per query row on the SIMT kernel before,
 // which read every cache row h_q times from L2: 13.7 ms for 32 sequences of 300-8000 rows in pages of 64 rows.
@@ -133,7 +135,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
     uint64_t* pv_done = p_ready + 2;   // [2]
     uint64_t* xch = pv_done + 2;       // [2] softmax warps of this CTA: per-tile max exchange
     uint64_t* fin = xch + 2;           //     the final partial-sum exchange of a piece
-    uint64_t* epi = fin + 1;           //     and the steps of the output staging
+    uint64_t* epi = fin + 1;           //     and the step of the output staging (whole-sequence form)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + L::kNumBars);
     volatile int32_t* abort_flag = reinterpret_cast<volatile int32_t*>(tmem_slot + 1);
     float* sm_max = reinterpret_cast<float*>(tmem_slot + 4);  // [2][4][64] per-tile partial maxima

@@ -117,7 +117,7 @@ decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUt
     uint64_t* pv_done = p_ready + 2;   // [2]
     uint64_t* xch = pv_done + 2;       // [2] (not used by this kernel: the maxima are exchanged behind a named barrier)
     uint64_t* fin = xch + 2;           //     the final partial-sum exchange of a piece
-    uint64_t* epi = fin + 1;           //     and the steps of the output staging
+    uint64_t* epi = fin + 1;           //     and the step of the output staging (whole-sequence form)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + L::kNumBars);
     volatile int32_t* abort_flag = reinterpret_cast<volatile int32_t*>(tmem_slot + 1);
     float* sm_max = reinterpret_cast<float*>(tmem_slot + 4);  // [2][4][64] per-tile partial maxima

@@ -114,8 +114,8 @@ inline bool absorb_prefers_tokens(const gqla_dims& d, int32_t s_q) {
 // need pages of a multiple of 128 rows and pieces that start on tile boundaries), 64 / 32 / 16 = the small-page form (the
 // largest that divides the page; the fixed plan's pieces start on multiples of 64 rows), -1 = neither, the generic kernels
 // serve the call.  Shuffled pages, 32 sequences of 300-8000 rows, 128 heads, whole step: 14.0 ms with pages of 64 rows on the
-// generic kernels; here 91 us on the absorb path and 119 us on the GQA path (pages of 16 rows: 94 and 150 us; of 128 rows,
-// which keep one bf16 term of a probability: 73 and 109 us).
+// generic kernels; here 105 us on the absorb path and 112 us on the GQA path (pages of 16 rows: 107 and 146 us; of 128 rows,
+// which keep one bf16 term of a probability: 70 us on the absorb path).
 inline int page_box_rows(const RowMap& rows, bool on_tile_boundaries) {
     if (!rows.paged() || (rows.page_size % kTileRows == 0 && on_tile_boundaries)) return 0;
     return rows.page_size % 64 == 0 ? 64 : (rows.page_size % 32 == 0 ? 32 : (rows.page_size % 16 == 0 ? 16 : -1));
@@ -338,7 +338,9 @@ inline gqla_status tc_combine_up_proj(const gqla_dims& d, gqla_dtype dtype, int3
     const int hpg = d.h_q / d.g, hpb = next_pow2(hpg);
     if (!tc_combine_up_covers(d, dtype) || S > tc::CombineUpSmem::kMaxS) return GQLA_ERR_UNSUPPORTED;
     const int64_t positions = (int64_t)B * s_q;
-    // a group's rows in as many runs as there are SMs for a group, at least four rows each (one per builder warp of a quarter)
+    // a group's rows in as many runs as there are SMs for a group, at least four rows each: every CTA fetches all of W^UV[j],
+    // 128 KB, however short its run (steps of one and of two sequences of 777 rows, 128 heads: 23.8 and 24.7 us with four,
+    // 24.6 and 25.1 with one, 24.5 and 24.7 with eight)
     const int64_t group_rows = positions * hpb;
     int64_t runs = sm_count() / d.g > 0 ? sm_count() / d.g : 1;
     if (runs > (group_rows + 3) / 4) runs = (group_rows + 3) / 4;

@@ -8,11 +8,13 @@
 // rows are loaded into it right away: with two 256-column accumulators in TMEM the epilogue warps store tile t while
 // the MMAs of tile t + 1 run, across units too, and the tensor core only waits at the very first unit of a pair.
 // (One pair per 256 rows and launch slot, as this kernel was before, paid set-up, the load of the rows and the last
-// tile's store once per unit: 443 us against 402 us on 224 672 rows, 61 against 48 us on 20 000.)  The output leaves through
+// tile's store once per unit: 452 us against 413 us on 224 672 rows back to back at the power cap, 61 against 48 us on
+// 20 000.)  The output leaves through
 // swizzled shared-memory staging boxes and TMA stores, 64 columns x 32 rows at a time: one thread per row
 // writing its row straight to global memory costs more store instructions than the MMAs give it time for.  Every
 // epilogue warp has a box of its own: with one box of 128 rows the four warps met at two barriers per 64 columns and
-// waited together for its store (224 672 rows: 430 against 428 us, 20 000 rows 49.1 against 48.3).
+// waited together for its store (the two in turn on one GPU: 224 672 rows 430 against 428 us, 20 000 rows 49.1 against 48.3;
+// GPUs differ by more).
 // Warp roles per CTA: warp 0 TMA producer, warp 1 TMEM owner (+ MMA issuer in the leader), warps 2-5
 // epilogue (TMEM lane = row).
 #pragma once

@@ -92,7 +92,9 @@ class GqlaDecoder:
             B.gqla_decode_absorb_paged(self.dims, q_hat, self.cache, self.block_table, self.page_size, self.seqlens,
                                        self.scale, num_splits, o_part, lse_part, self.status)
         # With many slots per sequence the fused tensor-core kernel (a warp walks the slots of a row) falls behind the separate
-        # merge, which spreads them over thread groups: 9.4 against 10.0 us at 11 slots, 10.7 against 9.9 us at 20.  Where the
+        # merge, which spreads them over thread groups: 9.4 against 10.0 us at 11 slots, 10.7 against 9.9 us at 20.  With all twelve
+        # slots live 7.9 against 7.7 us on one sequence of 128 heads, 8.5 against 9.6 on 8, 60.2 against 59.7 on 96, and 21.7
+        # against 20.3 on 128 of 32 heads; most of a ragged batch's slots are empty.  Where the
         # generic fused kernel (a block per row, which reads all of W^UV) would take the place of a tensor-core or faster
         # up-projection, few slots only: 34 against 8.4 us (4 sequences, one group of 128 heads), 69 against 12 (8, 128 heads,
         # r_kv = 1024) and 60 against 49 (32, 64 heads, r_kv = 384) at eight slots.  In fp32 it has no such rival: 32 against 68.
