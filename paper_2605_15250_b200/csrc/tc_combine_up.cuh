@@ -14,7 +14,8 @@
 // before the first load, empty slots are passed over, and three live slots of a row are in flight together.
 // Partials from HBM, kernel alone: 4 sequences of 128 heads in four slots 6.2 us (9.0 with one CTA per 64 rows and two rows
 // of a warp at a time), 48 x 2 positions in three slots 21.4 (25.1), 128 sequences of 32 heads 10.1 (11.7).  The 18 warps leave
-// 96 registers a thread, into which three slots of a row just fit (16 bytes of spills).
+// 96 registers a thread, into which three slots of a row just fit (16 bytes of spills).  Weights and MMAs issued by converged warps
+// (tc_common.cuh): one sequence of 777 rows (eight slots) 7.2 -> 6.5 us, 48 x 2 positions 17.8 -> 16.2, back to back.
 #pragma once
 #include "tc_common.cuh"
 
@@ -74,7 +75,7 @@ combine_up_tc_kernel(const CombineUpParams p, const __grid_constant__ CUtensorMa
     volatile int32_t* abort_flag = reinterpret_cast<volatile int32_t*>(tmem_slot + 1);
     float* sm_w = reinterpret_cast<float*>(tmem_slot + 4);  // [64][kMaxS] normalised weight of every slot of every tile row
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const Abort ab{abort_flag, p.status};
     const int j = blockIdx.y;
     const int64_t row0 = (int64_t)blockIdx.x * p.run, group_rows = p.positions * p.hpb;
@@ -96,40 +97,38 @@ combine_up_tc_kernel(const CombineUpParams p, const __grid_constant__ CUtensorMa
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
     pdl_wait();  // set-up done; the partials come from the previous kernel of the stream
 
     if (warp == 0) {
         // ------------------------------------------------------------------ W^UV chunks (MN-major B operand)
-        if (elect_one()) {
-            tma_prefetch_desc(&tmB);
-            mbar_expect_tx(b_full, n_chunks * L::kBBytes);
-            for (int c = 0; c < n_chunks; ++c)
-                for (int kb = 0; kb < 2; ++kb)
-                    for (int nb = 0; nb < 2; ++nb)
-                        tma_load_2d(b_smem + c * L::kBBytes + (kb * 2 + nb) * 8192, &tmB, nb * 64,
-                                    j * p.r_kv + c * L::kChunkK + kb * 64, b_full);
-        }
+        const uint32_t e = elect_one();
+        if (e) tma_prefetch_desc(&tmB);
+        mbar_expect_tx(b_full, n_chunks * L::kBBytes, e);
+        for (int c = 0; c < n_chunks; ++c)
+            for (int kb = 0; kb < 2; ++kb)
+                for (int nb = 0; nb < 2; ++nb)
+                    tma_load_2d(b_smem + c * L::kBBytes + (kb * 2 + nb) * 8192, &tmB, nb * 64,
+                                j * p.r_kv + c * L::kChunkK + kb * 64, b_full, e);
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (elect_one()) {
-            constexpr uint32_t idesc = idesc_bf16(64, 128, 0, 1);
-            bool ok = mbar_wait(b_full, 0, ab, 2);
-            for (int t = 0; t < n_tiles && ok; ++t) {
-                if (!(ok = mbar_wait(a_ready, t & 1, ab, 3))) break;
-                tc_fence_after();
-                for (int c = 0; c < n_chunks; ++c) {
-                    const uint32_t a_addr = smem_u32(a_smem + c * L::kABytes);
-                    const uint32_t b_addr = smem_u32(b_smem + c * L::kBBytes);
+        const uint32_t e = elect_one();
+        constexpr uint32_t idesc = idesc_bf16(64, 128, 0, 1);
+        bool ok = warp_all(mbar_wait(b_full, 0, ab, 2));
+        for (int t = 0; t < n_tiles && ok; ++t) {
+            if (!(ok = warp_all(mbar_wait(a_ready, t & 1, ab, 3)))) break;
+            tc_fence_after();
+            for (int c = 0; c < n_chunks; ++c) {
+                const uint32_t a_addr = smem_u32(a_smem + c * L::kABytes);
+                const uint32_t b_addr = smem_u32(b_smem + c * L::kBBytes);
 #pragma unroll
-                    for (int kb = 0; kb < 2; ++kb)
+                for (int kb = 0; kb < 2; ++kb)
 #pragma unroll
-                        for (int ks = 0; ks < 4; ++ks)
-                            umma_ss(tmem_base, desc_kmajor_sw128(a_addr + kb * 8192 + ks * 32),
-                                    desc_mnmajor_sw128(b_addr + kb * 16384 + ks * 2048, 8192), idesc, (c | kb | ks) != 0);
-                }
-                umma_commit(acc_full);
+                    for (int ks = 0; ks < 4; ++ks)
+                        umma_ss(tmem_base, desc_kmajor_sw128(a_addr + kb * 8192 + ks * 32),
+                                desc_mnmajor_sw128(b_addr + kb * 16384 + ks * 2048, 8192), idesc, (c | kb | ks) != 0, e);
             }
+            umma_commit(acc_full, e);
         }
     } else {
         // ------------------------------------------------------------------ builders, then epilogue

@@ -16,9 +16,11 @@
 //
 // Staging: two rings per CTA, one of K groups (three 8 KB boxes = 192 columns of 64 rows) and one of
 // V groups (two box pairs = one token half of a tile), each one tile deep, each filled by a producer
-// thread of its own (a thread issues a tensor load only every few hundred cycles, and a tile needs 17);
+// warp of its own;
 // the loads of tile t+1 are in flight while the MMAs of tile t run, and the K loads of the next piece
 // while this piece is stored.
+// The issuer and the producers run converged (tc_common.cuh): 64 x 4096 rows 85.2 -> 82.8 us at the power cap, 48 x 1000-9001
+// rows at s_q = 2 153 -> 147, one of 777 rows 10.3 -> 9.8, small pages (32 x 300-8000 rows, pages of 64) 88.0 -> 83.3.
 // Barriers are per group, not per box: every barrier operation of the issuing threads costs on the
 // order of 100 cycles next to tensor-core operand traffic, and one MMA of this shape is only 32-64
 // cycles of tensor work.
@@ -143,7 +145,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
     // arrived on p_ready of its last tile and hence finished reading sm_max
     float* sm_l = sm_max;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const uint32_t cta = cluster_ctarank();  // 0 = leader
     const Abort ab{abort_flag, p.status};
 
@@ -171,7 +173,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
     __syncthreads();
     cluster_sync();  // both CTAs' barriers exist before any remote arrival
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
     pdl_wait();  // set-up is done (behind the preceding kernel's tail); everything below reads the caller's tensors
     // the plan of this pair: row block rb, and either one (sequence, split) piece or worker w's share
     const int pair = blockIdx.x >> 1;
@@ -224,33 +226,37 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 }
                 ++pi;
             }
-        } else if (elect_one()) {
+        } else {
+            const uint32_t e = elect_one();
             const uint32_t q_full_l = mapa(smem_u32(q_full), 0);
             int ks = 0;
             uint32_t kph = 1;  // parity that means "slot is free"
             bool ok = true;
-            while (ok && walk.next(pc)) {
-                if (pc.n_tiles == 0) continue;
+            while (ok && warp_all(walk.next(pc))) {
+                const int n_tiles = warp_uniform(pc.n_tiles);
+                if (n_tiles == 0) continue;
                 // Q rows of this piece's sequence; the previous piece's Qh Kh^T must all have completed
-                if (pi > 0 && !(ok = mbar_wait(q_empty, (pi - 1) & 1, ab, 13))) break;
-                if (cta == 0) mbar_expect_tx(q_full, 2 * L::kQBytes);
+                if (pi > 0 && !(ok = warp_all(mbar_wait(q_empty, (pi - 1) & 1, ab, 13)))) break;
+                if (cta == 0) mbar_expect_tx(q_full, 2 * L::kQBytes, e);
+                const int32_t q_row = warp_uniform(pc.b * p.rows_total + rho0);
+#pragma unroll
                 for (int kb = 0; kb < 9; ++kb)
-                    tma_load_2d_pair(tiles + kb * L::kBox, &tmQ, kb * 64, pc.b * p.rows_total + rho0, q_full_l);
+                    tma_load_2d_pair(tiles + kb * L::kBox, &tmQ, kb * 64, q_row, q_full_l, e);
                 // K groups in the order (tile, column third); a tile never straddles a page
                 int64_t tile_row = p.rows.row(pc.b, pc.tok_begin);
-                for (int kt = 0; kt < pc.n_tiles && ok; ++kt) {
-                    const int32_t row = (int32_t)(tile_row + cta * 64);
+                for (int kt = 0; kt < n_tiles && ok; ++kt) {
+                    const int32_t row = warp_uniform((int32_t)(tile_row + cta * 64));
                     // the next tile's row is fetched while this tile's slots are waited for
-                    if (kt + 1 < pc.n_tiles)
+                    if (kt + 1 < n_tiles)
                         tile_row = p.rows.paged() ? p.rows.row(pc.b, pc.tok_begin + (kt + 1) * 128) : tile_row + 128;
 #pragma unroll 1
                     for (int kg = 0; kg < 3; ++kg) {
-                        if (!(ok = mbar_wait(&kempty[ks], kph, ab, 1))) break;
-                        if (cta == 0) mbar_expect_tx(&kfull[ks], 2 * L::kKGroup);
+                        if (!(ok = warp_all(mbar_wait(&kempty[ks], kph, ab, 1)))) break;
+                        if (cta == 0) mbar_expect_tx(&kfull[ks], 2 * L::kKGroup, e);
                         const uint32_t bar = mapa(smem_u32(&kfull[ks]), 0);
                         uint8_t* dst = tiles + L::kOffK + ks * L::kKGroup;
 #pragma unroll
-                        for (int i = 0; i < 3; ++i) tma_load_2d_pair(dst + i * L::kBox, &tmC, (3 * kg + i) * 64, row, bar);
+                        for (int i = 0; i < 3; ++i) tma_load_2d_pair(dst + i * L::kBox, &tmC, (3 * kg + i) * 64, row, bar, e);
                         if (++ks == L::kNK) { ks = 0; kph ^= 1; }
                     }
                 }
@@ -259,8 +265,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
         }
     } else if (warp == L::kVProducerWarp) {
         // ------------------------------------------------------------------ TMA producer of the V ring (both
-        // CTAs).  A thread issues a tensor load only every few hundred cycles, and a tile needs 17 of them:
-        // the two rings are fed by two threads.  V groups in the order (tile, token half); a V slot is free
+        // CTAs): the two rings fill independently of one another.  V groups in the order (tile, token half); a V slot is free
         // only after P.V of the previous tile, i.e. after Qh Kh^T of this tile has read the same cache rows
         // as K boxes, so the V boxes come out of L2.
         if constexpr (PG != 0) {
@@ -298,31 +303,33 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 }
                 ++pi;
             }
-        } else if (elect_one()) {
+        } else {
+            const uint32_t e = elect_one();
             int vs = 0;
             uint32_t vph = 1;
             bool ok = true;
-            while (ok && walk.next(pc)) {
-                if (pc.n_tiles == 0) continue;
+            while (ok && warp_all(walk.next(pc))) {
+                const int n_tiles = warp_uniform(pc.n_tiles);
+                if (n_tiles == 0) continue;
                 // the V ring doubles as the output staging of the previous piece
-                if (pi > 0 && !(ok = mbar_wait(epi_done, (pi - 1) & 1, ab, 16))) break;
+                if (pi > 0 && !(ok = warp_all(mbar_wait(epi_done, (pi - 1) & 1, ab, 16)))) break;
                 int64_t tile_row = p.rows.row(pc.b, pc.tok_begin);
-                for (int vt = 0; vt < pc.n_tiles && ok; ++vt) {
+                for (int vt = 0; vt < n_tiles && ok; ++vt) {
                     const int64_t row0 = tile_row;
-                    if (vt + 1 < pc.n_tiles)
+                    if (vt + 1 < n_tiles)
                         tile_row = p.rows.paged() ? p.rows.row(pc.b, pc.tok_begin + (vt + 1) * 128) : tile_row + 128;
 #pragma unroll 1
                     for (int vh = 0; vh < 2; ++vh) {
-                        if (!(ok = mbar_wait(&vempty[vs], vph, ab, 2))) break;
-                        if (cta == 0) mbar_expect_tx(&vfull[vs], 2 * L::kVGroup);
-                        const int32_t row = (int32_t)(row0 + vh * 64);
+                        if (!(ok = warp_all(mbar_wait(&vempty[vs], vph, ab, 2)))) break;
+                        if (cta == 0) mbar_expect_tx(&vfull[vs], 2 * L::kVGroup, e);
+                        const int32_t row = warp_uniform((int32_t)(row0 + vh * 64));
                         const uint32_t bar = mapa(smem_u32(&vfull[vs]), 0);
                         uint8_t* dst = tiles + L::kOffV + vs * L::kVGroup;
                         // box (m, i): latent columns [256m + 128cta + 64i, +64) -- this CTA's half of MMA m's N
 #pragma unroll
                         for (int mi = 0; mi < 4; ++mi)
                             tma_load_2d_pair(dst + mi * L::kBox, &tmC, 256 * (mi >> 1) + 128 * (int)cta + 64 * (mi & 1), row,
-                                             bar);
+                                             bar, e);
                         if (++vs == L::kNV) { vs = 0; vph ^= 1; }
                     }
                 }
@@ -331,7 +338,8 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leader CTA only)
-        if (cta == 0 && elect_one()) {
+        if (cta == 0) {
+            const uint32_t e = elect_one();
             constexpr uint32_t idesc_qk = idesc_bf16(128, 128, 0, 0);
             constexpr uint32_t idesc_pv = idesc_bf16(128, 256, 0, 1);
             const uint64_t q_desc = desc_kmajor_sw128(smem_u32(tiles));
@@ -343,48 +351,49 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 const uint32_t d = tmem_base + kAColS + (uint32_t)(n & 1) * 64;
 #pragma unroll 1
                 for (int g = 0; g < 9 / L::kKBlocks; ++g) {
-                    if (!mbar_wait_fast(&kfull[ks], kph, ab, 3)) return false;
+                    if (!warp_all(mbar_wait_fast(&kfull[ks], kph, ab, 3))) return false;
                     tc_fence_after();
                     // descriptors as low words: the high word is a constant, stepping is one 32-bit add
                     const uint32_t kd = desc_lo(desc_kmajor_sw128(smem_u32(tiles + L::kOffK + ks * L::kKGroup)));
                     const uint32_t qd = desc_lo(q_desc) + ((g * L::kKBlocks * L::kBox) >> 4);
                     if (g == 0)
-                        umma_ss2_lo<false>(d, qd, kd, idesc_qk);  // the tile's first MMA overwrites S
+                        umma_ss2_lo<false>(d, qd, kd, idesc_qk, e);  // the tile's first MMA overwrites S
                     else
-                        umma_ss2_lo<true>(d, qd, kd, idesc_qk);
+                        umma_ss2_lo<true>(d, qd, kd, idesc_qk, e);
 #pragma unroll
                     for (int i = 0; i < L::kKBlocks; ++i)
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk)
                             if ((i | kk) != 0)
                                 umma_ss2_lo<true>(d, qd + ((i * L::kBox + kk * 32) >> 4), kd + ((i * L::kBox + kk * 32) >> 4),
-                                                  idesc_qk);
-                    umma_commit2(&kempty[ks], 3);
+                                                  idesc_qk, e);
+                    umma_commit2(&kempty[ks], 3, e);
                     if (++ks == L::kNK) { ks = 0; kph ^= 1; }
                 }
-                umma_commit2(&s_full[n & 1], 3);
+                umma_commit2(&s_full[n & 1], 3, e);
                 return true;
             };
             bool ok = true;
-            while (ok && walk.next(pc)) {
-                if (pc.n_tiles == 0) continue;
-                if (!(ok = mbar_wait(q_full, pi & 1, ab, 4))) break;
+            while (ok && warp_all(walk.next(pc))) {
+                const int n_tiles = warp_uniform(pc.n_tiles);
+                if (n_tiles == 0) continue;
+                if (!(ok = warp_all(mbar_wait(q_full, pi & 1, ab, 4)))) break;
                 tc_fence_after();
                 if (!(ok = issue_qk(gt))) break;
-                for (int t = 0; t < pc.n_tiles && ok; ++t) {
+                for (int t = 0; t < n_tiles && ok; ++t) {
                     const int n = gt + t;
-                    if (t + 1 < pc.n_tiles) {
+                    if (t + 1 < n_tiles) {
                         if (!(ok = issue_qk(n + 1))) break;
                     } else {
-                        umma_commit2(q_empty, 3);  // every Qh Kh^T of this piece has been issued
+                        umma_commit2(q_empty, 3, e);  // every Qh Kh^T of this piece has been issued
                     }
-                    if (!(ok = mbar_wait_fast(&p_ready[n & 1], (n >> 1) & 1, ab, 5))) break;
+                    if (!(ok = warp_all(mbar_wait_fast(&p_ready[n & 1], (n >> 1) & 1, ab, 5)))) break;
                     // the first P.V of a piece overwrites O: the previous piece's O must have been read
-                    if (t == 0 && pi > 0 && !(ok = mbar_wait(o_free, (pi - 1) & 1, ab, 14))) break;
+                    if (t == 0 && pi > 0 && !(ok = warp_all(mbar_wait(o_free, (pi - 1) & 1, ab, 14)))) break;
                     tc_fence_after();
 #pragma unroll 1
                     for (int h = 0; h < 2; ++h) {
-                        if (!(ok = mbar_wait_fast(&vfull[vs], vph, ab, 6))) break;
+                        if (!(ok = warp_all(mbar_wait_fast(&vfull[vs], vph, ab, 6)))) break;
                         tc_fence_after();
                         const uint32_t vd = desc_lo(desc_mnmajor_sw128(smem_u32(tiles + L::kOffV + vs * L::kVGroup), L::kBox));
                         const uint32_t pd = desc_lo(p_desc) + ((h * L::kBox) >> 4);
@@ -392,29 +401,29 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                         for (int m = 0; m < 2; ++m) {
                             const uint32_t dm = tmem_base + kAColO + (uint32_t)m * 128;
                             if ((t | h) == 0)
-                                umma_ss2_lo<false>(dm, pd, vd + ((m * 2 * L::kBox) >> 4), idesc_pv);  // first P.V of a piece
+                                umma_ss2_lo<false>(dm, pd, vd + ((m * 2 * L::kBox) >> 4), idesc_pv, e);  // first P.V of a piece
                             else
-                                umma_ss2_lo<true>(dm, pd, vd + ((m * 2 * L::kBox) >> 4), idesc_pv);
+                                umma_ss2_lo<true>(dm, pd, vd + ((m * 2 * L::kBox) >> 4), idesc_pv, e);
 #pragma unroll
                             for (int kk = 1; kk < 4; ++kk)
-                                umma_ss2_lo<true>(dm, pd + ((kk * 32) >> 4), vd + ((m * 2 * L::kBox + kk * 2048) >> 4), idesc_pv);
+                                umma_ss2_lo<true>(dm, pd + ((kk * 32) >> 4), vd + ((m * 2 * L::kBox + kk * 2048) >> 4), idesc_pv, e);
 #pragma unroll
                             for (int kk = 4; kk < 4 * L::kPTerms; ++kk) {  // the other terms of P
                                 const uint32_t d = m == 0 ? tmem_base + kAColRest : dm;
                                 const uint32_t a = pd + (((kk >> 2) * L::kPTerm + (kk & 3) * 32) >> 4);
                                 const uint32_t b = vd + ((m * 2 * L::kBox + (kk & 3) * 2048) >> 4);
                                 if (m == 0 && kk == 4 && (t | h) == 0)
-                                    umma_ss2_lo<false>(d, a, b, idesc_pv);
+                                    umma_ss2_lo<false>(d, a, b, idesc_pv, e);
                                 else
-                                    umma_ss2_lo<true>(d, a, b, idesc_pv);
+                                    umma_ss2_lo<true>(d, a, b, idesc_pv, e);
                             }
                         }
-                        umma_commit2(&vempty[vs], 3);
+                        umma_commit2(&vempty[vs], 3, e);
                         if (++vs == L::kNV) { vs = 0; vph ^= 1; }
                     }
-                    if (ok) umma_commit2(&pv_done[n & 1], 3);
+                    if (ok) umma_commit2(&pv_done[n & 1], 3, e);
                 }
-                gt += pc.n_tiles;
+                gt += n_tiles;
                 ++pi;
             }
         }

@@ -18,6 +18,7 @@
 //     the choice of the two constants above), and barriers that have usually completed are probed before a suspending
 //     wait.  The exchange of every tile's maxima and a reference that followed the maximum within one binade (O
 //     rescaled on 40 % of the tiles) cost a quarter of the kernel.
+//   * Issuer and producers run converged (tc_common.cuh): 64 x 4096 rows 53.0 -> 51.9 us at the power cap, 46.2 -> 44.9 in a burst.
 #pragma once
 #include "common.cuh"
 #include "sched.cuh"
@@ -80,12 +81,13 @@ constexpr float kAF8Grow = 8.75f;  // a score this far above its row's reference
 constexpr uint32_t kDescHiSw64 = (uint32_t)(((1ull << 46) | (4ull << 61) | ((uint64_t)(512 >> 4) << 32)) >> 32);
 // cta_group::2 MMA of kind::f8f6f4; descriptors as (low word, constant high word of their swizzle mode).
 template <bool ACCUMULATE>
-__device__ __forceinline__ void umma_f8_ss2_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t hi) {
+__device__ __forceinline__ void umma_f8_ss2_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t hi,
+                                               uint32_t on = 1) {
     asm volatile(
-        "{\n\t.reg .b64 da, db;\n\t.reg .pred p;\n\t"
-        "mov.b64 da, {%1, %4};\n\tmov.b64 db, {%2, %4};\n\tsetp.ne.b32 p, %5, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(hi), "n"(ACCUMULATE ? 1 : 0)
+        "{\n\t.reg .b64 da, db;\n\t.reg .pred p, e;\n\t"
+        "mov.b64 da, {%1, %4};\n\tmov.b64 db, {%2, %4};\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 e, %6, 0;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(hi), "n"(ACCUMULATE ? 1 : 0), "r"(on)
         : "memory");
 }
 
@@ -125,7 +127,7 @@ decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUt
     // arrived on p_ready of its last tile and hence finished reading sm_max
     float* sm_l = sm_max;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const uint32_t cta = cluster_ctarank();  // 0 = leader
     const Abort ab{abort_flag, p.status};
 
@@ -155,7 +157,7 @@ decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUt
     __syncthreads();
     cluster_sync();  // both CTAs' barriers exist before any remote arrival
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
     pdl_wait();  // set-up is done (behind the preceding kernel's tail); everything below reads the caller's tensors
     // the plan of this pair: row block rb, and either one (sequence, split) piece or worker w's share
     const int pair = blockIdx.x >> 1;
@@ -176,80 +178,82 @@ decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUt
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer of Q and the K ring
         // (both CTAs).  Every "full" barrier lives in the leader and counts the bytes of BOTH CTAs.
-        if (elect_one()) {
-            const uint32_t q_full_l = mapa(smem_u32(q_full), 0);
-            int ks = 0;
-            uint32_t kph = 1;  // parity that means "slot is free"
-            bool ok = true;
-            while (ok && walk.next(pc)) {
-                if (pc.n_tiles == 0) continue;
-                // Q rows of this piece's sequence; the previous piece's Qh Kh^T must all have completed
-                if (pi > 0 && !(ok = mbar_wait(q_empty, (pi - 1) & 1, ab, 13))) break;
-                if (cta == 0) mbar_expect_tx(q_full, 2 * L::kQBytes);
-                for (int kb = 0; kb < 4; ++kb)
-                    tma_load_2d_pair(tiles + kb * L::kBox, &tmQ, kb * 128, pc.b * p.rows_total + rho0, q_full_l);
-                tma_load_2d_pair(tiles + 4 * L::kBox, &tmQr, 512, pc.b * p.rows_total + rho0, q_full_l);
-                // K groups in the order (tile, column half); a tile never straddles a page
-                int64_t tile_row = p.rows.row(pc.b, pc.tok_begin);
-                for (int kt = 0; kt < pc.n_tiles && ok; ++kt) {
-                    const int32_t row = (int32_t)(tile_row + cta * 64);
-                    // the next tile's row is fetched while this tile's slots are waited for
-                    if (kt + 1 < pc.n_tiles)
-                        tile_row = p.rows.paged() ? p.rows.row(pc.b, pc.tok_begin + (kt + 1) * 128) : tile_row + 128;
-#pragma unroll 1
-                    for (int kg = 0; kg < 2; ++kg) {
-                        if (!(ok = mbar_wait(&kempty[ks], kph, ab, 1))) break;
-                        // group 0: latent boxes 0, 1;  group 1: latent boxes 2, 3 and the RoPE box
-                        if (cta == 0) mbar_expect_tx(&kfull[ks], 2 * (2 * L::kBox + (kg == 1 ? L::kRBox : 0)));
-                        const uint32_t bar = mapa(smem_u32(&kfull[ks]), 0);
-                        uint8_t* dst = tiles + L::kOffK + ks * L::kKGroup;
+        const uint32_t e = elect_one();
+        const uint32_t q_full_l = mapa(smem_u32(q_full), 0);
+        int ks = 0;
+        uint32_t kph = 1;  // parity that means "slot is free"
+        bool ok = true;
+        while (ok && warp_all(walk.next(pc))) {
+            const int n_tiles = warp_uniform(pc.n_tiles);
+            if (n_tiles == 0) continue;
+            // Q rows of this piece's sequence; the previous piece's Qh Kh^T must all have completed
+            if (pi > 0 && !(ok = warp_all(mbar_wait(q_empty, (pi - 1) & 1, ab, 13)))) break;
+            if (cta == 0) mbar_expect_tx(q_full, 2 * L::kQBytes, e);
+            const int32_t q_row = warp_uniform(pc.b * p.rows_total + rho0);
 #pragma unroll
-                        for (int i = 0; i < 2; ++i) tma_load_2d_pair(dst + i * L::kBox, &tmC, (2 * kg + i) * 128, row, bar);
-                        if (kg == 1) tma_load_2d_pair(dst + 2 * L::kBox, &tmCr, 512, row, bar);
-                        if (++ks == L::kNK) { ks = 0; kph ^= 1; }
-                    }
+            for (int kb = 0; kb < 4; ++kb)
+                tma_load_2d_pair(tiles + kb * L::kBox, &tmQ, kb * 128, q_row, q_full_l, e);
+            tma_load_2d_pair(tiles + 4 * L::kBox, &tmQr, 512, q_row, q_full_l, e);
+            // K groups in the order (tile, column half); a tile never straddles a page
+            int64_t tile_row = p.rows.row(pc.b, pc.tok_begin);
+            for (int kt = 0; kt < n_tiles && ok; ++kt) {
+                const int32_t row = warp_uniform((int32_t)(tile_row + cta * 64));
+                // the next tile's row is fetched while this tile's slots are waited for
+                if (kt + 1 < n_tiles)
+                    tile_row = p.rows.paged() ? p.rows.row(pc.b, pc.tok_begin + (kt + 1) * 128) : tile_row + 128;
+#pragma unroll 1
+                for (int kg = 0; kg < 2; ++kg) {
+                    if (!(ok = warp_all(mbar_wait(&kempty[ks], kph, ab, 1)))) break;
+                    // group 0: latent boxes 0, 1;  group 1: latent boxes 2, 3 and the RoPE box
+                    if (cta == 0) mbar_expect_tx(&kfull[ks], 2 * (2 * L::kBox + (kg == 1 ? L::kRBox : 0)), e);
+                    const uint32_t bar = mapa(smem_u32(&kfull[ks]), 0);
+                    uint8_t* dst = tiles + L::kOffK + ks * L::kKGroup;
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) tma_load_2d_pair(dst + i * L::kBox, &tmC, (2 * kg + i) * 128, row, bar, e);
+                    if (kg == 1) tma_load_2d_pair(dst + 2 * L::kBox, &tmCr, 512, row, bar, e);
+                    if (++ks == L::kNK) { ks = 0; kph ^= 1; }
                 }
-                ++pi;
             }
+            ++pi;
         }
     } else if (warp == L::kVProducerWarp) {
         // ------------------------------------------------------------------ TMA producer of the V ring (both
-        // CTAs).  A thread issues a tensor load only every few hundred cycles, and a tile needs 17 of them:
-        // the two rings are fed by two threads.  V groups in the order (tile, token half); a V slot is free
+        // CTAs): the two rings fill independently of one another.  V groups in the order (tile, token half); a V slot is free
         // only after P.V of the previous tile, i.e. after Qh Kh^T of this tile has read the same cache rows
         // as K boxes, so the V boxes come out of L2.
-        if (elect_one()) {
-            int vs = 0;
-            uint32_t vph = 1;
-            bool ok = true;
-            while (ok && walk.next(pc)) {
-                if (pc.n_tiles == 0) continue;
-                // the V ring doubles as the output staging of the previous piece
-                if (pi > 0 && !(ok = mbar_wait(epi_done, (pi - 1) & 1, ab, 16))) break;
-                int64_t tile_row = p.rows.row(pc.b, pc.tok_begin);
-                for (int vt = 0; vt < pc.n_tiles && ok; ++vt) {
-                    const int64_t row0 = tile_row;
-                    if (vt + 1 < pc.n_tiles)
-                        tile_row = p.rows.paged() ? p.rows.row(pc.b, pc.tok_begin + (vt + 1) * 128) : tile_row + 128;
+        const uint32_t e = elect_one();
+        int vs = 0;
+        uint32_t vph = 1;
+        bool ok = true;
+        while (ok && warp_all(walk.next(pc))) {
+            const int n_tiles = warp_uniform(pc.n_tiles);
+            if (n_tiles == 0) continue;
+            // the V ring doubles as the output staging of the previous piece
+            if (pi > 0 && !(ok = warp_all(mbar_wait(epi_done, (pi - 1) & 1, ab, 16)))) break;
+            int64_t tile_row = p.rows.row(pc.b, pc.tok_begin);
+            for (int vt = 0; vt < n_tiles && ok; ++vt) {
+                const int64_t row0 = tile_row;
+                if (vt + 1 < n_tiles)
+                    tile_row = p.rows.paged() ? p.rows.row(pc.b, pc.tok_begin + (vt + 1) * 128) : tile_row + 128;
 #pragma unroll 1
-                    for (int vh = 0; vh < 2; ++vh) {
-                        if (!(ok = mbar_wait(&vempty[vs], vph, ab, 2))) break;
-                        if (cta == 0) mbar_expect_tx(&vfull[vs], 2 * L::kVGroup);
-                        const int32_t row = (int32_t)(row0 + vh * 64);
-                        const uint32_t bar = mapa(smem_u32(&vfull[vs]), 0);
-                        uint8_t* dst = tiles + L::kOffV + vs * L::kVGroup;
-                        // box m: latent columns [256m + 128cta, +128) -- this CTA's half of MMA m's N
+                for (int vh = 0; vh < 2; ++vh) {
+                    if (!(ok = warp_all(mbar_wait(&vempty[vs], vph, ab, 2)))) break;
+                    if (cta == 0) mbar_expect_tx(&vfull[vs], 2 * L::kVGroup, e);
+                    const int32_t row = warp_uniform((int32_t)(row0 + vh * 64));
+                    const uint32_t bar = mapa(smem_u32(&vfull[vs]), 0);
+                    uint8_t* dst = tiles + L::kOffV + vs * L::kVGroup;
+                    // box m: latent columns [256m + 128cta, +128) -- this CTA's half of MMA m's N
 #pragma unroll
-                        for (int m = 0; m < 2; ++m) tma_load_2d_pair(dst + m * L::kBox, &tmC, 256 * m + 128 * (int)cta, row, bar);
-                        if (++vs == L::kNV) { vs = 0; vph ^= 1; }
-                    }
+                    for (int m = 0; m < 2; ++m) tma_load_2d_pair(dst + m * L::kBox, &tmC, 256 * m + 128 * (int)cta, row, bar, e);
+                    if (++vs == L::kNV) { vs = 0; vph ^= 1; }
                 }
-                ++pi;
             }
+            ++pi;
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leader CTA only)
-        if (cta == 0 && elect_one()) {
+        if (cta == 0) {
+            const uint32_t e = elect_one();
             constexpr uint32_t idesc_qk = idesc_e4m3(128, 128, 0, 0);
             constexpr uint32_t idesc_pv = idesc_e4m3(128, 256, 0, 1);
             const uint32_t q_lo = desc_lo(desc_kmajor_sw128(smem_u32(tiles)));
@@ -262,53 +266,54 @@ decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUt
                 const uint32_t d = tmem_base + kA8ColS + (uint32_t)(n & 1) * 64;
 #pragma unroll 1
                 for (int g2 = 0; g2 < 2; ++g2) {
-                    if (!mbar_wait(&kfull[ks], kph, ab, 3)) return false;
+                    if (!warp_all(mbar_wait(&kfull[ks], kph, ab, 3))) return false;
                     tc_fence_after();
                     const uint32_t kd = desc_lo(desc_kmajor_sw128(smem_u32(tiles + L::kOffK + ks * L::kKGroup)));
                     const uint32_t qd = q_lo + ((g2 * 2 * L::kBox) >> 4);
                     if (g2 == 0)
-                        umma_f8_ss2_lo<false>(d, qd, kd, idesc_qk, kDescHiSw128);  // the tile's first MMA overwrites S
+                        umma_f8_ss2_lo<false>(d, qd, kd, idesc_qk, kDescHiSw128, e);  // the tile's first MMA overwrites S
                     else
-                        umma_f8_ss2_lo<true>(d, qd, kd, idesc_qk, kDescHiSw128);
+                        umma_f8_ss2_lo<true>(d, qd, kd, idesc_qk, kDescHiSw128, e);
 #pragma unroll
                     for (int i = 0; i < 2; ++i)
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk)
                             if ((i | kk) != 0)
                                 umma_f8_ss2_lo<true>(d, qd + ((i * L::kBox + kk * 32) >> 4), kd + ((i * L::kBox + kk * 32) >> 4),
-                                                     idesc_qk, kDescHiSw128);
+                                                     idesc_qk, kDescHiSw128, e);
                     if (g2 == 1) {  // the RoPE part: 64 elements = 2 x 32, 64-byte swizzle
                         const uint32_t krd = desc_lo(desc_kmajor_sw64(smem_u32(tiles + L::kOffK + ks * L::kKGroup + 2 * L::kBox)));
 #pragma unroll
                         for (int kk = 0; kk < 2; ++kk)
-                            umma_f8_ss2_lo<true>(d, qr_lo + ((kk * 32) >> 4), krd + ((kk * 32) >> 4), idesc_qk, kDescHiSw64);
+                            umma_f8_ss2_lo<true>(d, qr_lo + ((kk * 32) >> 4), krd + ((kk * 32) >> 4), idesc_qk, kDescHiSw64, e);
                     }
-                    umma_commit2(&kempty[ks], 3);
+                    umma_commit2(&kempty[ks], 3, e);
                     if (++ks == L::kNK) { ks = 0; kph ^= 1; }
                 }
-                umma_commit2(&s_full[n & 1], 3);
+                umma_commit2(&s_full[n & 1], 3, e);
                 return true;
             };
             bool ok = true;
-            while (ok && walk.next(pc)) {
-                if (pc.n_tiles == 0) continue;
-                if (!(ok = mbar_wait(q_full, pi & 1, ab, 4))) break;
+            while (ok && warp_all(walk.next(pc))) {
+                const int n_tiles = warp_uniform(pc.n_tiles);
+                if (n_tiles == 0) continue;
+                if (!(ok = warp_all(mbar_wait(q_full, pi & 1, ab, 4)))) break;
                 tc_fence_after();
                 if (!(ok = issue_qk(gt))) break;
-                for (int t = 0; t < pc.n_tiles && ok; ++t) {
+                for (int t = 0; t < n_tiles && ok; ++t) {
                     const int n = gt + t;
-                    if (t + 1 < pc.n_tiles) {
+                    if (t + 1 < n_tiles) {
                         if (!(ok = issue_qk(n + 1))) break;
                     } else {
-                        umma_commit2(q_empty, 3);  // every Qh Kh^T of this piece has been issued
+                        umma_commit2(q_empty, 3, e);  // every Qh Kh^T of this piece has been issued
                     }
-                    if (!(ok = mbar_wait(&p_ready[n & 1], (n >> 1) & 1, ab, 5))) break;
+                    if (!(ok = warp_all(mbar_wait(&p_ready[n & 1], (n >> 1) & 1, ab, 5)))) break;
                     // the first P.V of a piece overwrites O: the previous piece's O must have been read
-                    if (t == 0 && pi > 0 && !(ok = mbar_wait(o_free, (pi - 1) & 1, ab, 14))) break;
+                    if (t == 0 && pi > 0 && !(ok = warp_all(mbar_wait(o_free, (pi - 1) & 1, ab, 14)))) break;
                     tc_fence_after();
 #pragma unroll 1
                     for (int h = 0; h < 2; ++h) {
-                        if (!(ok = mbar_wait(&vfull[vs], vph, ab, 6))) break;
+                        if (!(ok = warp_all(mbar_wait(&vfull[vs], vph, ab, 6)))) break;
                         tc_fence_after();
                         // V box m: [64 tokens x 128 latent columns], MN-major; a k-step is 32 token rows (4 KB)
                         const uint32_t vd = desc_lo(desc_mnmajor_sw128(smem_u32(tiles + L::kOffV + vs * L::kVGroup), L::kBox));
@@ -317,17 +322,17 @@ decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUt
                         for (int m = 0; m < 2; ++m) {
                             const uint32_t dm = tmem_base + kA8ColO + (uint32_t)m * 128;
                             if ((t | h) == 0)
-                                umma_f8_ss2_lo<false>(dm, pd, vd + ((m * L::kBox) >> 4), idesc_pv, kDescHiSw128);  // first P.V of a piece
+                                umma_f8_ss2_lo<false>(dm, pd, vd + ((m * L::kBox) >> 4), idesc_pv, kDescHiSw128, e);  // first P.V of a piece
                             else
-                                umma_f8_ss2_lo<true>(dm, pd, vd + ((m * L::kBox) >> 4), idesc_pv, kDescHiSw128);
-                            umma_f8_ss2_lo<true>(dm, pd + (32 >> 4), vd + ((m * L::kBox + 4096) >> 4), idesc_pv, kDescHiSw128);
+                                umma_f8_ss2_lo<true>(dm, pd, vd + ((m * L::kBox) >> 4), idesc_pv, kDescHiSw128, e);
+                            umma_f8_ss2_lo<true>(dm, pd + (32 >> 4), vd + ((m * L::kBox + 4096) >> 4), idesc_pv, kDescHiSw128, e);
                         }
-                        umma_commit2(&vempty[vs], 3);
+                        umma_commit2(&vempty[vs], 3, e);
                         if (++vs == L::kNV) { vs = 0; vph ^= 1; }
                     }
-                    if (ok) umma_commit2(&pv_done[n & 1], 3);
+                    if (ok) umma_commit2(&pv_done[n & 1], 3, e);
                 }
-                gt += pc.n_tiles;
+                gt += n_tiles;
                 ++pi;
             }
         }

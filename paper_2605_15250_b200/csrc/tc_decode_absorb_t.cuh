@@ -25,7 +25,8 @@
 // sequences of 8-32 K tokens, balanced plan, one GPU): 437 us in a burst against 541 us for the pair kernel; launched
 // back to back for seconds under the power cap, a quarter of the tensor work leaves the clocks at 1.70 GHz where the pair
 // kernel's drop to 1.21 GHz: 505 us against 633 us per launch.  With 64 rows (sixteen per softmax warp, one P^T buffer):
-// 502 against 554 us in a burst.
+// 502 against 554 us in a burst.  Issuer and producer converged (tc_common.cuh): 388.6 -> 385.4 us in a burst on 128 sequences of
+// 512-32768 rows, 450 -> 448 at the power cap.
 #pragma once
 #include "common.cuh"
 #include "sched.cuh"
@@ -112,7 +113,7 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
     constexpr uint32_t kColS = 0, kColO = 2 * R, kColsUsed = (2 + 4 * L::kAcc) * R;
     constexpr uint32_t kTmemCols = kColsUsed <= 128 ? 128 : (kColsUsed <= 256 ? 256 : 512);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const Abort ab{abort_flag, p.status};
 
     if (threadIdx.x == 0) {
@@ -133,7 +134,7 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
     pdl_wait();  // set-up is done (behind the preceding kernel's tail); everything below reads the caller's tensors
     const int unit = blockIdx.x;
     Walker walk;
@@ -193,35 +194,39 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                 }
                 ++pi;
             }
-        } else if (elect_one()) {
+        } else {
+            const uint32_t e = elect_one();
             bool ok = true;
-            while (ok && walk.next(pc)) {
-                if (pc.n_tiles == 0) continue;
-                const int nt = (pc.tok_end - pc.tok_begin + TK - 1) / TK;
-                if (pi > 0 && !(ok = mbar_wait(q_empty, (pi - 1) & 1, ab, 13))) break;
-                mbar_expect_tx(q_full, L::kQBytes);
+            while (ok && warp_all(walk.next(pc))) {
+                const int n_tiles = warp_uniform(pc.n_tiles);
+                if (n_tiles == 0) continue;
+                const int nt = warp_uniform((pc.tok_end - pc.tok_begin + TK - 1) / TK);
+                if (pi > 0 && !(ok = warp_all(mbar_wait(q_empty, (pi - 1) & 1, ab, 13)))) break;
+                mbar_expect_tx(q_full, L::kQBytes, e);
+                const int32_t q_row = warp_uniform(pc.b * p.rows_total);
+#pragma unroll
                 for (int kb = 0; kb < 9; ++kb)
-                    tma_load_2d(q_smem + kb * L::kQBlock, &tmQ, kb * 64, pc.b * p.rows_total, q_full);
+                    tma_load_2d(q_smem + kb * L::kQBlock, &tmQ, kb * 64, q_row, q_full, e);
                 for (int t = 0; t < nt; ++t, ++gt) {
                     const int s = gt & 1;
                     uint8_t* st = stage0 + s * L::kStageBytes;
                     // a page holds a multiple of 128 rows and pieces start on multiples of 64: no tile straddles pages
-                    const int32_t row = (int32_t)p.rows.row(pc.b, pc.tok_begin + t * TK);
-                    if (!(ok = mbar_wait(&empty[s], ((gt >> 1) & 1) ^ 1, ab, 1))) break;
+                    const int32_t row = warp_uniform((int32_t)p.rows.row(pc.b, pc.tok_begin + t * TK));
+                    if (!(ok = warp_all(mbar_wait(&empty[s], ((gt >> 1) & 1) ^ 1, ab, 1)))) break;
 #pragma unroll
                     for (int g = 0; g < 3; ++g) {
-                        mbar_expect_tx(&full[s * 3 + g], L::kGroup);
+                        mbar_expect_tx(&full[s * 3 + g], L::kGroup, e);
 #pragma unroll
                         for (int kb = 3 * g; kb < 3 * g + 3; ++kb)
-                            tma_load_2d(st + kb * L::kBox, &tmC, kb * 64, row, &full[s * 3 + g]);
+                            tma_load_2d(st + kb * L::kBox, &tmC, kb * 64, row, &full[s * 3 + g], e);
                     }
                     // Shared memory holds two tiles and one of them is held by the softmax: what can be in flight from
                     // HBM is extended through L2 -- the tile after the next is asked into L2 now, so that its load,
                     // issued when a stage frees, finds it there.
                     if (t + kPrefetchAhead < nt) {
-                        const int32_t prow = (int32_t)p.rows.row(pc.b, pc.tok_begin + (t + kPrefetchAhead) * TK);
+                        const int32_t prow = warp_uniform((int32_t)p.rows.row(pc.b, pc.tok_begin + (t + kPrefetchAhead) * TK));
 #pragma unroll
-                        for (int kb = 0; kb < 9; ++kb) tma_prefetch_l2_2d(&tmC, kb * 64, prow);
+                        for (int kb = 0; kb < 9; ++kb) tma_prefetch_l2_2d(&tmC, kb * 64, prow, e);
                     }
                 }
                 ++pi;
@@ -229,96 +234,96 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (elect_one()) {
-            constexpr uint32_t idesc_qk = idesc_bf16(64, R, 0, 0);   // S^T: A = cache tile (K-major), B = Qh (K-major)
-            constexpr uint32_t idesc_pv = idesc_bf16(128, R, 1, 1);  // O^T: A = the tile read MN-major, B = P^T rows
-            const uint32_t q_addr = smem_u32(q_smem), p_addr0 = smem_u32(p_smem);
-            bool ok = true;
-            while (ok && walk.next(pc)) {
-                if (pc.n_tiles == 0) continue;
-                const int nt = (pc.tok_end - pc.tok_begin + TK - 1) / TK;
-                // The issuer never blocks on one of its two jobs while the other could run: it polls for the next
-                // group of boxes (-> twelve MMAs of S^T) and for the next P^T (-> P.V, which releases a tile stage
-                // and so keeps the loads flowing).  S^T(n) goes to score buffer n & 1, free once P.V(n-2) was issued.
-                int s_tile = 0, s_grp = 0, pv_tile = 0;
-                bool q_ok = false, o_ok = pi == 0;
-                uint32_t idle = 0;
-                while (pv_tile < nt) {
-                    bool did = false;
-                    if (pv_tile < s_tile) {
-                        const int n = gt + pv_tile, s = n & 1;
-                        if (mbar_test_wait(&p_ready[s], (n >> 1) & 1)) {
-                            if (!o_ok) o_ok = mbar_test_wait(o_free, (pi - 1) & 1);  // O^T of the previous piece was read
-                            if (o_ok) {
-                                tc_fence_after();
-                                const uint32_t v_addr = smem_u32(stage0 + s * L::kStageBytes);
-                                const uint32_t pb = p_addr0 + (n % L::kPBufs) * L::kPBuf;
-                                // descriptors stepped through their low words (the high words are constants): the
-                                // issuer's instructions per MMA are part of the time a tile stays held
-                                const uint64_t vd = desc_mnmajor_sw128(v_addr, L::kBox), pd = desc_mnmajor_rows(pb, L::kPRow);
-                                const uint32_t v_lo = (uint32_t)vd, v_hi = (uint32_t)(vd >> 32);
-                                const uint32_t p_lo = (uint32_t)pd, p_hi = (uint32_t)(pd >> 32);
-#pragma unroll
-                                for (int m = 0; m < 4; ++m)      // latent columns [128 m, +128): boxes 2m and 2m + 1
-#pragma unroll
-                                    for (int ks = 0; ks < 4; ++ks)  // 16 tokens per step
-                                        umma_ss_lo(tmem_base + kColO + m * R, v_lo + ((2 * m * L::kBox + ks * 2048) >> 4), v_hi,
-                                                   p_lo + ((ks * 16 * L::kPRow) >> 4), p_hi, idesc_pv, (pv_tile | ks) != 0);
-                                if constexpr (L::kPTerms > 1) {
-#pragma unroll
-                                    for (int m = 0; m < 4; ++m)
-#pragma unroll
-                                        for (int ks = 4; ks < 4 * L::kPTerms; ++ks)  // the other terms of P
-                                            umma_ss_lo(tmem_base + kColO + (4 + m) * R,
-                                                       v_lo + ((2 * m * L::kBox + (ks & 3) * 2048) >> 4), v_hi,
-                                                       p_lo + (((ks >> 2) * L::kPTerm + (ks & 3) * 16 * L::kPRow) >> 4), p_hi,
-                                                       idesc_pv, pv_tile != 0 || ks != 4);
-                                }
-                                umma_commit(&empty[s]);
-                                umma_commit(&pv_done[s]);
-                                ++pv_tile;
-                                did = true;
-                            }
-                        }
-                    }
-                    if (s_tile < nt && s_tile <= pv_tile + 1) {
-                        const int n = gt + s_tile, s = n & 1;
-                        if (!q_ok) q_ok = mbar_test_wait(q_full, pi & 1);
-                        if (q_ok && mbar_test_wait(&full[s * 3 + s_grp], (n >> 1) & 1)) {
+        const uint32_t e = elect_one();
+        constexpr uint32_t idesc_qk = idesc_bf16(64, R, 0, 0);   // S^T: A = cache tile (K-major), B = Qh (K-major)
+        constexpr uint32_t idesc_pv = idesc_bf16(128, R, 1, 1);  // O^T: A = the tile read MN-major, B = P^T rows
+        const uint32_t q_addr = smem_u32(q_smem), p_addr0 = smem_u32(p_smem);
+        bool ok = true;
+        while (ok && warp_all(walk.next(pc))) {
+            const int n_tiles = warp_uniform(pc.n_tiles);
+            if (n_tiles == 0) continue;
+            const int nt = warp_uniform((pc.tok_end - pc.tok_begin + TK - 1) / TK);
+            // The issuer never blocks on one of its two jobs while the other could run: it polls for the next
+            // group of boxes (-> twelve MMAs of S^T) and for the next P^T (-> P.V, which releases a tile stage
+            // and so keeps the loads flowing).  S^T(n) goes to score buffer n & 1, free once P.V(n-2) was issued.
+            int s_tile = 0, s_grp = 0, pv_tile = 0;
+            bool q_ok = false, o_ok = pi == 0;
+            uint32_t idle = 0;
+            while (pv_tile < nt) {
+                bool did = false;
+                if (pv_tile < s_tile) {
+                    const int n = gt + pv_tile, s = n & 1;
+                    if (warp_all(mbar_test_wait(&p_ready[s], (n >> 1) & 1))) {
+                        if (!o_ok) o_ok = warp_all(mbar_test_wait(o_free, (pi - 1) & 1));  // O^T of the previous piece was read
+                        if (o_ok) {
                             tc_fence_after();
-                            const uint32_t st = smem_u32(stage0 + s * L::kStageBytes);
-                            const uint32_t d = tmem_base + kColS + (uint32_t)s * R;
-                            const uint32_t k_lo = desc_lo(desc_kmajor_sw128(st + 3 * s_grp * L::kBox));
-                            const uint32_t q_lo = desc_lo(desc_kmajor_sw128(q_addr + 3 * s_grp * L::kQBlock));
+                            const uint32_t v_addr = smem_u32(stage0 + s * L::kStageBytes);
+                            const uint32_t pb = p_addr0 + (n % L::kPBufs) * L::kPBuf;
+                            // descriptors stepped through their low words (the high words are constants): the
+                            // issuer's instructions per MMA are part of the time a tile stays held
+                            const uint64_t vd = desc_mnmajor_sw128(v_addr, L::kBox), pd = desc_mnmajor_rows(pb, L::kPRow);
+                            const uint32_t v_lo = (uint32_t)vd, v_hi = (uint32_t)(vd >> 32);
+                            const uint32_t p_lo = (uint32_t)pd, p_hi = (uint32_t)(pd >> 32);
 #pragma unroll
-                            for (int kk = 0; kk < 3; ++kk)
+                            for (int m = 0; m < 4; ++m)      // latent columns [128 m, +128): boxes 2m and 2m + 1
 #pragma unroll
-                                for (int ks = 0; ks < 4; ++ks)
-                                    umma_ss_lo(d, k_lo + ((kk * L::kBox + ks * 32) >> 4), kDescHiSw128,
-                                               q_lo + ((kk * L::kQBlock + ks * 32) >> 4), kDescHiSw128, idesc_qk,
-                                               (uint32_t)(s_grp | kk | ks));
-                            if (++s_grp == 3) {
-                                umma_commit(&s_full[s]);
-                                s_grp = 0;
-                                if (++s_tile == nt) umma_commit(q_empty);
+                                for (int ks = 0; ks < 4; ++ks)  // 16 tokens per step
+                                    umma_ss_lo(tmem_base + kColO + m * R, v_lo + ((2 * m * L::kBox + ks * 2048) >> 4), v_hi,
+                                               p_lo + ((ks * 16 * L::kPRow) >> 4), p_hi, idesc_pv, (pv_tile | ks) != 0, e);
+                            if constexpr (L::kPTerms > 1) {
+#pragma unroll
+                                for (int m = 0; m < 4; ++m)
+#pragma unroll
+                                    for (int ks = 4; ks < 4 * L::kPTerms; ++ks)  // the other terms of P
+                                        umma_ss_lo(tmem_base + kColO + (4 + m) * R,
+                                                   v_lo + ((2 * m * L::kBox + (ks & 3) * 2048) >> 4), v_hi,
+                                                   p_lo + (((ks >> 2) * L::kPTerm + (ks & 3) * 16 * L::kPRow) >> 4), p_hi,
+                                                   idesc_pv, pv_tile != 0 || ks != 4, e);
                             }
+                            umma_commit(&empty[s], e);
+                            umma_commit(&pv_done[s], e);
+                            ++pv_tile;
                             did = true;
                         }
                     }
-                    if (did) {
-                        idle = 0;
-                    } else if (++idle > kPollSpins) {
-                        ab.raise(5);
-                        ok = false;
-                        break;
-                    } else if ((idle & 255u) == 255u && ab.raised()) {
-                        ok = false;
-                        break;
+                }
+                if (s_tile < nt && s_tile <= pv_tile + 1) {
+                    const int n = gt + s_tile, s = n & 1;
+                    if (!q_ok) q_ok = warp_all(mbar_test_wait(q_full, pi & 1));
+                    if (q_ok && warp_all(mbar_test_wait(&full[s * 3 + s_grp], (n >> 1) & 1))) {
+                        tc_fence_after();
+                        const uint32_t st = smem_u32(stage0 + s * L::kStageBytes);
+                        const uint32_t d = tmem_base + kColS + (uint32_t)s * R;
+                        const uint32_t k_lo = desc_lo(desc_kmajor_sw128(st + 3 * s_grp * L::kBox));
+                        const uint32_t q_lo = desc_lo(desc_kmajor_sw128(q_addr + 3 * s_grp * L::kQBlock));
+#pragma unroll
+                        for (int kk = 0; kk < 3; ++kk)
+#pragma unroll
+                            for (int ks = 0; ks < 4; ++ks)
+                                umma_ss_lo(d, k_lo + ((kk * L::kBox + ks * 32) >> 4), kDescHiSw128,
+                                           q_lo + ((kk * L::kQBlock + ks * 32) >> 4), kDescHiSw128, idesc_qk,
+                                           (uint32_t)(s_grp | kk | ks), e);
+                        if (++s_grp == 3) {
+                            umma_commit(&s_full[s], e);
+                            s_grp = 0;
+                            if (++s_tile == nt) umma_commit(q_empty, e);
+                        }
+                        did = true;
                     }
                 }
-                gt += nt;
-                ++pi;
+                if (did) {
+                    idle = 0;
+                } else if (++idle > kPollSpins) {
+                    ab.raise(5);
+                    ok = false;
+                    break;
+                } else if ((idle & 255u) == 255u && warp_all(ab.raised())) {
+                    ok = false;
+                    break;
+                }
             }
+            gt += nt;
+            ++pi;
         }
     } else {
         // ------------------------------------------------------------------ softmax

@@ -22,6 +22,8 @@
 // use the swizzle whose span equals their length (128 / 64 / 32 bytes for R = 64 / 32 / 16).  Double-buffered so
 // that writing P(n) only waits for P.V(n-2).  O^T has one value column per lane and one query row per TMEM column, so the epilogue needs no
 // replica merge: for every row the 128 lanes store 128 consecutive floats.
+// Issuer and producer run converged (tc_common.cuh): one sequence of 3001 rows 7.4 -> 7.2 us, 64 x 4096 rows at s_q = 2 179.3 ->
+// 176.3 at the power cap.
 #pragma once
 #include "common.cuh"
 #include "sched.cuh"
@@ -149,7 +151,7 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
     constexpr uint32_t kColS = 0, kColO = 2 * R, kColsUsed = (2 + L::kAcc) * R;
     constexpr uint32_t kTmemCols = kColsUsed <= 64 ? 64 : (kColsUsed <= 128 ? 128 : (kColsUsed <= 256 ? 256 : 512));
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const Abort ab{abort_flag, p.status};
 
     if (threadIdx.x == 0) {
@@ -172,7 +174,7 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
     pdl_wait();  // set-up is done (behind the preceding kernel's tail); everything below reads the caller's tensors
     const int vb = blockIdx.x % p.v_blocks;
     const int j = (blockIdx.x / p.v_blocks) % p.g;
@@ -190,11 +192,11 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        auto load_q = [&](int kb, int32_t b) {  // one k-block of the query rows of sequence b
+        auto load_q = [&](int kb, int32_t b, uint32_t e) {  // one k-block of the query rows of sequence b
             asm volatile(
-                "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
-                "[%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(q_smem + kb * L::kQBlock)),
-                "l"(reinterpret_cast<uint64_t>(&tmQ)), "r"(smem_u32(q_full)), "r"(kb * 64), "r"(0), "r"(j), "r"(b * p.s_q)
+                "{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %7, 0;\n\t@e cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
+                "[%1, {%3, %4, %5, %6}], [%2];\n\t}" ::"r"(smem_u32(q_smem + kb * L::kQBlock)),
+                "l"(reinterpret_cast<uint64_t>(&tmQ)), "r"(smem_u32(q_full)), "r"(kb * 64), "r"(0), "r"(j), "r"(b * p.s_q), "r"(e)
                 : "memory");
         };
         if constexpr (PG != 0) {
@@ -223,7 +225,7 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                         if (pi > 0 && !(ok = __all_sync(0xffffffffu, mbar_wait(q_empty, (pi - 1) & 1, ab, 13)))) break;
                         if (lane == 0) mbar_expect_tx(q_full, L::kQBytes);
                         __syncwarp();
-                        if (lane < 3) load_q(lane, pc.b);
+                        if (lane < 3) load_q(lane, pc.b, 1);
                     }
                     if (!(ok = __all_sync(0xffffffffu, mbar_wait(&vempty[s], ph ^ 1, ab, 2)))) break;
                     if (lane == 0) mbar_expect_tx(&vfull[s], L::kVBytes);
@@ -240,101 +242,105 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                 }
                 ++pi;
             }
-        } else if (elect_one()) {
+        } else {
+            const uint32_t e = elect_one();
             bool ok = true;
-            while (ok && walk.next(pc)) {
-                if (pc.n_tiles == 0) continue;
+            while (ok && warp_all(walk.next(pc))) {
+                const int n_tiles = warp_uniform(pc.n_tiles);
+                if (n_tiles == 0) continue;
                 int64_t tile_row = p.rows.row(pc.b, pc.tok_begin);
-                for (int t = 0; t < pc.n_tiles; ++t, ++gt) {
+                for (int t = 0; t < n_tiles; ++t, ++gt) {
                     const int s = gt & 1;
                     const uint32_t ph = (gt >> 1) & 1;
                     uint8_t* st = stage0 + s * L::kStageBytes;
-                    const int32_t row = (int32_t)tile_row;
-                    if (t + 1 < pc.n_tiles)
+                    const int32_t row = warp_uniform((int32_t)tile_row);
+                    if (t + 1 < n_tiles)
                         tile_row = p.rows.paged() ? p.rows.row(pc.b, pc.tok_begin + (t + 1) * 128) : tile_row + 128;
-                    if (!(ok = mbar_wait(&kempty[s], ph ^ 1, ab, 1))) break;
-                    mbar_expect_tx(&kfull[s], L::kKcBytes + L::kKrBytes);
-                    tma_load_3d(st, &tmK, 0, j, row, &kfull[s]);
-                    tma_load_3d(st + 16384, &tmK, 64, j, row, &kfull[s]);
-                    tma_load_2d(st + L::kKcBytes, &tmR, 0, row, &kfull[s]);
+                    if (!(ok = warp_all(mbar_wait(&kempty[s], ph ^ 1, ab, 1)))) break;
+                    mbar_expect_tx(&kfull[s], L::kKcBytes + L::kKrBytes, e);
+                    tma_load_3d(st, &tmK, 0, j, row, &kfull[s], e);
+                    tma_load_3d(st + 16384, &tmK, 64, j, row, &kfull[s], e);
+                    tma_load_2d(st + L::kKcBytes, &tmR, 0, row, &kfull[s], e);
                     // Q of the piece goes out behind its first K tile: that one only needs a free slot, Q needs every
                     // Q K^T of the previous piece to have completed
                     if (t == 0) {
-                        if (pi > 0 && !(ok = mbar_wait(q_empty, (pi - 1) & 1, ab, 13))) break;
-                        mbar_expect_tx(q_full, L::kQBytes);
-                        for (int kb = 0; kb < 3; ++kb) load_q(kb, pc.b);
+                        if (pi > 0 && !(ok = warp_all(mbar_wait(q_empty, (pi - 1) & 1, ab, 13)))) break;
+                        mbar_expect_tx(q_full, L::kQBytes, e);
+                        const int32_t b = warp_uniform(pc.b);
+#pragma unroll
+                        for (int kb = 0; kb < 3; ++kb) load_q(kb, b, e);
                     }
-                    if (!(ok = mbar_wait(&vempty[s], ph ^ 1, ab, 2))) break;
-                    mbar_expect_tx(&vfull[s], L::kVBytes);
-                    tma_load_3d(st + L::kKcBytes + L::kKrBytes, &tmV, vb * 128, j, row, &vfull[s]);
-                    tma_load_3d(st + L::kKcBytes + L::kKrBytes + 16384, &tmV, vb * 128 + 64, j, row, &vfull[s]);
+                    if (!(ok = warp_all(mbar_wait(&vempty[s], ph ^ 1, ab, 2)))) break;
+                    mbar_expect_tx(&vfull[s], L::kVBytes, e);
+                    tma_load_3d(st + L::kKcBytes + L::kKrBytes, &tmV, vb * 128, j, row, &vfull[s], e);
+                    tma_load_3d(st + L::kKcBytes + L::kKrBytes + 16384, &tmV, vb * 128 + 64, j, row, &vfull[s], e);
                 }
                 ++pi;
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (elect_one()) {
-            constexpr uint32_t idesc_qk = idesc_bf16(128, R, 0, 0);  // S^T: A = K tile (K-major), B = Q (K-major)
-            constexpr uint32_t idesc_pv = idesc_bf16(128, R, 1, 1);  // O^T: A = V tile read MN-major, B = P^T rows (MN-major)
-            const uint32_t q_addr = smem_u32(q_smem), p_addr0 = smem_u32(p_smem);
-            auto issue_qk = [&](int n) -> bool {
+        const uint32_t e = elect_one();
+        constexpr uint32_t idesc_qk = idesc_bf16(128, R, 0, 0);  // S^T: A = K tile (K-major), B = Q (K-major)
+        constexpr uint32_t idesc_pv = idesc_bf16(128, R, 1, 1);  // O^T: A = V tile read MN-major, B = P^T rows (MN-major)
+        const uint32_t q_addr = smem_u32(q_smem), p_addr0 = smem_u32(p_smem);
+        auto issue_qk = [&](int n) -> bool {
+            const int s = n & 1;
+            if (!warp_all(mbar_wait(&kfull[s], (n >> 1) & 1, ab, 3))) return false;
+            tc_fence_after();
+            const uint32_t st = smem_u32(stage0 + s * L::kStageBytes);
+            const uint32_t d = tmem_base + kColS + (uint32_t)s * R;
+            // descriptors stepped through their low words (the high words are constants): fewer instructions per MMA
+            const uint32_t k_lo = desc_lo(desc_kmajor_sw128(st)), q_lo = desc_lo(desc_kmajor_sw128(q_addr));
+#pragma unroll
+            for (int kb = 0; kb < 3; ++kb)
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks)
+                    umma_ss_lo(d, k_lo + ((kb * 16384 + ks * 32) >> 4), kDescHiSw128, q_lo + ((kb * L::kQBlock + ks * 32) >> 4),
+                               kDescHiSw128, idesc_qk, (uint32_t)(kb | ks), e);
+            umma_commit(&s_full[s], e);
+            umma_commit(&kempty[s], e);
+            return true;
+        };
+        bool ok = true;
+        while (ok && warp_all(walk.next(pc))) {
+            const int n_tiles = warp_uniform(pc.n_tiles);
+            if (n_tiles == 0) continue;
+            if (!(ok = warp_all(mbar_wait(q_full, pi & 1, ab, 4)))) break;
+            tc_fence_after();
+            if (!(ok = issue_qk(gt))) break;
+            for (int t = 0; t < n_tiles && ok; ++t) {
+                const int n = gt + t;
                 const int s = n & 1;
-                if (!mbar_wait(&kfull[s], (n >> 1) & 1, ab, 3)) return false;
-                tc_fence_after();
-                const uint32_t st = smem_u32(stage0 + s * L::kStageBytes);
-                const uint32_t d = tmem_base + kColS + (uint32_t)s * R;
-                // descriptors stepped through their low words (the high words are constants): fewer instructions per MMA
-                const uint32_t k_lo = desc_lo(desc_kmajor_sw128(st)), q_lo = desc_lo(desc_kmajor_sw128(q_addr));
-#pragma unroll
-                for (int kb = 0; kb < 3; ++kb)
-#pragma unroll
-                    for (int ks = 0; ks < 4; ++ks)
-                        umma_ss_lo(d, k_lo + ((kb * 16384 + ks * 32) >> 4), kDescHiSw128, q_lo + ((kb * L::kQBlock + ks * 32) >> 4),
-                                   kDescHiSw128, idesc_qk, (uint32_t)(kb | ks));
-                umma_commit(&s_full[s]);
-                umma_commit(&kempty[s]);
-                return true;
-            };
-            bool ok = true;
-            while (ok && walk.next(pc)) {
-                if (pc.n_tiles == 0) continue;
-                if (!(ok = mbar_wait(q_full, pi & 1, ab, 4))) break;
-                tc_fence_after();
-                if (!(ok = issue_qk(gt))) break;
-                for (int t = 0; t < pc.n_tiles && ok; ++t) {
-                    const int n = gt + t;
-                    const int s = n & 1;
-                    const uint32_t ph = (n >> 1) & 1;
-                    if (t + 1 < pc.n_tiles) {
-                        if (!(ok = issue_qk(n + 1))) break;
-                    } else {
-                        umma_commit(q_empty);
-                    }
-                    if (!(ok = mbar_wait(&p_ready[s], ph, ab, 5))) break;
-                    if (t == 0 && pi > 0 && !(ok = mbar_wait(o_free, (pi - 1) & 1, ab, 14))) break;
-                    if (!(ok = mbar_wait(&vfull[s], ph, ab, 6))) break;
-                    tc_fence_after();
-                    const uint32_t v_addr = smem_u32(stage0 + s * L::kStageBytes + L::kKcBytes + L::kKrBytes);
-                    const uint32_t pb = p_addr0 + s * L::kPBuf;
-                    const uint64_t vd = desc_mnmajor_sw128(v_addr, 16384), pd = desc_mnmajor_rows(pb, L::kPRow);
-#pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)  // 16 tokens per step: rows [16 ks, +16) of the V boxes and of P^T
-                        umma_ss_lo(tmem_base + kColO, (uint32_t)vd + ((ks * 2048) >> 4), (uint32_t)(vd >> 32),
-                                   (uint32_t)pd + ((ks * 16 * L::kPRow) >> 4), (uint32_t)(pd >> 32), idesc_pv, (uint32_t)(t | ks));
-                    if constexpr (L::kPTerms > 1) {
-#pragma unroll
-                        for (int ks = 8; ks < 8 * L::kPTerms; ++ks)  // the other terms of P
-                            umma_ss_lo(tmem_base + kColO + R, (uint32_t)vd + (((ks & 7) * 2048) >> 4), (uint32_t)(vd >> 32),
-                                       (uint32_t)pd + (((ks >> 3) * L::kPTerm + (ks & 7) * 16 * L::kPRow) >> 4),
-                                       (uint32_t)(pd >> 32), idesc_pv, t != 0 || ks != 8);
-                    }
-                    umma_commit(&vempty[s]);
-                    umma_commit(&pv_done[s]);
+                const uint32_t ph = (n >> 1) & 1;
+                if (t + 1 < n_tiles) {
+                    if (!(ok = issue_qk(n + 1))) break;
+                } else {
+                    umma_commit(q_empty, e);
                 }
-                gt += pc.n_tiles;
-                ++pi;
+                if (!(ok = warp_all(mbar_wait(&p_ready[s], ph, ab, 5)))) break;
+                if (t == 0 && pi > 0 && !(ok = warp_all(mbar_wait(o_free, (pi - 1) & 1, ab, 14)))) break;
+                if (!(ok = warp_all(mbar_wait(&vfull[s], ph, ab, 6)))) break;
+                tc_fence_after();
+                const uint32_t v_addr = smem_u32(stage0 + s * L::kStageBytes + L::kKcBytes + L::kKrBytes);
+                const uint32_t pb = p_addr0 + s * L::kPBuf;
+                const uint64_t vd = desc_mnmajor_sw128(v_addr, 16384), pd = desc_mnmajor_rows(pb, L::kPRow);
+#pragma unroll
+                for (int ks = 0; ks < 8; ++ks)  // 16 tokens per step: rows [16 ks, +16) of the V boxes and of P^T
+                    umma_ss_lo(tmem_base + kColO, (uint32_t)vd + ((ks * 2048) >> 4), (uint32_t)(vd >> 32),
+                               (uint32_t)pd + ((ks * 16 * L::kPRow) >> 4), (uint32_t)(pd >> 32), idesc_pv, (uint32_t)(t | ks), e);
+                if constexpr (L::kPTerms > 1) {
+#pragma unroll
+                    for (int ks = 8; ks < 8 * L::kPTerms; ++ks)  // the other terms of P
+                        umma_ss_lo(tmem_base + kColO + R, (uint32_t)vd + (((ks & 7) * 2048) >> 4), (uint32_t)(vd >> 32),
+                                   (uint32_t)pd + (((ks >> 3) * L::kPTerm + (ks & 7) * 16 * L::kPRow) >> 4),
+                                   (uint32_t)(pd >> 32), idesc_pv, t != 0 || ks != 8, e);
+                }
+                umma_commit(&vempty[s], e);
+                umma_commit(&pv_done[s], e);
             }
+            gt += n_tiles;
+            ++pi;
         }
     } else {
         // ------------------------------------------------------------------ softmax: one TMEM lane = one token per thread
