@@ -265,6 +265,12 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
                  : "r"(taddr)
                  : "memory");
 }
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* r) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr)
+                 : "memory");
+}
 // 16 lanes x 8 columns spread over the 32 threads of the warp: thread t receives, of lanes t/4 and t/4 + 8 (counted
 // from the address's lane), the columns 2 (t % 4) and 2 (t % 4) + 1 -- r[0], r[1] of the first lane, r[2], r[3] of the other.
 __device__ __forceinline__ void tmem_ld_16x256b(uint32_t taddr, uint32_t* r) {
@@ -292,8 +298,9 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
 }
 template <int N>
 __device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t* r) {
-    static_assert(N == 8 || N == 16 || N == 32, "unsupported width");
-    if constexpr (N == 8) tmem_ld8(taddr, r);
+    static_assert(N == 4 || N == 8 || N == 16 || N == 32, "unsupported width");
+    if constexpr (N == 4) tmem_ld4(taddr, r);
+    else if constexpr (N == 8) tmem_ld8(taddr, r);
     else if constexpr (N == 16) tmem_ld16(taddr, r);
     else tmem_ld32(taddr, r);
 }
