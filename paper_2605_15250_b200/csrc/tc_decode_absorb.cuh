@@ -30,19 +30,21 @@
 // and one half of that lane's 64 score columns, so a row's 128 scores of a tile sit in four threads of
 // four different warps; they share the tile maximum through shared memory and keep separate partial sums.
 //
-// Small pages (template parameter PG = rows of a box: 64, 32 or 16; 0 = the form above).  A paged cache whose pages are
+// Small pages (template parameter PG = rows of a box: 32 or 16; 0 = the form above).  A paged cache whose pages are
 // no multiple of the 128-row tile is fetched in boxes of PG rows that no page boundary cuts (PG divides the page size
 // and the tile's halves): the boxes of a group go out together, one lane of the producer warp each, after every lane has
 // looked its page up; boxes behind the sequence's end start behind the cache's last row and are filled with zeros, and of the
 // box that the end cuts V gets zeros behind it (load_cut_run): rows outside a sequence may hold anything.  Such
 // calls keep 32-bit probabilities: P is split into three bf16 terms, which hold all of its 24 bits, and P V is issued for each of
-// them.  The two further P buffers are paid for by a K ring of five single column blocks in place of three groups of three, and
-// the products of the second and third term go to accumulators of their own where tensor memory has room for them (half of O
-// here, all of it in the tokens-on-M kernels): the tensor core truncates its running sums, so every further addition into one of
-// them costs bits (relative to O about 1.7e-8 per 16 rows and term).  What bounds it: what the MMAs read through shared memory
-// (with the loads 616 KB a tile and CTA; 504 with two terms, 392 in the form above); 105 us a step on 32 sequences of 300-8000
-// rows in pages of 64 rows, 128 heads, where two terms took 88.  Neither an issuer that polls for K groups and P alike nor P
-// written by token halves while P V of the other half runs made it faster (101-110 and 104 us).
+// them.  The two further P buffers are paid for by a K ring of seven single column blocks in place of three groups of three and a
+// V ring of three groups of 32 tokens in place of two of 64: P V takes three quarters of a tile's MMA time, so V streams through
+// less, and all but two of the next tile's K blocks wait for their turn in shared memory (five K blocks and one tile of V: 99.4 us
+// a step on the batch below instead of 96.3; nine blocks and two V groups 96.5).  The products of the second and third term go to
+// accumulators of their own where tensor memory has room for them (half of O here, all of it in the tokens-on-M kernels): the
+// tensor core truncates its running sums, so every further addition into one of them costs bits (relative to O about 1.7e-8 per
+// 16 rows and term).  What bounds it: what the MMAs read through shared memory (with the loads 616 KB a tile and CTA; 504 with two
+// terms, 392 in the form above); 96 us a step on 32 sequences of 300-8000 rows in pages of 64 rows, 128 heads.  Neither an issuer
+// that polls for K groups and P alike nor P written by token halves while P V of the other half runs made it faster.
 // Errors of the merged partials there, against 64 bits: 3.6e-6 of the 2-norm (two terms 3.8e-6, SIMT kernel 3.4e-7); of the step:
 // 2.79e-3 with each of the three, from the roundings to bf16.  These calls ran one warp per query row on the SIMT kernel before,
 // which read every cache row h_q times from L2: 13.7 ms for 32 sequences of 300-8000 rows in pages of 64 rows.
@@ -77,9 +79,11 @@ struct AbsorbSmemT {
     static constexpr int kPBytes = kPTerms * kPTerm;
     static constexpr int kKBlocks = PG != 0 ? 1 : 3;  // column blocks of a K group
     static constexpr int kKGroup = kKBlocks * kBox;   // of this CTA's 64 rows of a tile
-    static constexpr int kVGroup = 4 * kBox;       // 64 tokens x this CTA's 2 x 128 latent columns
-    static constexpr int kNK = PG != 0 ? 5 : 3;    // ring of K groups (Qh Kh^T operand)
-    static constexpr int kNV = 2;                  // ring of V groups (P V operand): one tile
+    static constexpr int kVRows = PG != 0 ? 32 : 64;  // tokens of a V group
+    static constexpr int kVBox = kVRows * 128;        // kVRows tokens x 64 latent columns
+    static constexpr int kVGroup = 4 * kVBox;         // kVRows tokens x this CTA's 2 x 128 latent columns
+    static constexpr int kNK = PG != 0 ? 7 : 3;    // ring of K groups (Qh Kh^T operand)
+    static constexpr int kNV = PG != 0 ? 3 : 2;    // ring of V groups (P V operand)
     static constexpr int kOffK = kQBytes;
     static constexpr int kOffP = kOffK + kNK * kKGroup;
     static constexpr int kOffV = kOffP + kPBytes;
@@ -102,7 +106,7 @@ struct AbsorbSmemT {
     static_assert(2 * 4 * 64 >= kThreads + 4, "plan scratch must fit in sm_max");
     static_assert(kTotal <= 232448, "shared memory budget of one CTA");
     static_assert(OneCtaPerSM<kTotal>::value, "");
-    static_assert(PG == 0 || PG == 64 || PG == 32 || PG == 16, "");
+    static_assert(PG == 0 || PG == 32 || PG == 16, "");
 };
 using AbsorbSmem = AbsorbSmemT<0>;
 
@@ -269,7 +273,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
         // only after P.V of the previous tile, i.e. after Qh Kh^T of this tile has read the same cache rows
         // as K boxes, so the V boxes come out of L2.
         if constexpr (PG != 0) {
-            constexpr int NB = 64 / PG;
+            constexpr int NB = L::kVRows / PG, NG = 128 / L::kVRows;  // boxes of a column block, groups of a tile
             const int run = lane % NB, mi = lane / NB;
             int vs = 0;
             uint32_t vph = 1;
@@ -280,23 +284,23 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 if (pi > 0 && !(ok = __all_sync(0xffffffffu, mbar_wait(epi_done, (pi - 1) & 1, ab, 16)))) break;
                 const uint32_t tok = pc.tok_begin + run * PG;
                 int32_t next_row = p.rows.run_row(pc.b, tok, T, p.n_rows);
-                for (int vg = 0; vg < 2 * pc.n_tiles; ++vg) {  // (tile, token half)
+                for (int vg = 0; vg < NG * pc.n_tiles; ++vg) {
                     const int32_t row = next_row;
-                    const int32_t left = T - (pc.tok_begin + vg * 64);
-                    const int cut = cut_run<PG>(left, 64);
-                    if (vg + 1 < 2 * pc.n_tiles) next_row = p.rows.run_row(pc.b, tok + (vg + 1) * 64, T, p.n_rows);
+                    const int32_t left = T - (pc.tok_begin + vg * L::kVRows);
+                    const int cut = cut_run<PG>(left, L::kVRows);
+                    if (vg + 1 < NG * pc.n_tiles) next_row = p.rows.run_row(pc.b, tok + (vg + 1) * L::kVRows, T, p.n_rows);
                     if (!(ok = __all_sync(0xffffffffu, mbar_wait(&vempty[vs], vph, ab, 2)))) break;
                     if (cta == 0 && lane == 0) mbar_expect_tx(&vfull[vs], 2 * L::kVGroup);
                     __syncwarp();
                     uint8_t* dst = tiles + L::kOffV + vs * L::kVGroup;
                     const uint32_t bar = mapa(smem_u32(&vfull[vs]), 0);
                     if (mi < 4 && run != cut)
-                        tma_load_2d_pair(dst + mi * L::kBox + run * PG * 128, &tmC,
+                        tma_load_2d_pair(dst + mi * L::kVBox + run * PG * 128, &tmC,
                                          256 * (mi >> 1) + 128 * (int)cta + 64 * (mi & 1), row, bar);
                     if (cut >= 0)
                         load_cut_run<PG, 4>(cut_maps, lane, left % PG, __shfl_sync(0xffffffffu, row, cut), p.n_rows,
                                             [&](const CUtensorMap* m, int b, int r, int32_t y) {
-                                                tma_load_2d_pair(dst + b * L::kBox + (cut * PG + r) * 128, m,
+                                                tma_load_2d_pair(dst + b * L::kVBox + (cut * PG + r) * 128, m,
                                                                  256 * (b >> 1) + 128 * (int)cta + 64 * (b & 1), y, bar);
                                             });
                     if (++vs == L::kNV) { vs = 0; vph ^= 1; }
@@ -392,31 +396,34 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                     if (t == 0 && pi > 0 && !(ok = warp_all(mbar_wait(o_free, (pi - 1) & 1, ab, 14)))) break;
                     tc_fence_after();
 #pragma unroll 1
-                    for (int h = 0; h < 2; ++h) {
+                    for (int g = 0; g < 128 / L::kVRows; ++g) {
                         if (!(ok = warp_all(mbar_wait_fast(&vfull[vs], vph, ab, 6)))) break;
                         tc_fence_after();
-                        const uint32_t vd = desc_lo(desc_mnmajor_sw128(smem_u32(tiles + L::kOffV + vs * L::kVGroup), L::kBox));
-                        const uint32_t pd = desc_lo(p_desc) + ((h * L::kBox) >> 4);
+                        const uint32_t vd = desc_lo(desc_mnmajor_sw128(smem_u32(tiles + L::kOffV + vs * L::kVGroup), L::kVBox));
+                        const int tok = g * L::kVRows;  // P: 64 tokens a k-block
+                        const uint32_t pd = desc_lo(p_desc) + ((tok / 64 * L::kBox + tok % 64 * 2) >> 4);
 #pragma unroll
                         for (int m = 0; m < 2; ++m) {
                             const uint32_t dm = tmem_base + kAColO + (uint32_t)m * 128;
-                            if ((t | h) == 0)
-                                umma_ss2_lo<false>(dm, pd, vd + ((m * 2 * L::kBox) >> 4), idesc_pv, e);  // first P.V of a piece
+                            const uint32_t vm = vd + ((m * 2 * L::kVBox) >> 4);
+                            if ((t | g) == 0)
+                                umma_ss2_lo<false>(dm, pd, vm, idesc_pv, e);  // first P.V of a piece
                             else
-                                umma_ss2_lo<true>(dm, pd, vd + ((m * 2 * L::kBox) >> 4), idesc_pv, e);
+                                umma_ss2_lo<true>(dm, pd, vm, idesc_pv, e);
 #pragma unroll
-                            for (int kk = 1; kk < 4; ++kk)
-                                umma_ss2_lo<true>(dm, pd + ((kk * 32) >> 4), vd + ((m * 2 * L::kBox + kk * 2048) >> 4), idesc_pv, e);
+                            for (int kk = 1; kk < L::kVRows / 16; ++kk)
+                                umma_ss2_lo<true>(dm, pd + ((kk * 32) >> 4), vm + ((kk * 2048) >> 4), idesc_pv, e);
 #pragma unroll
-                            for (int kk = 4; kk < 4 * L::kPTerms; ++kk) {  // the other terms of P
-                                const uint32_t d = m == 0 ? tmem_base + kAColRest : dm;
-                                const uint32_t a = pd + (((kk >> 2) * L::kPTerm + (kk & 3) * 32) >> 4);
-                                const uint32_t b = vd + ((m * 2 * L::kBox + (kk & 3) * 2048) >> 4);
-                                if (m == 0 && kk == 4 && (t | h) == 0)
-                                    umma_ss2_lo<false>(d, a, b, idesc_pv, e);
-                                else
-                                    umma_ss2_lo<true>(d, a, b, idesc_pv, e);
-                            }
+                            for (int n = 1; n < L::kPTerms; ++n)  // the other terms of P
+#pragma unroll
+                                for (int kk = 0; kk < L::kVRows / 16; ++kk) {
+                                    const uint32_t d = m == 0 ? tmem_base + kAColRest : dm;
+                                    const uint32_t a = pd + ((n * L::kPTerm + kk * 32) >> 4), b = vm + ((kk * 2048) >> 4);
+                                    if (m == 0 && n == 1 && kk == 0 && (t | g) == 0)
+                                        umma_ss2_lo<false>(d, a, b, idesc_pv, e);
+                                    else
+                                        umma_ss2_lo<true>(d, a, b, idesc_pv, e);
+                                }
                         }
                         umma_commit2(&vempty[vs], 3, e);
                         if (++vs == L::kNV) { vs = 0; vph ^= 1; }

@@ -427,8 +427,9 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
     const int32_t workers = S >= 0 ? 0 : (tokens_on_m ? sm_count() : pair_balanced_workers(d, s_q));
     const bool balanced = S < 0 && workers > 0;
     if (S < 0) S = -S;
-    const int pg = page_box_rows(rows, balanced || S == 1);
+    int pg = page_box_rows(rows, balanced || S == 1);
     if (pg < 0 || (pg > 0 && tokens_on_m && rows_t > 32)) return GQLA_ERR_UNSUPPORTED;
+    if (pg > 32 && !tokens_on_m) pg = 32;  // the pair kernel's V groups have 32 rows
     const int64_t pairs = balanced ? (int64_t)workers * row_blocks : (int64_t)B * S * row_blocks;
     if (2 * pairs > 0x7fffffffLL) return GQLA_ERR_UNSUPPORTED;
     CUtensorMap tmQ, tmC;
@@ -458,7 +459,8 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
             constexpr int PG = decltype(box_rows)::value;
             tc::CutMaps<PG> cut;
             if (!make_cut_maps(&cut, cache, 2, cdims, cstr)) return cudaErrorInvalidValue;
-            if (!tokens_on_m) return absorb_pair_launch<PG>(p, tmQ, tmC, grid, st, cut);
+            if constexpr (PG <= 32)
+                if (!tokens_on_m) return absorb_pair_launch<PG>(p, tmQ, tmC, grid, st, cut);
             return rows_t == 16 ? absorb_t_launch<16, PG>(p, tmQ, tmC, grid, st, cut)
                                 : absorb_t_launch<32, PG>(p, tmQ, tmC, grid, st, cut);
         });
