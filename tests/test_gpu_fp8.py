@@ -162,3 +162,42 @@ def test_fp8_decode_both_paths(dims, policy, s_q):
         assert_close(gl_m.cpu().numpy(), gl_ref, "balanced decode_gqa_fp8, merged lse", 1e-2, 1e-3)
     torch.cuda.synchronize()
     assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("h_q,g,s_q", [(128, 8, 1), (128, 8, 2), (28, 4, 3), (20, 4, 1), (32, 8, 2)])
+@pytest.mark.parametrize("splits", [1, 3, -4])
+def test_fp8_gqa_tokens_on_m_edges(h_q, g, s_q, splits):
+    """At most 32 query rows per group: tiles of 256 tokens in halves of 128, odd and even counts of halves, ends on and
+    beside their edges, pieces that start inside a half (three equal splits start on multiples of 64), empty sequences,
+    16 and 32 padded rows; scores that keep outgrowing their references (growing keys)."""
+    seqlens = np.array([1, 0, 127, 128, 129, 256, 257, 640, 1100], dtype=np.int32)
+    rng = np.random.default_rng(5)
+    N, n = int(seqlens.sum()), len(seqlens)
+    ss = np.concatenate([[0], np.cumsum(seqlens)[:-1]]).astype(np.int64)
+    grow = np.concatenate([np.linspace(0.2, 1.0, t) for t in seqlens if t > 0])[:, None]  # later keys score higher
+    scale = 1.0 / np.sqrt(192.0)
+
+    def codes(shape, mul=1.0):
+        x = torch.from_numpy((rng.standard_normal(shape) * mul).astype(np.float32)).clamp(-4, 4)
+        return (x * 100).to(torch.float8_e4m3fn).view(torch.uint8).contiguous()
+
+    kc8, v8, kr8 = codes((N, g, 128), grow[:, :, None]), codes((N, g, 128)), codes((N, 64), grow)
+    q8 = codes((n, s_q, h_q, 192))
+    qs = torch.from_numpy((rng.uniform(0.5, 2.0, (n, s_q, h_q)) * 3e-4).astype(np.float32))
+    od, bd = O.Dims(h_q, g, 128, 512, 64), B.make_dims(h_q, g, 128, 512, 64)
+    S = abs(splits)
+    o_part = torch.full((n, S, s_q, h_q, 128), float("nan"), dtype=torch.float32, device="cuda")
+    lse_part = torch.full((n, S, s_q, h_q), float("nan"), dtype=torch.float32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.gqla_decode_gqa_fp8(bd, q8.cuda(), qs.cuda(), kc8.cuda(), v8.cuda(), kr8.cuda(), 0.01, torch.from_numpy(ss).cuda(),
+                          torch.from_numpy(seqlens).cuda(), scale, splits, o_part, lse_part, status)
+    assert int(status.item()) == 0
+    o_ref, l_ref = O.decode_gqa_fp8_partials(od, q8.numpy(), qs.numpy(), kc8.numpy(), v8.numpy(), kr8.numpy(), 0.01, ss, seqlens,
+                                             s_q, scale, max(splits, 1))
+    if splits < 0:  # the balanced plan cuts elsewhere: compare what its pieces merge to
+        o_m = torch.empty((n, s_q, h_q, 128), dtype=torch.float32, device="cuda")
+        l_m = torch.empty((n, s_q, h_q), dtype=torch.float32, device="cuda")
+        B.gqla_combine_splits(o_part, lse_part, o_m, l_m)
+        o_part, lse_part, o_ref, l_ref = o_m, l_m, o_ref[:, 0], l_ref[:, 0]
+    assert_close(o_part.cpu().numpy(), o_ref, "gqa fp8 tokens o", REL_TC, ABS_TC)
+    assert_close(lse_part.cpu().numpy(), l_ref, "gqa fp8 tokens lse", 1e-2, 1e-3)
