@@ -68,9 +68,10 @@ struct AbsorbParams {
                              // (o_part unused, lse_part may be null)
     int32_t* status;
     int32_t n_rows;   // rows of the cache (small pages: where the zero-filled boxes start)
+    int32_t workers;  // column halves, balanced plan: worker ids launched per row block, the last of them stands for W - 1
 };
 
-template <int PG>
+template <int PG, bool HALF = false>
 struct AbsorbSmemT {
     static constexpr int kBox = 8192;              // 64 rows x 64 bf16, 128-byte swizzle
     static constexpr int kQBytes = 9 * kBox;       // 64 query rows x 576
@@ -81,9 +82,10 @@ struct AbsorbSmemT {
     static constexpr int kKGroup = kKBlocks * kBox;   // of this CTA's 64 rows of a tile
     static constexpr int kVRows = PG != 0 ? 32 : 64;  // tokens of a V group
     static constexpr int kVBox = kVRows * 128;        // kVRows tokens x 64 latent columns
-    static constexpr int kVGroup = 4 * kVBox;         // kVRows tokens x this CTA's 2 x 128 latent columns
+    static constexpr int kBlocks = HALF ? 1 : 2;      // blocks of 256 latent columns that a pair gives
+    static constexpr int kVGroup = 2 * kBlocks * kVBox;  // kVRows tokens x this CTA's 128 columns of each block
     static constexpr int kNK = PG != 0 ? 7 : 3;    // ring of K groups (Qh Kh^T operand)
-    static constexpr int kNV = PG != 0 ? 3 : 2;    // ring of V groups (P V operand)
+    static constexpr int kNV = PG != 0 ? 3 : (HALF ? 4 : 2);    // ring of V groups (P V operand)
     static constexpr int kOffK = kQBytes;
     static constexpr int kOffP = kOffK + kNK * kKGroup;
     static constexpr int kOffV = kOffP + kPBytes;
@@ -107,6 +109,7 @@ struct AbsorbSmemT {
     static_assert(kTotal <= 232448, "shared memory budget of one CTA");
     static_assert(OneCtaPerSM<kTotal>::value, "");
     static_assert(PG == 0 || PG == 32 || PG == 16, "");
+    static_assert(!HALF || PG == 0, "small pages: both blocks");
 };
 using AbsorbSmem = AbsorbSmemT<0>;
 
@@ -116,11 +119,15 @@ constexpr uint32_t kAColRest = 384;  // small pages: the part of O's MMA 0 that 
 
 // FINAL: the whole-sequence call (o_final set); a form of its own, so that neither output's registers weigh on the softmax
 // loop of the other.
-template <int PG, bool FINAL = false>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(AbsorbSmemT<PG>::kThreads, 1)
+// HALF: a pair gives one block of 256 latent columns of O; two pairs (blockIdx / 2 even and odd) share a piece and both compute
+// its scores.  For calls that leave at least half of the device idle: half of a pair's P V, V loads and output (an SM writes about
+// 30 B a clock, 128 KB of partials are 2.3 us).  Whole steps, us: one sequence of 777 rows 22.5 -> 20.7, of 100 rows 20.9 -> 18.7, of
+// 1500 rows at s_q = 2 25.3 -> 23.2; two of 300-900 rows 23.3 -> 21.0, four of 200-500 rows 24.6 -> 22.5.
+template <int PG, bool FINAL = false, bool HALF = false>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(AbsorbSmemT<PG, HALF>::kThreads, 1)
 decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap tmQ,
                         const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CutMaps<PG> cut_maps) {
-    using L = AbsorbSmemT<PG>;
+    using L = AbsorbSmemT<PG, HALF>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* tiles = smem_raw;
     if ((smem_u32(tiles) & 1023u) != 0) {  // swizzled tiles need 1 KB alignment; same answer in both CTAs
@@ -180,13 +187,15 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
     const uint32_t tmem_base = warp_uniform(*tmem_slot);
     pdl_wait();  // set-up is done (behind the preceding kernel's tail); everything below reads the caller's tensors
     // the plan of this pair: row block rb, and either one (sequence, split) piece or worker w's share
-    const int pair = blockIdx.x >> 1;
+    const int pair = HALF ? blockIdx.x >> 2 : blockIdx.x >> 1;
+    const int blk0 = HALF ? (blockIdx.x >> 1) & 1 : 0;  // first block of 256 columns of this pair
     const int rb = pair % p.row_blocks;
     Walker walk;
     if (p.balanced) {
-        const BalancedStart st = balanced_prepass(p.seqlens, p.B, p.S, pair / p.row_blocks, p.W,
-                                                  reinterpret_cast<int32_t*>(sm_max), L::kThreads);
-        walk.init_balanced(p.seqlens, p.B, p.S, pair / p.row_blocks, p.W, st);
+        int w = pair / p.row_blocks;
+        if (HALF && w == p.workers - 1) w = p.W - 1;  // the workers in between have no tiles
+        const BalancedStart st = balanced_prepass(p.seqlens, p.B, p.S, w, p.W, reinterpret_cast<int32_t*>(sm_max), L::kThreads);
+        walk.init_balanced(p.seqlens, p.B, p.S, w, p.W, st);
     } else {
         const int unit = pair / p.row_blocks;
         walk.init_fixed(p.seqlens, p.B, p.S, unit / p.S, unit % p.S);
@@ -331,9 +340,9 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                         uint8_t* dst = tiles + L::kOffV + vs * L::kVGroup;
                         // box (m, i): latent columns [256m + 128cta + 64i, +64) -- this CTA's half of MMA m's N
 #pragma unroll
-                        for (int mi = 0; mi < 4; ++mi)
-                            tma_load_2d_pair(dst + mi * L::kBox, &tmC, 256 * (mi >> 1) + 128 * (int)cta + 64 * (mi & 1), row,
-                                             bar, e);
+                        for (int mi = 0; mi < 2 * L::kBlocks; ++mi)
+                            tma_load_2d_pair(dst + mi * L::kBox, &tmC, 256 * (blk0 + (mi >> 1)) + 128 * (int)cta + 64 * (mi & 1),
+                                             row, bar, e);
                         if (++vs == L::kNV) { vs = 0; vph ^= 1; }
                     }
                 }
@@ -403,7 +412,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                         const int tok = g * L::kVRows;  // P: 64 tokens a k-block
                         const uint32_t pd = desc_lo(p_desc) + ((tok / 64 * L::kBox + tok % 64 * 2) >> 4);
 #pragma unroll
-                        for (int m = 0; m < 2; ++m) {
+                        for (int m = 0; m < L::kBlocks; ++m) {
                             const uint32_t dm = tmem_base + kAColO + (uint32_t)m * 128;
                             const uint32_t vm = vd + ((m * 2 * L::kVBox) >> 4);
                             if ((t | g) == 0)
@@ -461,7 +470,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
             GQLA_DEBUG_CHECK(!p.balanced || pc.tok_begin % 128 == 0, p.status, 36);  // balanced pieces start on tile boundaries
             GQLA_DEBUG_CHECK(pc.fill_begin >= 0 && pc.fill_begin <= pc.fill_end && pc.fill_end <= p.S || pc.fill_end == 0, p.status, 37);
             // split slots this worker marks empty
-            if (part == 0 && row_valid && p.lse_part != nullptr)
+            if (part == 0 && blk0 == 0 && row_valid && p.lse_part != nullptr)
                 for (int kk = pc.fill_begin; kk < pc.fill_end; ++kk) p.lse_part[(slot0 + kk) * p.rows_total + rho] = -INFINITY;
             if (pc.n_tiles == 0 && p.balanced) continue;  // an empty sequence: its slots were marked above
             int32_t lim = visible_limit(T, p.s_q, pq);
@@ -536,7 +545,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 if (__any_sync(0xffffffffu, need) && t > 0) {
                     // this thread's share of the lane's O: columns [128m + 64ch, +64) for m = 0, 1
 #pragma unroll 1
-                    for (int c = 0; c < (L::kPTerms > 1 ? 6 : 4); ++c) {
+                    for (int c = 0; c < (L::kPTerms > 1 ? 6 : 2 * L::kBlocks); ++c) {
                         const uint32_t col = (c < 4 ? kAColO + (uint32_t)(c >> 1) * 128 : kAColRest) + ch * 64 + (c & 1) * 32;
                         uint32_t o[32];
                         tmem_ld32(lane_base + col, o);
@@ -579,7 +588,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 // whole-sequence call: the final bf16 rows (1 KB each) fit the staging at once -- one pass
                 uint4* dst = reinterpret_cast<uint4*>(stage + r * L::kOutPitch + (128 * hf + 64 * ch) * 2);
 #pragma unroll 1
-                for (int mc = 0; mc < 4; ++mc) {  // (m, 32-column half) of this thread's 64 columns of each m
+                for (int mc = 0; mc < 2 * L::kBlocks; ++mc) {  // (m, 32-column half) of this thread's 64 columns of each m
                     const int m = mc >> 1, c = (mc & 1) * 32;
                     uint32_t o[32];
                     if (pc.n_tiles > 0 && ok) {  // warp-uniform
@@ -603,8 +612,8 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 if (ok && lane < 8) {
                     const int rr = (warp - 2) * 8 + lane;
                     if (rho0 + rr < p.rows_total) {
-                        bulk_store(p.o_final + ((int64_t)pc.b * p.rows_total + rho0 + rr) * 512, stage + rr * L::kOutPitch,
-                                   512 * 2);
+                        bulk_store(p.o_final + ((int64_t)pc.b * p.rows_total + rho0 + rr) * 512 + 256 * blk0,
+                                   stage + rr * L::kOutPitch, L::kBlocks * 256 * 2);
                         bulk_commit();
                         bulk_wait_read();
                     }
@@ -615,9 +624,9 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                 // stages while others' stores drain (73 sequences of 300-500 rows: 53.6 us a step with two passes of the whole
                 // CTA and 1 KB stores, 52.3 like this; straight from registers 54.9; an SM writes about 30 B per clock).
                 uint8_t* own = stage + ((warp - 2) * 32 + lane) * L::kWarpPitch;
-                float* grow = p.o_part + ((slot0 + pc.k) * p.rows_total + rho) * 512 + 128 * hf + 64 * ch;
+                float* grow = p.o_part + ((slot0 + pc.k) * p.rows_total + rho) * 512 + 256 * blk0 + 128 * hf + 64 * ch;
 #pragma unroll 1
-                for (int m = 0; m < 2; ++m) {
+                for (int m = 0; m < L::kBlocks; ++m) {
                     if (m == 1) bulk_wait_read();  // this lane's row of m = 0 has left the staging
 #pragma unroll 1
                     for (int c = 0; c < 64; c += 32) {
@@ -640,7 +649,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
                                                    __uint_as_float(o[4 * i + 2]) * inv, __uint_as_float(o[4 * i + 3]) * inv)
                                      : make_float4(0.f, 0.f, 0.f, 0.f);
                     }
-                    if (m == 1) {  // O has been read: the next piece's first P.V may overwrite it
+                    if (m == L::kBlocks - 1) {  // O has been read: the next piece's first P.V may overwrite it
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive_cluster(o_free_l);
@@ -656,7 +665,7 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
             __syncwarp();
             if (lane == 0) mbar_arrive(epi_done);
             if (!__all_sync(0xffffffffu, mbar_wait(epi_done, pi & 1, ab, 12))) ok = false;
-            if (row_valid && part == 0 && p.lse_part != nullptr)
+            if (row_valid && part == 0 && blk0 == 0 && p.lse_part != nullptr)
                 p.lse_part[(slot0 + pc.k) * p.rows_total + rho] =
                     live ? (m_used + log2f(Lt)) * 0.6931471805599453f : -INFINITY;
             gt += pc.n_tiles;

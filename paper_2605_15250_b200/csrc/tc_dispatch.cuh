@@ -399,11 +399,11 @@ inline cudaError_t absorb_t_launch(const tc::AbsorbParams& p, const CUtensorMap&
     return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, c, cut);
 }
 
-template <int PG, bool FINAL = false>
+template <int PG, bool FINAL = false, bool HALF = false>
 inline cudaError_t absorb_pair_launch(const tc::AbsorbParams& p, const CUtensorMap& q, const CUtensorMap& c, unsigned grid,
                                       cudaStream_t st, const tc::CutMaps<PG>& cut = {}) {
-    using L = tc::AbsorbSmemT<PG>;
-    auto kern = tc::decode_absorb_tc_kernel<PG, FINAL>;
+    using L = tc::AbsorbSmemT<PG, HALF>;
+    auto kern = tc::decode_absorb_tc_kernel<PG, FINAL, HALF>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
     if (e != cudaSuccess) return e;
     return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, c, cut);
@@ -452,6 +452,9 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
     p.rows = rows; p.seqlens = seqlens; p.o_part = o_part; p.lse_part = lse_part; p.status = status;
     p.o_final = (__nv_bfloat16*)o_final; p.n_rows = (int32_t)cache_rows;
     if (o_final != nullptr && (balanced || S != 1)) return GQLA_ERR_UNSUPPORTED;
+    // pairs that can have a piece: the balanced plan cuts B sequences into B (S - 1) shares at most, those of its first workers, and
+    // its last worker marks the empty sequences behind them
+    const int64_t piece_pairs = balanced ? ((int64_t)B * S + 1 < workers ? (int64_t)B * S + 1 : workers) * row_blocks : pairs;
     const unsigned grid = (unsigned)(!tokens_on_m ? 2 * pairs : (balanced ? workers : B * S));  // pairs, or single CTAs
     cudaError_t e;
     if (pg != 0)
@@ -468,7 +471,12 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
         e = rows_t == 16   ? absorb_t_launch<16>(p, tmQ, tmC, grid, st)
             : rows_t == 32 ? absorb_t_launch<32>(p, tmQ, tmC, grid, st)
                            : absorb_t_launch<64>(p, tmQ, tmC, grid, st);
-    else
+    else if (2 * piece_pairs <= absorb_resident_pairs()) {
+        // Pieces for at most half of the device: two pairs per piece, a block of 256 latent columns each.
+        p.workers = balanced ? (int32_t)(piece_pairs / row_blocks) : 0;
+        e = o_final != nullptr ? absorb_pair_launch<0, true, true>(p, tmQ, tmC, (unsigned)(4 * piece_pairs), st)
+                               : absorb_pair_launch<0, false, true>(p, tmQ, tmC, (unsigned)(4 * piece_pairs), st);
+    } else
         e = o_final != nullptr ? absorb_pair_launch<0, true>(p, tmQ, tmC, grid, st) : absorb_pair_launch<0>(p, tmQ, tmC, grid, st);
     return e == cudaSuccess ? GQLA_OK : GQLA_ERR_CUDA;
 }

@@ -951,3 +951,51 @@ def test_gqa_partials_are_divided_by_their_sum(dims, s_q):
             t = int(n) - (s_q - 1 - p)
             ref = v[lo:lo + t].float().sum(0) / max(t, 1)  # whole numbers below 2^24: exact in any order
             assert torch.equal(got[b, p], ref[:, None].expand(-1, w.h_q // w.g, -1)), (int(n), p)
+
+
+@pytest.mark.parametrize("s_q", [1, 2])
+@pytest.mark.parametrize("S", [1, 2, -3])
+def test_absorb_column_halves_give_what_whole_pairs_give(s_q, S):
+    """A call whose pieces leave half of the device idle runs two pairs per piece, 256 latent columns each: bit for bit what one
+    pair per piece computes (a larger batch of the same sequences), in fp32 partials and in the final bf16 rows.  Under the balanced
+    plan the cuts differ with the batch, so there the merged output is compared (bf16 probabilities against other references)."""
+    seqlens = np.array([1, 0, 63, 64, 65, 127, 128, 129, 700, 0], dtype=np.int32)
+    n, few = len(seqlens), 8
+    if S == -3:
+        seqlens, n, few = seqlens[1:], n - 1, 9  # an empty sequence first, too
+    w = _wl("halves", n * few, s_q, 907, **CANON)
+    x = {k: t.cuda() for k, t in synth.make_inputs(w, seqlens=np.tile(seqlens, few), q_gain=4.0).items()}
+    dims = B.make_dims(w.h_q, w.g, w.d_h, w.r_kv, w.d_r)
+    q_hat = torch.empty((n * few, s_q, w.h_q, w.d_abs), dtype=torch.bfloat16, device="cuda")
+    B.gqla_absorb_q(dims, x["q_c"], x["q_r"], x["w_uk"], q_hat)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def run(lo, hi):
+        b, slots = hi - lo, abs(S)
+        q, ss, sl = q_hat[lo:hi].contiguous(), x["seq_start"][lo:hi].contiguous(), x["seqlens"][lo:hi].contiguous()
+        o = torch.full((b, slots, s_q, w.h_q, w.r_kv), float("nan"), dtype=torch.float32, device="cuda")
+        lse = torch.full((b, slots, s_q, w.h_q), float("nan"), dtype=torch.float32, device="cuda")
+        B.gqla_decode_absorb(dims, q, x["cache"], ss, sl, w.scale, S, o, lse, status)
+        if S < 0:
+            o_m = torch.empty((b, s_q, w.h_q, w.r_kv), dtype=torch.float32, device="cuda")
+            lse_m = torch.empty((b, s_q, w.h_q), dtype=torch.float32, device="cuda")
+            B.gqla_combine_splits(o, lse, o_m, lse_m)
+            return o_m, lse_m
+        if S > 1:
+            return o, lse
+        o_f = torch.full((b, s_q, w.h_q, w.r_kv), float("nan"), dtype=torch.bfloat16, device="cuda")
+        lse_f = torch.full((b, s_q, w.h_q), float("nan"), dtype=torch.float32, device="cuda")
+        B.gqla_decode_absorb_final(dims, q, x["cache"], ss, sl, w.scale, o_f, lse_f, status)
+        return o, lse, o_f, lse_f
+
+    whole = run(0, n * few)
+    for lo in range(0, n * few, n):
+        for got, ref in zip(run(lo, lo + n), whole):
+            ref = ref[lo:lo + n]
+            if S > 0:
+                assert torch.equal(got, ref)
+            else:
+                assert torch.equal(got.isinf(), ref.isinf())
+                fin = ~ref.isinf()
+                assert (got[fin] - ref[fin]).abs().max() <= 1e-2 * ref[fin].abs().max() + 1e-3
+    assert int(status.item()) == 0
