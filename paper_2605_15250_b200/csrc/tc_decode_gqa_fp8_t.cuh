@@ -5,18 +5,26 @@
 //   O^T = V^T P^T   M = 128 value columns, N = 32,    K = 128 tokens (A = V tile read MN-major, B = P^T rows; 4 MMAs)
 //
 // The tensor core does the method's FLOPs and not 128/R times as many: the row-replicating kernel is bound by the board's power
-// (a fourfold product at 32 rows per group, a sixteenfold one at 8), this one by the cache stream.  Whole steps, us at the power
-// cap and in a burst, row-replicating -> this kernel, both in turn on one GPU: 64 x 4096 rows, 128 heads, s_q = 2 149.0 -> 128.0
-// and 123.7 -> 120.1; s_q = 1 146.9 -> 105.3 and 123.0 -> 100.9; 64 x 512-20000 rows, 32 heads 316.7 -> 222.9 and 263.8 -> 208.1.
+// (a fourfold product at 32 rows per group, a sixteenfold one at 8), this one by the cache stream.  Whole steps, us back to back,
+// row-replicating -> this kernel, both in turn on one GPU: 64 x 4096 rows, 128 heads, s_q = 2 142.8 -> 116.0, s_q = 1 145.3 -> 103.9;
+// 64 x 512-20000 rows, 32 heads 310.0 -> 221.5; four sequences of 3001 rows, 128 heads, s_q = 2 17.1 -> 16.2, s_q = 1 16.4 -> 14.6.
+// Only where no CTA has more than one tile and 32 rows is the other one ahead (one sequence of 300 rows, s_q = 2: 11.1 and 11.8).
 //
 //   * A tile is 256 tokens, two halves of 128 that are loaded, multiplied and released by themselves (a ring of five halves,
 //     40 KB each): what the softmax warps pay per tile -- barrier wake-ups, the vote, the hand-over of P^T -- is as long as the
 //     work on 128 tokens of one byte.
 //   * Sixteen softmax warps: two per half, TMEM lane quadrant and half of the query rows.  A thread owns one token and R/2 rows.
-//   * References (m_ref) are those of the E4M3 kernels: a row's is put kF8Bias binades below the row's maximum and raised when a
-//     score exceeds it by more than kF8Grow; whether any does is one barrier.red per tile, the maxima are exchanged only then.
-//   * P^T rows are 32 bytes per token (32-byte swizzle).  With 16 query rows the upper half of a row stays zero and so do 16 of
-//     the 32 columns of O^T: the MMAs of these shapes are paced by the A operand's reads.
+//   * References (m_ref) are those of the E4M3 kernels: one is put kF8Bias binades below the maximum that raised it and raised when
+//     a score exceeds it by more than kF8Grow; whether any does is one barrier.red per tile behind a piece's first.  E4M3 reaches
+//     2^-10, 16 binades below such a maximum, and what is smaller loses its bits, so ONE key that holds most of a row's weight costs
+//     the tail of every token under its reference.  A row therefore has one reference, one row sum and one accumulator of O^T per
+//     GROUP of tokens, as it has in the replicas of the row-replicating kernel, and the groups are weighed against each other in
+//     fp32 at the end of a piece.  A group is the 32 tokens of a warp with 32 query rows (a k-step of P V is exactly one half's TMEM
+//     quadrant: eight groups, four replicas there), its lower or upper 16 tokens with 16 (sixteen groups, eight or sixteen replicas
+//     there).  With one reference per row, one key with 0.8 of the weight of 32768 rows gave errors of twice the tolerance.
+//     A raise is passed on through shared memory, since a warp reads one lane quadrant of O^T only.
+//   * P^T rows are 32 bytes per token (32-byte swizzle).  With 16 query rows the lower 16 tokens of a warp fill the lower half of
+//     their rows and the upper 16 the upper half, the other half stays zero: a group each in the lower and upper 16 columns of O^T.
 //   * Issuer and producer run converged (tc_common.cuh).
 #pragma once
 #include "common.cuh"
@@ -44,16 +52,22 @@ struct GqaFp8TSmem {
     static constexpr int kPBuf = 256 * kPRow;
     static constexpr int kOffStage = kQRegion;
     static constexpr int kOffP = kOffStage + kStages * kStageBytes;
-    static constexpr int kOffRed = kOffP + 2 * kPBuf;        // [R][8] row maxima / sums of the warps; the plan scratch
-    static constexpr int kOffScale = kOffRed + R * 8 * 4;    // [R] score scales of the piece's query rows
-    static constexpr int kTileBytes = kOffScale + R * 4;
+    // Tables by column of the 8 x 32 columns of O^T (accumulator, column in it), i.e. by (group of tokens, query row):
+    static constexpr int kCols = 8 * 32;
+    static constexpr int kOffSum = kOffP + 2 * kPBuf;        // [kCols] row sums at a piece's end, maxima of a raise before; the plan scratch
+    static constexpr int kOffRef = kOffSum + kCols * 4;      // [kCols] references
+    static constexpr int kOffWeight = kOffRef + kCols * 4;   // [kCols] factors of a raise; the groups' weights in the output
+    static constexpr int kOffScale = kOffWeight + kCols * 4; // [R] score scales of the piece's query rows
+    static constexpr int kOffRow = kOffScale + R * 4;        // [R] row maxima of the piece's first tile
+    static constexpr int kOffRaised = kOffRow + R * 4;       // [16] softmax warps that raised references
+    static constexpr int kTileBytes = kOffRaised + 16 * 4;
     // q_full q_empty o_free kfull[5] vfull[5] kempty[5] vempty[5] s_full[2] p_ready[2] pv_done[2]
     static constexpr int kNumBars = 3 + 4 * kStages + 6;
     static constexpr int kSoftmaxWarps = 16;
     static constexpr int kThreads = 64 + 32 * kSoftmaxWarps;
     static constexpr int kTotal = kTileBytes + kNumBars * 8 + 16;
     static_assert(R == 16 || R == 32, "query rows are padded to 16 or 32");
-    static_assert(R * 8 >= 3 * 32 + 4, "plan scratch must fit in the reduction buffer");
+    static_assert(kCols >= 3 * 32 + 4, "plan scratch must fit in the table of sums");
     static_assert(kTotal <= 232448, "shared memory budget of one CTA");
     static_assert(OneCtaPerSM<kTotal>::value, "");
 };
@@ -69,6 +83,36 @@ __device__ __forceinline__ void umma_f8_ss_lo(uint32_t d_tmem, uint32_t a_lo, ui
         : "memory");
 }
 
+// A group's first reference is that of the largest maximum among its row's groups on the piece's first tile, but at most this far
+// above its own: the maximum of 16 or 32 tokens is soon outgrown by the 2.75 binades between kF8Bias and kF8Grow, and a raise costs
+// 1.5 us (64 x 4096 rows, s_q = 2: raises on 63 % of the tiles and 180 us a step without this; 3 % with it, 116 us).  The group of
+// the row's largest key keeps its full reach, one with a smaller maximum 14 of its 16 binades.
+constexpr float kF8FirstUp = 2.0f;
+// Floats as integers of the same order, and back.
+__device__ __forceinline__ int float_order(float x) {
+    const int i = __float_as_int(x);
+    return i ^ ((i >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float float_unorder(int i) { return __int_as_float(i ^ ((i >> 31) & 0x7fffffff)); }
+// A group that has no reference yet: finite, so that scores below every float still have the probability zero and not NaN.
+constexpr float kF8NoRef = -FLT_MAX;
+
+// N floats, N a multiple of 4, to and from 16-byte aligned shared memory.
+template <int N>
+__device__ __forceinline__ void store_row(float* dst, const float* v) {
+#pragma unroll
+    for (int c = 0; c < N; c += 4) *reinterpret_cast<float4*>(dst + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+}
+
+template <int N>
+__device__ __forceinline__ void load_row(float* v, const float* src) {
+#pragma unroll
+    for (int c = 0; c < N; c += 4) {
+        const float4 a = *reinterpret_cast<const float4*>(src + c);
+        v[c] = a.x; v[c + 1] = a.y; v[c + 2] = a.z; v[c + 3] = a.w;
+    }
+}
+
 template <int R>
 __global__ void __launch_bounds__(GqaFp8TSmem<R>::kThreads, 1)
 decode_gqa_fp8_t_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorMap tmQc, const __grid_constant__ CUtensorMap tmQr,
@@ -77,7 +121,9 @@ decode_gqa_fp8_t_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorMa
     using L = GqaFp8TSmem<R>;
     constexpr int NS = L::kStages;
     constexpr int RW = R / 2;   // query rows of a softmax thread
-    constexpr int EW = RW / 2;  // rows (columns of O^T) that a warp rescales and stores
+    constexpr int EW = RW / 2;  // rows that a warp stores
+    constexpr int G = R;        // tokens (lanes of a warp) that share a reference
+    constexpr int kGroups = L::kCols / R;
     constexpr int kSmT = 32 * L::kSoftmaxWarps;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* tiles = smem_raw;
@@ -89,8 +135,13 @@ decode_gqa_fp8_t_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorMa
     uint8_t* qr_smem = tiles + L::kQcBytes;
     uint8_t* stage0 = tiles + L::kOffStage;
     uint8_t* p_smem = tiles + L::kOffP;
-    float* red = reinterpret_cast<float*>(tiles + L::kOffRed);
+    float* sm_sum = reinterpret_cast<float*>(tiles + L::kOffSum);
+    float* sm_ref = reinterpret_cast<float*>(tiles + L::kOffRef);
+    float* sm_w = reinterpret_cast<float*>(tiles + L::kOffWeight);
+    float* sm_max = sm_sum;  // a tile's maxima
     float* sm_scale = reinterpret_cast<float*>(tiles + L::kOffScale);
+    int* sm_row = reinterpret_cast<int*>(tiles + L::kOffRow);
+    int* sm_raised = reinterpret_cast<int*>(tiles + L::kOffRaised);
     uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + L::kTileBytes);
     uint64_t* q_full = bars + 0;
     uint64_t* q_empty = bars + 1;
@@ -105,9 +156,10 @@ decode_gqa_fp8_t_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorMa
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + L::kNumBars);
     volatile int32_t* abort_flag = reinterpret_cast<volatile int32_t*>(tmem_slot + 1);
 
-    // TMEM columns: two score buffers of 2 x R columns (a half each), then the 32-column output accumulator
+    // TMEM columns: two score buffers of 2 x R columns (a half each), then the eight 32-column output accumulators
     constexpr uint32_t kColS = 0, kColO = 4 * R;
-    constexpr uint32_t kTmemCols = kColO + 32 <= 128 ? 128 : 256;
+    constexpr uint32_t kTmemCols = 512;
+    static_assert(kColO + L::kCols <= kTmemCols, "");
 
     const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const Abort ab{abort_flag, p.status};
@@ -142,7 +194,7 @@ decode_gqa_fp8_t_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorMa
     const int unit = blockIdx.x / p.g;
     Walker walk;
     if (p.balanced) {
-        const BalancedStart st = balanced_prepass(p.seqlens, p.B, p.S, unit, p.W, reinterpret_cast<int32_t*>(red), L::kThreads);
+        const BalancedStart st = balanced_prepass(p.seqlens, p.B, p.S, unit, p.W, reinterpret_cast<int32_t*>(sm_sum), L::kThreads);
         walk.init_balanced(p.seqlens, p.B, p.S, unit, p.W, st);
     } else {
         walk.init_fixed(p.seqlens, p.B, p.S, unit / p.S, unit % p.S);
@@ -248,9 +300,10 @@ decode_gqa_fp8_t_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorMa
                         desc_mnmajor_sw128(smem_u32(stage0 + vs * L::kStageBytes + L::kKcBytes + L::kKrBytes), 16384);
                     const uint32_t p_lo = (uint32_t)pd0 + (((n & 1) * L::kPBuf + h * 128 * L::kPRow) >> 4);
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)  // 32 tokens per step: rows [32 kk, +32) of V and of P^T
-                        umma_f8_ss_lo(tmem_base + kColO, (uint32_t)vd + ((kk * 4096) >> 4), (uint32_t)(vd >> 32),
-                                      p_lo + ((kk * 32 * L::kPRow) >> 4), (uint32_t)(pd0 >> 32), idesc_pv, (t | h | kk) != 0, e);
+                    for (int kk = 0; kk < 4; ++kk)  // 32 tokens per step, an accumulator each: rows [32 kk, +32) of V and of P^T
+                        umma_f8_ss_lo(tmem_base + kColO + (uint32_t)(h * 4 + kk) * 32, (uint32_t)vd + ((kk * 4096) >> 4),
+                                      (uint32_t)(vd >> 32), p_lo + ((kk * 32 * L::kPRow) >> 4), (uint32_t)(pd0 >> 32), idesc_pv,
+                                      t != 0, e);
                     umma_commit(&vempty[vs], e);
                     if (++vs == NS) { vs = 0; vph ^= 1; }
                 }
@@ -265,19 +318,24 @@ decode_gqa_fp8_t_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorMa
         const int sub = (warp - 2) >> 3;         // which half of the tile
         const int half = ((warp - 2) >> 2) & 1;  // which half of the query rows: [r0, +RW)
         const int r0 = half * RW;
-        const int e0 = r0 + sub * EW;            // columns of O^T this warp rescales and stores: [e0, +EW)
+        const int e0 = r0 + sub * EW;            // rows this warp stores: [e0, +EW)
         const int tl = sub * 128 + q * 32 + lane;  // token within the tile
+        const int si = threadIdx.x - 64;           // index among the softmax threads
+        // this thread's rows in the tables: accumulator (half of the tile, quadrant), with 16 rows its lower or upper columns
+        static_assert(G / RW == 2 && kGroups * EW == 64, "");
+        const int col0 = (sub * 4 + q) * 32 + (R == 32 ? 0 : lane & 16) + r0;
         const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
         const int hshift = __ffs(p.hpg_box) - 1;  // hpg_box is a power of two: query position of row r = r >> hshift
         const int r_hi = p.s_q << hshift;
         const uint32_t pswz = ((uint32_t)(tl * L::kPRow) >> 7) & 1u;  // XOR of the row's 16-byte chunks
-        uint8_t* prow = p_smem + tl * L::kPRow + ((R == 32 ? (uint32_t)half ^ pswz : pswz) << 4) + (R == 32 ? 0 : half * 8);
-        float m_ref[RW], l[RW];  // of rows r0 .. r0 + RW - 1, in log2 units
+        const uint32_t pchunk = R == 32 ? (uint32_t)half : (uint32_t)lane >> 4;  // 16-byte chunk that holds this thread's rows
+        uint8_t* prow = p_smem + tl * L::kPRow + ((pchunk ^ pswz) << 4) + (R == 32 ? 0 : half * 8);
+        float m_ref[RW], l[RW];  // of rows r0 .. r0 + RW - 1 and this thread's group, in log2 units
 
-        if (R == 16 && half == 0) {  // the upper 16 bytes of every P^T row stay zero
+        if (R == 16 && half == 0) {  // the other 16 bytes of every P^T row stay zero
 #pragma unroll
             for (int s = 0; s < 2; ++s)
-                *reinterpret_cast<uint4*>(p_smem + s * L::kPBuf + tl * L::kPRow + ((1u ^ pswz) << 4)) = make_uint4(0, 0, 0, 0);
+                *reinterpret_cast<uint4*>(p_smem + s * L::kPBuf + tl * L::kPRow + ((pchunk ^ 1u ^ pswz) << 4)) = make_uint4(0, 0, 0, 0);
         }
 
         while (walk.next(pc)) {
@@ -287,12 +345,13 @@ decode_gqa_fp8_t_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorMa
             GQLA_DEBUG_CHECK(pc.n_tiles == 0 || (pc.k >= 0 && pc.k < p.S), p.status, 33);
             GQLA_DEBUG_CHECK(pc.tok_begin >= 0 && pc.tok_begin <= pc.tok_end && pc.tok_end <= (T > 0 ? T : 0), p.status, 34);
             const int64_t out_row0 = ((slot0 + pc.k) * p.s_q) * p.h_q + (int64_t)j * p.hpg;
-            if (sub == 0 && half == 0 && q * 32 + lane < R) {  // thread r of the first R: row r's empty slots and its score scale
-                const int r = q * 32 + lane, pq = r >> hshift, il = r & (p.hpg_box - 1);
+            if (si < R) {  // thread r of the first R: row r's empty slots and its score scale
+                const int r = si, pq = r >> hshift, il = r & (p.hpg_box - 1);
                 const bool row_valid = il < p.hpg && pq < p.s_q;
                 if (row_valid)
                     for (int kk = pc.fill_begin; kk < pc.fill_end; ++kk)
                         p.lse_part[((slot0 + kk) * p.s_q + pq) * p.h_q + (int64_t)j * p.hpg + il] = -INFINITY;
+                sm_row[r] = float_order(-INFINITY);
                 // softmax scale x log2(e) x the query row's quantisation scale
                 sm_scale[r] = p.scale_log2 *
                               (row_valid ? p.q_scale[((int64_t)pc.b * p.s_q + pq) * p.h_q + (int64_t)j * p.hpg + il] : 1.f);
@@ -300,7 +359,7 @@ decode_gqa_fp8_t_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorMa
             if (pc.n_tiles == 0 && p.balanced) continue;
             named_bar_sync(1, kSmT);  // the scales are there
 #pragma unroll
-            for (int r = 0; r < RW; ++r) { m_ref[r] = -INFINITY; l[r] = 0.f; }
+            for (int r = 0; r < RW; ++r) { m_ref[r] = kF8NoRef; l[r] = 0.f; }
             const int nt = (pc.n_tiles + 1) >> 1;
             bool ok = true;
 
@@ -324,69 +383,87 @@ decode_gqa_fp8_t_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorMa
                     tmem_ld<RW>(lane_base + kColS + (uint32_t)(2 * s + sub) * R + r0, x);
                     tmem_wait_ld();
                 }
-                float d[RW], top = -INFINITY;  // scores against their references
-                auto against_refs = [&]() {
+                float d[RW];
+                auto against = [&](const float* ref) {  // scores against references (log2 units), -inf where the token is not visible
+                    load_row<RW>(d, sm_scale + r0);
 #pragma unroll
-                    for (int c = 0; c < RW; c += 4) {
-                        const float4 sc = *reinterpret_cast<const float4*>(sm_scale + r0 + c);
-                        d[c] = fmaf(__uint_as_float(x[c]), sc.x, -m_ref[c]);
-                        d[c + 1] = fmaf(__uint_as_float(x[c + 1]), sc.y, -m_ref[c + 1]);
-                        d[c + 2] = fmaf(__uint_as_float(x[c + 2]), sc.z, -m_ref[c + 2]);
-                        d[c + 3] = fmaf(__uint_as_float(x[c + 3]), sc.w, -m_ref[c + 3]);
-                    }
+                    for (int c = 0; c < RW; ++c) d[c] = fmaf(__uint_as_float(x[c]), d[c], ref != nullptr ? -ref[c] : 0.f);
                     if (!full) {
 #pragma unroll
                         for (int c = 0; c < RW; ++c)
                             if (!(okl && r0 + c >= r_lo && r0 + c < r_hi)) d[c] = -INFINITY;
                     }
                 };
-                against_refs();
+                auto group_maxima = [&]() {  // of d, into the table
+                    warp_reduce_scatter<RW, G>(d, lane, [](float a, float b) { return fmaxf(a, b); });
+                    if (lane % 2 == 0) sm_max[col0 + lane % G / 2] = d[0];
+                };
+                if (t == 0) {
+                    // a piece's first tile gives the references: the maxima meet in shared memory
+                    against(nullptr);
+                    group_maxima();
+                    if (lane % 2 == 0) atomicMax(sm_row + r0 + lane % G / 2, float_order(d[0]));
+                    if (bar_or(!okl, kSmT)) { ok = false; break; }
+                    load_row<RW>(d, sm_max + col0);
 #pragma unroll
-                for (int c = 0; c < RW; ++c) top = fmaxf(top, d[c]);
-                if (bar_or(top > kF8Grow || !okl, kSmT)) {
-                    if (ab.raised()) { ok = false; break; }  // same answer in every thread: the flag was set before the barrier
+                    for (int c = 0; c < RW; c += 4) {
+                        const int4 top4 = *reinterpret_cast<const int4*>(sm_row + r0 + c);
+                        const int top[4] = {top4.x, top4.y, top4.z, top4.w};
 #pragma unroll
-                    for (int c = 0; c < RW; ++c) {
-                        const bool vis = okl && r0 + c >= r_lo && r0 + c < r_hi;
-                        const float wm = warp_max_redux(vis ? __uint_as_float(x[c]) * sm_scale[r0 + c] : -INFINITY);
-                        if (lane == 0) red[(r0 + c) * 8 + sub * 4 + q] = wm;
+                        for (int i = 0; i < 4; ++i)
+                            m_ref[c + i] = d[c + i] > kF8NoRef ? fminf(float_unorder(top[i]), d[c + i] + kF8FirstUp) - kF8Bias : kF8NoRef;
                     }
-                    named_bar_sync(1, kSmT);
-                    float factor[EW];  // of the rows this warp rescales
-                    bool any = false;
+                    against(m_ref);
+                } else {
+                    against(m_ref);
+                    float top = -INFINITY;
 #pragma unroll
-                    for (int c = 0; c < RW; ++c) {
-                        const float4 a = *reinterpret_cast<const float4*>(red + (r0 + c) * 8);
-                        const float4 b = *reinterpret_cast<const float4*>(red + (r0 + c) * 8 + 4);
-                        const float tm = fmaxf(fmaxf(fmaxf(a.x, a.y), fmaxf(a.z, a.w)), fmaxf(fmaxf(b.x, b.y), fmaxf(b.z, b.w)));
-                        const bool need = tm > m_ref[c] + kF8Grow;
-                        const float mn = need ? tm - kF8Bias : m_ref[c];
-                        const float f = need ? ex2(m_ref[c] - mn) : 1.f;  // ex2(-inf) = 0 on first use
-                        if (c < EW || sub) factor[c % EW] = f;
-                        any |= need;
-                        l[c] *= f;
-                        m_ref[c] = mn;
-                    }
-                    named_bar_sync(1, kSmT);  // red may be rewritten
-                    // (`any` is the same in the threads of a warp -- they hold the same rows; no barrier follows inside this branch)
-                    if (any && t > 0 && okl) {
+                    for (int c = 0; c < RW; ++c) top = fmaxf(top, d[c]);
+                    if (bar_or(top > kF8Grow || !okl, kSmT)) {
+                        if (ab.raised()) { ok = false; break; }  // same answer in every thread: the flag was set before the barrier
+                        const bool raise = __any_sync(0xffffffffu, top > kF8Grow);
+                        if (raise) {
+                            against(nullptr);
+                            group_maxima();
+                            __syncwarp();
+                            load_row<RW>(d, sm_max + col0);  // (of this warp's own groups)
+#pragma unroll
+                            for (int c = 0; c < RW; ++c) {
+                                const bool need = d[c] > m_ref[c] + kF8Grow;
+                                const float mn = need ? d[c] - kF8Bias : m_ref[c];
+                                d[c] = need ? ex2(m_ref[c] - mn) : 1.f;  // ex2(-FLT_MAX - ..) = 0 on first use
+                                l[c] *= d[c];
+                                m_ref[c] = mn;
+                            }
+                            if (lane % G == 0) store_row<RW>(sm_w + col0, d);
+                        }
+                        if (lane == 0) sm_raised[(sub * 2 + half) * 4 + q] = raise;
+                        named_bar_sync(1, kSmT);  // the factors are there
                         // O^T may be rescaled only between P.V(n-1) completing and P.V(n) being issued
                         if (!__all_sync(0xffffffffu, mbar_wait(&pv_done[(n - 1) & 1], ((n - 1) >> 1) & 1, ab, 8))) {
                             okl = false;  // noticed by everybody at the next barrier
                         } else {
                             tc_fence_after();
-                            uint32_t o[EW];
-                            tmem_ld<EW>(lane_base + kColO + e0, o);
-                            tmem_wait_ld();
+                            // the four warps of a lane quadrant take two of the eight accumulators each, of these the
+                            // columns of the warps that raised
+#pragma unroll 1
+                            for (int i = 0; i < 8; ++i) {
+                                const int a = (sub * 2 + half) * 2 + (i >> 2), h = (i >> 1) & 1;
+                                if (!sm_raised[((a >> 2) * 2 + h) * 4 + (a & 3)]) continue;
+                                const int c = a * 32 + (R == 32 ? h * 16 + (i & 1) * 8 : h * 8 + (i & 1) * 16);
+                                uint32_t o[8];
+                                tmem_ld<8>(lane_base + kColO + c, o);
+                                tmem_wait_ld();
 #pragma unroll
-                            for (int c = 0; c < EW; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * factor[c]);
-                            tmem_st<EW>(lane_base + kColO + e0, o);
+                                for (int k = 0; k < 8; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * sm_w[c + k]);
+                                tmem_st<8>(lane_base + kColO + c, o);
+                            }
                             tmem_wait_st();
                         }
+                        against(m_ref);
                     }
-                    against_refs();
                 }
-                // probabilities of this token -> its row of P^T (a row that has no reference yet sees nothing: d = -inf there)
+                // probabilities of this token -> its row of P^T (a group that has no reference yet sees nothing: d = -inf there)
                 uint32_t pk[RW / 4];
 #pragma unroll
                 for (int c = 0; c < RW; c += 4) {
@@ -409,40 +486,67 @@ decode_gqa_fp8_t_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorMa
             }
 
             // -------------------------------------------------------------- row sums over the tokens, then the output
-            // (the sums do not need the last P.V, so they are exchanged while it runs)
-            warp_sums_scatter<RW>(l, lane);
-            if (lane % (32 / RW) == 0) red[(r0 + lane / (32 / RW)) * 8 + sub * 4 + q] = l[0];
+            // (neither the sums nor the weights need the last P.V: they are made while it runs)
+            warp_reduce_scatter<RW, G>(l, lane, [](float a, float b) { return a + b; });
+            if (lane % 2 == 0) sm_sum[col0 + lane % G / 2] = l[0];
+            if (lane % G == 0) store_row<RW>(sm_ref + col0, m_ref);
+            named_bar_sync(1, kSmT);
+            // the weights of this warp's EW rows in their kGroups groups, two a lane (the warps of the other quadrants write the
+            // same values to the same places)
+            constexpr int KB = 32 / EW;
+            const int wi = lane / EW * R + e0 + lane % EW;
+            const float m0 = sm_ref[wi], m1 = sm_ref[wi + KB * R];
+            float M = fmaxf(m0, m1);
+#pragma unroll
+            for (int o = EW; o < 32; o *= 2) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+            const float w0 = m0 > kF8NoRef ? ex2(m0 - M) : 0.f, w1 = m1 > kF8NoRef ? ex2(m1 - M) : 0.f;
+            float Lt = (m0 > kF8NoRef ? sm_sum[wi] * w0 : 0.f) + (m1 > kF8NoRef ? sm_sum[wi + KB * R] * w1 : 0.f);
+#pragma unroll
+            for (int o = EW; o < 32; o *= 2) Lt += __shfl_xor_sync(0xffffffffu, Lt, o);
+            const bool seen = Lt > 0.f;
+            const float inv = seen ? p.v_scale / Lt : 0.f;
+            sm_w[wi] = seen ? w0 * inv : 0.f;
+            sm_w[wi + KB * R] = seen ? w1 * inv : 0.f;
+            __syncwarp();
             const int n_last = gt + nt - 1;
             if (nt > 0 && ok) ok = __all_sync(0xffffffffu, mbar_wait_fast(&pv_done[n_last & 1], (n_last >> 1) & 1, ab, 9));
             tc_fence_after();
-            named_bar_sync(1, kSmT);
-            uint32_t o[EW];
-            if (nt > 0 && ok) {  // warp-uniform
-                tmem_ld<EW>(lane_base + kColO + e0, o);
-                tmem_wait_ld();
+            if (q == 0 && lane < EW) {
+                const int r = e0 + lane, pq = r >> hshift, il = r & (p.hpg_box - 1);
+                if (il < p.hpg && pq < p.s_q)
+                    p.lse_part[out_row0 + (int64_t)pq * p.h_q + il] = ok && seen ? (M + log2f(Lt)) * 0.6931471805599453f : -INFINITY;
             }
-            // lane c finishes row e0 + c (one division and one logarithm per warp side by side), the others get its factor
-            const int ec = lane & (EW - 1), re = e0 + ec;
-            float mr = sub ? m_ref[EW] : m_ref[0];
+            float acc[EW];
 #pragma unroll
-            for (int c = 1; c < EW; ++c) mr = ec == c ? (sub ? m_ref[EW + c] : m_ref[c]) : mr;
-            const float4 sa = *reinterpret_cast<const float4*>(red + re * 8), sb = *reinterpret_cast<const float4*>(red + re * 8 + 4);
-            const float Lt = ((sa.x + sa.y) + (sa.z + sa.w)) + ((sb.x + sb.y) + (sb.z + sb.w));
-            const bool live = ok && nt > 0 && Lt > 0.f && mr > -INFINITY;
-            const float inv = live ? p.v_scale / Lt : 0.f;
-            if (q == 0 && lane < EW && (re & (p.hpg_box - 1)) < p.hpg && (re >> hshift) < p.s_q)
-                p.lse_part[out_row0 + (int64_t)(re >> hshift) * p.h_q + (re & (p.hpg_box - 1))] =
-                    live ? (mr + log2f(Lt)) * 0.6931471805599453f : -INFINITY;
+            for (int c = 0; c < EW; ++c) acc[c] = 0.f;
+            if (nt > 0 && ok) {  // warp-uniform
+#pragma unroll 1
+                for (int k0 = 0; k0 < (pc.n_tiles > 1 ? kGroups : KB); k0 += KB) {  // (a single half: the other's accumulators hold anything)
+                    uint32_t o[KB * EW];
+#pragma unroll
+                    for (int k = 0; k < KB; ++k) tmem_ld<EW>(lane_base + kColO + (k0 + k) * R + e0, o + k * EW);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int k = 0; k < KB; ++k)
+#pragma unroll
+                        for (int c = 0; c < EW; c += 4) {
+                            const float4 w = *reinterpret_cast<const float4*>(sm_w + (k0 + k) * R + e0 + c);
+                            acc[c] = fmaf(__uint_as_float(o[k * EW + c]), w.x, acc[c]);
+                            acc[c + 1] = fmaf(__uint_as_float(o[k * EW + c + 1]), w.y, acc[c + 1]);
+                            acc[c + 2] = fmaf(__uint_as_float(o[k * EW + c + 2]), w.z, acc[c + 2]);
+                            acc[c + 3] = fmaf(__uint_as_float(o[k * EW + c + 3]), w.w, acc[c + 3]);
+                        }
+                }
+            }
 #pragma unroll
             for (int c = 0; c < EW; ++c) {
                 const int r = e0 + c, pq = r >> hshift, il = r & (p.hpg_box - 1);
-                const float f = __shfl_sync(0xffffffffu, inv, c);
+                const bool some = __shfl_sync(0xffffffffu, inv, c) != 0.f;
                 // a lane holds one value column of every row: 128 consecutive floats per row over the quadrants
                 if (il < p.hpg && pq < p.s_q)  // padding rows are computed and dropped
-                    p.o_part[(out_row0 + (int64_t)pq * p.h_q + il) * 128 + q * 32 + lane] =
-                        f != 0.f ? __uint_as_float(o[c]) * f : 0.f;
+                    p.o_part[(out_row0 + (int64_t)pq * p.h_q + il) * 128 + q * 32 + lane] = some ? acc[c] : 0.f;
             }
-            named_bar_sync(1, kSmT);  // red and the scales may be rewritten by the next piece
+            named_bar_sync(1, kSmT);  // the tables may be rewritten by the next piece
             // O^T has been read: the next piece's first P.V may overwrite it
             tc_fence_before();
             __syncwarp();

@@ -87,22 +87,26 @@ __device__ __forceinline__ float warp_max_redux(float x) {
     i ^= (i >> 31) & 0x7fffffff;
     return __int_as_float(i);
 }
-// Sums of N values over the warp, N = 8 or 16: halving exchanges leave the sum of value i in x[0] of the 32 / N lanes
-// [i * 32 / N, ..) -- N + log2(32 / N) - 1 shuffles instead of 5 N.
-template <int N>
-__device__ __forceinline__ void warp_sums_scatter(float* x, int lane) {
-    int o = 16;
+// Sums (or what `op` gives) of N values over the warp, N = 8 or 16: halving exchanges leave that of value i in x[0] of the 32 / N
+// lanes [i * 32 / N, ..) -- N + log2(32 / N) - 1 shuffles instead of 5 N.  G = 16: over the lower and the upper 16 lanes apart.
+template <int N, int G, typename Op>
+__device__ __forceinline__ void warp_reduce_scatter(float* x, int lane, Op op) {
+    int o = G / 2;
 #pragma unroll
     for (int n = N / 2; n > 0; n /= 2, o /= 2) {
         const bool up = lane & o;
 #pragma unroll
         for (int i = 0; i < n; ++i) {
             const float mine = up ? x[n + i] : x[i], theirs = up ? x[i] : x[n + i];
-            x[i] = mine + __shfl_xor_sync(0xffffffffu, theirs, o);
+            x[i] = op(mine, __shfl_xor_sync(0xffffffffu, theirs, o));
         }
     }
 #pragma unroll
-    for (; o > 0; o /= 2) x[0] += __shfl_xor_sync(0xffffffffu, x[0], o);
+    for (; o > 0; o /= 2) x[0] = op(x[0], __shfl_xor_sync(0xffffffffu, x[0], o));
+}
+template <int N>
+__device__ __forceinline__ void warp_sums_scatter(float* x, int lane) {
+    warp_reduce_scatter<N, 32>(x, lane, [](float a, float b) { return a + b; });
 }
 __device__ __forceinline__ void tmem_ld_n(uint32_t taddr, uint32_t* r, int n) {  // n in {8, 16}
     if (n == 8) tmem_ld8(taddr, r);

@@ -201,3 +201,42 @@ def test_fp8_gqa_tokens_on_m_edges(h_q, g, s_q, splits):
         o_part, lse_part, o_ref, l_ref = o_m, l_m, o_ref[:, 0], l_ref[:, 0]
     assert_close(o_part.cpu().numpy(), o_ref, "gqa fp8 tokens o", REL_TC, ABS_TC)
     assert_close(lse_part.cpu().numpy(), l_ref, "gqa fp8 tokens lse", 1e-2, 1e-3)
+
+
+@pytest.mark.parametrize("h_q,g,s_q", [(32, 2, 2), (32, 2, 1), (8, 2, 1)])
+@pytest.mark.parametrize("sink", [0, 11111, 32767])
+def test_fp8_gqa_one_key_with_most_of_the_weight(h_q, g, s_q, sink):
+    """One key (of a small value vector) holds most of every row's weight (about four fifths), the other 32767 share the rest: an attention sink.
+    E4M3 loses bits 14 binades below a reference, so the tail may be rounded against that key only in the few tokens that share its
+    reference.  The tolerance is that of ordinary scores; one reference for all tokens of a row misses it by a factor of two."""
+    T, n = 32768, 30
+    rng = np.random.default_rng(17)
+
+    def codes(x):
+        return torch.from_numpy((np.clip(x, -4, 4) * 100).astype(np.float32)).to(torch.float8_e4m3fn).view(torch.uint8).contiguous()
+
+    # n RoPE coordinates that only the sink's key uses: each adds 2.24 * 2.56 / sqrt(192) = 0.414 to its score
+    k_r = rng.standard_normal((T, 64))
+    k_r[:, :n] = 0
+    k_r[sink, :n] = 2.56
+    q = rng.standard_normal((1, s_q, h_q, 192))
+    q[..., 128:128 + n] = 2.24
+    v = rng.standard_normal((T, g, 128)) + 1
+    v[sink] *= 0.1
+    kc8, v8, kr8, q8 = codes(rng.standard_normal((T, g, 128))), codes(v), codes(k_r), codes(q)
+    qs = torch.full((1, s_q, h_q), 1e-4)
+    ss, sl = np.zeros(1, dtype=np.int64), np.array([T], dtype=np.int32)
+    scale = 1.0 / np.sqrt(192.0)
+    o_part = torch.full((1, 1, s_q, h_q, 128), float("nan"), dtype=torch.float32, device="cuda")
+    lse_part = torch.full((1, 1, s_q, h_q), float("nan"), dtype=torch.float32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.gqla_decode_gqa_fp8(B.make_dims(h_q, g, 128, 512, 64), q8.cuda(), qs.cuda(), kc8.cuda(), v8.cuda(), kr8.cuda(), 0.01,
+                          torch.from_numpy(ss).cuda(), torch.from_numpy(sl).cuda(), scale, 1, o_part, lse_part, status)
+    assert int(status.item()) == 0
+    o_ref, l_ref = O.decode_gqa_fp8_partials(O.Dims(h_q, g, 128, 512, 64), q8.numpy(), qs.numpy(), kc8.numpy(), v8.numpy(),
+                                             kr8.numpy(), 0.01, ss, sl, s_q, scale, 1)
+    # what the case is meant to be: the sink's share of the weight, read off what is left of the common value 1
+    seen = ~((np.arange(s_q) < s_q - 1) & (sink == T - 1))
+    assert 0.1 < np.median(o_ref[0, 0, seen].mean(-1)) < 0.4
+    assert_close(o_part.cpu().numpy(), o_ref, "gqa fp8 sink o", REL_TC, ABS_TC)
+    assert_close(lse_part.cpu().numpy(), l_ref, "gqa fp8 sink lse", 1e-2, 1e-3)
