@@ -316,6 +316,9 @@ __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 // OR of a predicate over the `nthreads` threads that call it (named barrier 1).
+// Warps that meet in named barriers leave a loop by such a vote on their own failed waits, not by the abort flag: a producer or
+// issuer may raise that between the reads of two warps, of which one would then leave and one go on to the next barrier, which
+// has no limit.
 __device__ __forceinline__ bool bar_or(bool v, int nthreads) {
     uint32_t r;
     asm volatile(

@@ -409,10 +409,9 @@ decode_absorb_fp8_tc_kernel(const AbsorbFp8Params p, const __grid_constant__ CUt
                 float factor = 1.f;
                 bool need = false;
                 if (bar_or(m_t > m_used + kAF8Grow || !okl, L::kSoftmaxWarps * 32)) {
-                    if (ab.raised()) { ok = false; break; }  // same answer in every thread: the flag was set before the barrier
                     float* mxs = sm_max;
                     mxs[part * 64 + r] = m_t;
-                    named_bar_sync(1, L::kSoftmaxWarps * 32);
+                    if (bar_or(!okl, L::kSoftmaxWarps * 32)) { ok = false; break; }  // leaving is agreed on (tc_common.cuh)
                     const float row_max = fmaxf(fmaxf(mxs[r], mxs[64 + r]), fmaxf(mxs[128 + r], mxs[192 + r]));
                     const float m_new = fmaxf(m_used, row_max - kAF8Bias);
                     need = m_new > m_used;

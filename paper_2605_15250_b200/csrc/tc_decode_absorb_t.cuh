@@ -384,7 +384,6 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                     }
                 }
                 if (bar_or(grow || !okl, kSmT)) {
-                    if (ab.raised()) { ok = false; break; }  // same answer in every thread: the flag was set before the barrier
                     float factor[NJ];
                     bool any = false;
 #pragma unroll
@@ -395,7 +394,7 @@ decode_absorb_t_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap
                         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
                         if (lane < 4) red[q * R + r0 + rj(j)] = mx;
                     }
-                    named_bar_sync(1, kSmT);
+                    if (bar_or(!okl, kSmT)) { ok = false; break; }  // leaving is agreed on (tc_common.cuh)
 #pragma unroll
                     for (int j = 0; j < NJ; ++j) {
                         const int r = r0 + rj(j);

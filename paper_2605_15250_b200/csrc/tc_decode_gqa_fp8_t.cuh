@@ -420,7 +420,6 @@ decode_gqa_fp8_t_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorMa
 #pragma unroll
                     for (int c = 0; c < RW; ++c) top = fmaxf(top, d[c]);
                     if (bar_or(top > kF8Grow || !okl, kSmT)) {
-                        if (ab.raised()) { ok = false; break; }  // same answer in every thread: the flag was set before the barrier
                         const bool raise = __any_sync(0xffffffffu, top > kF8Grow);
                         if (raise) {
                             against(nullptr);
@@ -438,7 +437,7 @@ decode_gqa_fp8_t_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorMa
                             if (lane % G == 0) store_row<RW>(sm_w + col0, d);
                         }
                         if (lane == 0) sm_raised[(sub * 2 + half) * 4 + q] = raise;
-                        named_bar_sync(1, kSmT);  // the factors are there
+                        if (bar_or(!okl, kSmT)) { ok = false; break; }  // the factors are there; leaving is agreed on (tc_common.cuh)
                         // O^T may be rescaled only between P.V(n-1) completing and P.V(n) being issued
                         if (!__all_sync(0xffffffffu, mbar_wait(&pv_done[(n - 1) & 1], ((n - 1) >> 1) & 1, ab, 8))) {
                             okl = false;  // noticed by everybody at the next barrier

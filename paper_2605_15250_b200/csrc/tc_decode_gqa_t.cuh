@@ -408,7 +408,6 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                         grow |= xs[c] > m_ref[rl] + kTRescaleThreshold;
                     }
                     if (bar_or(grow || !okl, kSmT)) {
-                        if (ab.raised()) { ok = false; break; }  // same answer in every thread: the flag was set before the barrier
                         // raise the references of this chunk's rows to the tile's true maxima and rescale O^T
                         float* redw = red + q * R + r0 + ch * CH;
 #pragma unroll
@@ -416,7 +415,7 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                             const float wm = warp_max_redux(xs[c]);
                             if (lane == 0) redw[c] = wm;
                         }
-                        named_bar_sync(1, kSmT);
+                        if (bar_or(!okl, kSmT)) { ok = false; break; }  // leaving is agreed on (tc_common.cuh)
                         float factor[CH];
                         bool any = false;
 #pragma unroll

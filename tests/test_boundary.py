@@ -167,3 +167,24 @@ def test_status_word_registration_round_trips():
     finally:
         L.gqla_set_status_word(None)
     assert B.get_status_word() == 0
+
+
+def test_warps_that_meet_in_barriers_leave_by_vote():
+    """Block barriers have no limit, so the warps that meet in them must leave a loop together.  The abort flag does not make
+    them: another warp may raise it between two reads.  It is read in the bounded waits and by roles that meet nobody only; the
+    kernels whose softmax warps vote on their references vote on their failed waits, too, before the next barrier."""
+    src = os.path.join(ROOT, "paper_2605_15250_b200", "csrc")
+    voting = []
+    for name in sorted(os.listdir(src)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(src, name)).read())
+        if name == "tc_common.cuh":
+            continue
+        for part in text.split("__global__")[1:]:
+            softmax = part.split("bar_or(")[0].rfind("} else {")
+            if "bar_or(" not in part:
+                continue
+            voting.append(name)
+            assert ".raised()" not in part[softmax:], name
+            assert re.search(r"if \(bar_or\(!okl, [^;{]*\)\) \{ ok = false; break; \}", part), name
+    assert sorted(set(voting)) == ["tc_decode_absorb_fp8.cuh", "tc_decode_absorb_t.cuh", "tc_decode_gqa_fp8_t.cuh",
+                                   "tc_decode_gqa_t.cuh"], voting
