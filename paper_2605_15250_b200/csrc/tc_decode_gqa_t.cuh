@@ -22,8 +22,10 @@
 // use the swizzle whose span equals their length (128 / 64 / 32 bytes for R = 64 / 32 / 16).  Double-buffered so
 // that writing P(n) only waits for P.V(n-2).  O^T has one value column per lane and one query row per TMEM column, so the epilogue needs no
 // replica merge: for every row the 128 lanes store 128 consecutive floats.
-// Issuer and producer run converged (tc_common.cuh): one sequence of 3001 rows 7.4 -> 7.2 us, 64 x 4096 rows at s_q = 2 179.3 ->
-// 176.3 at the power cap.
+// Issuer and producer run converged (tc_common.cuh): 64 x 4096 rows at s_q = 2 179.3 -> 176.3 us at the power cap, a step of one
+// sequence of 3001 rows 10.30 -> 10.20 in a chain of steps but 12.30 -> 12.6 in a graph of its own among others; 12.3 again with
+// the first tile's references set without a vote and the abort agreed on in the barrier behind it.  (With the producer in one lane's
+// branch instead 12.3, too, but 128 x 512-32768 rows of 32 heads 1361 -> 1383.)
 #pragma once
 #include "common.cuh"
 #include "sched.cuh"
@@ -407,7 +409,7 @@ decode_gqa_t_kernel(const GqaParams p, const __grid_constant__ CUtensorMap tmQ, 
                         xs[c] = vis ? __uint_as_float(x[c]) * p.scale_log2 : -INFINITY;
                         grow |= xs[c] > m_ref[rl] + kTRescaleThreshold;
                     }
-                    if (bar_or(grow || !okl, kSmT)) {
+                    if (t == 0 || bar_or(grow || !okl, kSmT)) {  // a piece's first tile raises in any case
                         // raise the references of this chunk's rows to the tile's true maxima and rescale O^T
                         float* redw = red + q * R + r0 + ch * CH;
 #pragma unroll
