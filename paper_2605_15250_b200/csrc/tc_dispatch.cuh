@@ -455,6 +455,14 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
     // pairs that can have a piece: the balanced plan cuts B sequences into B (S - 1) shares at most, those of its first workers, and
     // its last worker marks the empty sequences behind them
     const int64_t piece_pairs = balanced ? ((int64_t)B * S + 1 < workers ? (int64_t)B * S + 1 : workers) * row_blocks : pairs;
+    // Pieces for at most half of the device: two pairs per piece, a block of 256 latent columns each.  Both compute the scores, 1.5
+    // times the tensor work, which the power cap charges to calls that fill the device with it for long: whole pairs -> halves, us
+    // back to back, 36 sequences of 1200 rows 31.3 -> 29.6, 25 of 2400 42.3 -> 40.2, but 32 of 2400 45.2 -> 46.9, 36 of 5000
+    // 81.1 -> 91.7, 32 of 32768 408 -> 467, 4 x 131072 in eight splits each 213 -> 243; up to a quarter of the device 18 of 5000
+    // 70.7 -> 68.0, 4 of 131072 1295 -> 1229.  The lengths are on the device, but what they sum to is at most the cache's rows.
+    const bool column_halves = pg == 0 && !tokens_on_m &&
+                               (4 * piece_pairs <= absorb_resident_pairs() ||
+                                (2 * piece_pairs <= absorb_resident_pairs() && cache_rows * row_blocks <= 60000));
     const unsigned grid = (unsigned)(!tokens_on_m ? 2 * pairs : (balanced ? workers : B * S));  // pairs, or single CTAs
     cudaError_t e;
     if (pg != 0)
@@ -471,8 +479,7 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
         e = rows_t == 16   ? absorb_t_launch<16>(p, tmQ, tmC, grid, st)
             : rows_t == 32 ? absorb_t_launch<32>(p, tmQ, tmC, grid, st)
                            : absorb_t_launch<64>(p, tmQ, tmC, grid, st);
-    else if (2 * piece_pairs <= absorb_resident_pairs()) {
-        // Pieces for at most half of the device: two pairs per piece, a block of 256 latent columns each.
+    else if (column_halves) {
         p.workers = balanced ? (int32_t)(piece_pairs / row_blocks) : 0;
         e = o_final != nullptr ? absorb_pair_launch<0, true, true>(p, tmQ, tmC, (unsigned)(4 * piece_pairs), st)
                                : absorb_pair_launch<0, false, true>(p, tmQ, tmC, (unsigned)(4 * piece_pairs), st);
