@@ -120,9 +120,10 @@ constexpr uint32_t kAColRest = 384;  // small pages: the part of O's MMA 0 that 
 // FINAL: the whole-sequence call (o_final set); a form of its own, so that neither output's registers weigh on the softmax
 // loop of the other.
 // HALF: a pair gives one block of 256 latent columns of O; two pairs (blockIdx / 2 even and odd) share a piece and both compute
-// its scores.  For calls that leave at least half of the device idle (the rule stands in tc_dispatch.cuh): half of a pair's P V, V loads and output (an SM writes about
-// 30 B a clock, 128 KB of partials are 2.3 us).  Whole steps, us: one sequence of 777 rows 22.5 -> 20.7, of 100 rows 20.9 -> 18.7, of
-// 1500 rows at s_q = 2 25.3 -> 23.2; two of 300-900 rows 23.3 -> 21.0, four of 200-500 rows 24.6 -> 22.5.
+// its scores.  For calls that leave at least half of the device idle (the rule stands in tc_dispatch.cuh): half of a pair's P V, V
+// loads and output (an SM writes about 30 B a clock, 128 KB of partials are 2.3 us).  Whole steps, us: one sequence of 777 rows
+// 22.5 -> 20.7, of 100 rows 20.9 -> 18.7, of 1500 rows at s_q = 2 25.3 -> 23.2; two of 300-900 rows 23.3 -> 21.0, four of 200-500
+// rows 24.6 -> 22.5.
 template <int PG, bool FINAL = false, bool HALF = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(AbsorbSmemT<PG, HALF>::kThreads, 1)
 decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap tmQ,

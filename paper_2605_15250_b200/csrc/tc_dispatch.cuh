@@ -409,6 +409,13 @@ inline cudaError_t absorb_pair_launch(const tc::AbsorbParams& p, const CUtensorM
     return tc::launch_pdl(kern, dim3(grid), dim3(L::kThreads), L::kTotal, st, p, q, c, cut);
 }
 
+// Workers of a balanced plan that can have a piece: a share is at least 1 / (S - 1) of the longest sequence, so B sequences make
+// B (S - 1) shares at most, those of the first workers; the last worker marks the empty sequences behind them.
+inline int64_t absorb_piece_workers(int32_t B, int32_t S, int32_t workers) {
+    const int64_t n = (int64_t)B * (S - 1) + 1;
+    return n < workers ? n : workers;
+}
+
 inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, float scale, int32_t S,
                                     const void* q_hat, const void* cache, int64_t cache_row_stride,
                                     int64_t cache_rows, const RowMap& rows, const int32_t* seqlens,
@@ -452,9 +459,8 @@ inline gqla_status tc_decode_absorb(const gqla_dims& d, int32_t B, int32_t s_q, 
     p.rows = rows; p.seqlens = seqlens; p.o_part = o_part; p.lse_part = lse_part; p.status = status;
     p.o_final = (__nv_bfloat16*)o_final; p.n_rows = (int32_t)cache_rows;
     if (o_final != nullptr && (balanced || S != 1)) return GQLA_ERR_UNSUPPORTED;
-    // pairs that can have a piece: the balanced plan cuts B sequences into B (S - 1) shares at most, those of its first workers, and
-    // its last worker marks the empty sequences behind them
-    const int64_t piece_pairs = balanced ? ((int64_t)B * S + 1 < workers ? (int64_t)B * S + 1 : workers) * row_blocks : pairs;
+    // pairs that can have a piece
+    const int64_t piece_pairs = balanced ? absorb_piece_workers(B, S, workers) * row_blocks : pairs;
     // Pieces for at most half of the device: two pairs per piece, a block of 256 latent columns each.  Both compute the scores, 1.5
     // times the tensor work, which the power cap charges to calls that fill the device with it for long: whole pairs -> halves, us
     // back to back, 36 sequences of 1200 rows 31.3 -> 29.6, 25 of 2400 42.3 -> 40.2, but 32 of 2400 45.2 -> 46.9, 36 of 5000

@@ -76,6 +76,8 @@ def test_balanced_plan_matches_oracle():
         tiles = [-(-t // 128) for t in sl]
         share = max(-(-sum(tiles) // W), -(-max(tiles + [0]) // (S - 1)), 1)
         assert all(v <= share for v in load.values())
+        # the absorb path launches no more than these for a call of few pieces
+        assert all(w < len(sl) * (S - 1) for w in load), (sl, S, W)
     assert B.lib().gqla_balanced_plan(None, 1, 2, 1, None, None, None) == 1
     buf = (ctypes.c_int32 * 8)()
     assert B.lib().gqla_balanced_plan(buf, 2, 1, 4, buf, buf, None) == 2  # fewer than two slots
