@@ -1,7 +1,7 @@
 // GQA-path split-KV flash decoding over an FP8 (E4M3) expanded cache on tcgen05 (Eq. (mha); KV-cache
 // quantisation is among the effects the paper's model leaves out, Sec. 5.1 "Limitations").  Same structure as
-// the bf16 kernel of tc_decode_gqa.cuh -- one CTA per group, R query rows replicated F = 128/R times down the
-// 128-row MMA tile, replica f keeping the scores of tokens [f*R, (f+1)*R) of every 128-token tile, P handed
+// the bf16 kernel of tc_decode_gqa.cuh -- one CTA per group, R query rows replicated F = 128/R times (once or twice: it
+// serves 33 to 128 rows, tc_decode_gqa_fp8_t.cuh fewer) down the 128-row MMA tile, replica f keeping the scores of tokens [f*R, (f+1)*R) of every 128-token tile, P handed
 // to the P.V MMA through tensor memory -- with what one byte per element changes:
 //
 //   * MMAs are kind::f8f6f4 (E4M3 x E4M3 -> fp32), K = 32 elements per instruction: S = Q K^T takes 4 MMAs over
@@ -101,9 +101,9 @@ decode_gqa_fp8_tc_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorM
                          const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmV) {
     using L = GqaFp8Smem;
     constexpr int F = 128 / R;
-    constexpr int W = R < 32 ? 32 : R;   // columns of S a warp reads per tile
+    static_assert(R == 64 || R == 128, "fewer query rows per group are the tokens-on-M kernel's");
     constexpr int CH = 32;
-    constexpr int NCH = W / CH;
+    constexpr int NCH = R / CH;          // of the R columns of S a thread reads per tile
     constexpr int NS = L::kStages;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* tiles = smem_raw;
@@ -275,9 +275,7 @@ decode_gqa_fp8_tc_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorM
         const int il = r % p.hpg_box;
         const bool row_valid = il < p.hpg && pq < p.s_q;
         const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
-        const int col0 = R < 32 ? q * 32 : f * R;
-        const int sub = R < 32 ? lane / R : 0;
-        auto owns = [&](int c) -> bool { return R >= 32 || (c / R) == sub; };
+        const int col0 = f * R;
         const int mcg = Lr & 7, mrow0 = Lr >> 3;
 
         {   // a thread only ever writes its own columns of P; everything else stays zero for good
@@ -327,7 +325,7 @@ decode_gqa_fp8_tc_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorM
                     tmem_wait_ld();
 #pragma unroll
                     for (int c = 0; c < CH; ++c)
-                        if (owns(c) && tok0 + ch * CH + c < lim) mx = fmaxf(mx, __uint_as_float(x[c]));
+                        if (tok0 + ch * CH + c < lim) mx = fmaxf(mx, __uint_as_float(x[c]));
                 }
                 // m_used is the replica's softmax REFERENCE: raised to kF8Bias below the tile maximum that exceeded it by
                 // more than kF8Grow (a raise rescales O and has to wait for the previous tile's P.V: it is made rare)
@@ -358,19 +356,16 @@ decode_gqa_fp8_tc_kernel(const GqaFp8Params p, const __grid_constant__ CUtensorM
                 const uint32_t p_addr = lane_base + kF8ColP + (uint32_t)sb * 32 + col0 / 4;
 #pragma unroll
                 for (int ch = 0; ch < NCH; ++ch) {
-                    if (NCH > 1) {
-                        tmem_ld<CH>(s_addr + ch * CH, x);
-                        tmem_wait_ld();
-                    }
+                    tmem_ld<CH>(s_addr + ch * CH, x);
+                    tmem_wait_ld();
                     uint32_t pk[CH / 4];
 #pragma unroll
                     for (int c = 0; c < CH; c += 4) {
                         const int tok = tok0 + ch * CH + c;
-                        const bool mine = owns(c);  // R is a multiple of 8, so four neighbours share an owner
                         float e[4];
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            e[i] = (mine && tok + i < lim) ? ex2(fmaf(__uint_as_float(x[c + i]), sl2, -m_sub)) : 0.f;
+                            e[i] = tok + i < lim ? ex2(fmaf(__uint_as_float(x[c + i]), sl2, -m_sub)) : 0.f;
                             l += e[i];
                         }
                         pk[c / 4] = pack_e4m3x4(e[0], e[1], e[2], e[3]);

@@ -739,10 +739,9 @@ inline gqla_status tc_decode_gqa_fp8(const gqla_dims& d, int32_t B, int32_t s_q,
     const int hpg = d.h_q / d.g;
     int hpg_box = 0, sq_box = 0;
     int R = gqa_rows(d, s_q, &hpg_box, &sq_box);
-    // up to 32 query rows per group: the tokens-on-M kernel (1.16 times the speed at 32 rows, 1.40 at 16, 1.42 at 4); beyond, its
+    // up to 32 query rows per group: the tokens-on-M kernel (1.23 times the speed at 32 rows, 1.40 at 16 and at 4); beyond, its
     // threads would hold 32 references each, and the row-replicating kernel replicates two times at most
-    const int rows_t = gqa_rows_t(d, s_q, nullptr, nullptr);
-    const bool tokens_on_m = rows_t <= 32 && gqa_prefers_tokens(rows_t);
+    const bool tokens_on_m = gqa_rows_t(d, s_q, nullptr, nullptr) <= 32;
     if (tokens_on_m) R = gqa_rows_t(d, s_q, &hpg_box, &sq_box);
     CUtensorMap tmQc, tmQr, tmK, tmR, tmV;
     {
@@ -778,10 +777,7 @@ inline gqla_status tc_decode_gqa_fp8(const gqla_dims& d, int32_t B, int32_t s_q,
                     : gqa_fp8_t_launch<32>(p, tmQc, tmQr, tmK, tmR, tmV, (unsigned)units, st);
         return e == cudaSuccess ? GQLA_OK : GQLA_ERR_CUDA;
     }
-    switch (R) {
-        case 8: e = gqa_fp8_launch<8>(p, tmQc, tmQr, tmK, tmR, tmV, (unsigned)units, st); break;
-        case 16: e = gqa_fp8_launch<16>(p, tmQc, tmQr, tmK, tmR, tmV, (unsigned)units, st); break;
-        case 32: e = gqa_fp8_launch<32>(p, tmQc, tmQr, tmK, tmR, tmV, (unsigned)units, st); break;
+    switch (R) {  // 33 rows and more are padded to 64 or 128
         case 64: e = gqa_fp8_launch<64>(p, tmQc, tmQr, tmK, tmR, tmV, (unsigned)units, st); break;
         case 128: e = gqa_fp8_launch<128>(p, tmQc, tmQr, tmK, tmR, tmV, (unsigned)units, st); break;
         default: return GQLA_ERR_UNSUPPORTED;

@@ -164,12 +164,9 @@ def test_fp8_decode_both_paths(dims, policy, s_q):
     assert int(status.item()) == 0
 
 
-@pytest.mark.parametrize("h_q,g,s_q", [(128, 8, 1), (128, 8, 2), (28, 4, 3), (20, 4, 1), (32, 8, 2)])
-@pytest.mark.parametrize("splits", [1, 3, -4])
-def test_fp8_gqa_tokens_on_m_edges(h_q, g, s_q, splits):
-    """At most 32 query rows per group: tiles of 256 tokens in halves of 128, odd and even counts of halves, ends on and
-    beside their edges, pieces that start inside a half (three equal splits start on multiples of 64), empty sequences,
-    16 and 32 padded rows; scores that keep outgrowing their references (growing keys)."""
+def _fp8_gqa_edges(h_q, g, s_q, splits):
+    """Ends of sequences on and beside the edges of tiles and halves of tiles, empty sequences, pieces that start inside a half (three
+    equal splits start on multiples of 64); scores that keep outgrowing their references (growing keys)."""
     seqlens = np.array([1, 0, 127, 128, 129, 256, 257, 640, 1100], dtype=np.int32)
     rng = np.random.default_rng(5)
     N, n = int(seqlens.sum()), len(seqlens)
@@ -199,8 +196,22 @@ def test_fp8_gqa_tokens_on_m_edges(h_q, g, s_q, splits):
         l_m = torch.empty((n, s_q, h_q), dtype=torch.float32, device="cuda")
         B.gqla_combine_splits(o_part, lse_part, o_m, l_m)
         o_part, lse_part, o_ref, l_ref = o_m, l_m, o_ref[:, 0], l_ref[:, 0]
-    assert_close(o_part.cpu().numpy(), o_ref, "gqa fp8 tokens o", REL_TC, ABS_TC)
-    assert_close(lse_part.cpu().numpy(), l_ref, "gqa fp8 tokens lse", 1e-2, 1e-3)
+    assert_close(o_part.cpu().numpy(), o_ref, "gqa fp8 o", REL_TC, ABS_TC)
+    assert_close(lse_part.cpu().numpy(), l_ref, "gqa fp8 lse", 1e-2, 1e-3)
+
+
+@pytest.mark.parametrize("h_q,g,s_q", [(128, 8, 1), (128, 8, 2), (28, 4, 3), (20, 4, 1), (32, 8, 2)])
+@pytest.mark.parametrize("splits", [1, 3, -4])
+def test_fp8_gqa_tokens_on_m_edges(h_q, g, s_q, splits):
+    """At most 32 query rows per group: tiles of 256 tokens in halves of 128, odd and even counts of halves, 16 and 32 padded rows."""
+    _fp8_gqa_edges(h_q, g, s_q, splits)
+
+
+@pytest.mark.parametrize("h_q,g,s_q", [(128, 8, 3), (128, 8, 4), (128, 8, 8), (128, 4, 2), (28, 4, 5), (96, 1, 1)])
+@pytest.mark.parametrize("splits", [1, 3, -4])
+def test_fp8_gqa_replicated_rows_edges(h_q, g, s_q, splits):
+    """33 to 128 query rows per group, padded to 64 (replicated twice) or 128."""
+    _fp8_gqa_edges(h_q, g, s_q, splits)
 
 
 @pytest.mark.parametrize("h_q,g,s_q", [(32, 2, 2), (32, 2, 1), (8, 2, 1)])
