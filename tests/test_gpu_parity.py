@@ -963,9 +963,18 @@ def test_absorb_column_halves_give_what_whole_pairs_give(s_q, S):
     n, few = len(seqlens), 8
     if S == -3:
         seqlens, n, few = seqlens[1:], n - 1, 9  # an empty sequence first, too
+    if s_q == 2 and S != 1:  # two blocks of query rows: fewer pieces still are half of the device
+        seqlens, n, few = np.array([0, 1, 63, 65, 128, 129, 700, 0], dtype=np.int32), 8, 10
     w = _wl("halves", n * few, s_q, 907, **CANON)
     x = {k: t.cuda() for k, t in synth.make_inputs(w, seqlens=np.tile(seqlens, few), q_gain=4.0).items()}
     dims = B.make_dims(w.h_q, w.g, w.d_h, w.r_kv, w.d_r)
+    # the two sides run the forms they are named for: pairs that can have a piece, against the pairs the device holds
+    resident = B.gqla_balanced_workers(dims, torch.bfloat16, 1, "absorb")
+
+    def piece_pairs(b):
+        return s_q * (b * S if S > 0 else min(b * (-S - 1) + 1, resident // s_q))
+    assert 2 * piece_pairs(n) <= resident < 2 * piece_pairs(n * few)
+    assert x["cache"].shape[0] * s_q <= 60000  # beyond a quarter of the device halves are for small caches
     q_hat = torch.empty((n * few, s_q, w.h_q, w.d_abs), dtype=torch.bfloat16, device="cuda")
     B.gqla_absorb_q(dims, x["q_c"], x["q_r"], x["w_uk"], q_hat)
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
