@@ -15,8 +15,8 @@
 // operand shape comes out of L2 ([64 rows x 64 columns] 8 KB boxes, 128-byte swizzle).
 //
 // Staging: two rings per CTA, one of K groups (three 8 KB boxes = 192 columns of 64 rows) and one of
-// V groups (two box pairs = one token half of a tile), each one tile deep, each filled by a producer
-// warp of its own;
+// V groups (two box pairs = one token half of a tile), each one tile deep (the V ring of column halves
+// two), each filled by a producer warp of its own;
 // the loads of tile t+1 are in flight while the MMAs of tile t run, and the K loads of the next piece
 // while this piece is stored.
 // The issuer and the producers run converged (tc_common.cuh): 64 x 4096 rows 85.2 -> 82.8 us at the power cap, 48 x 1000-9001
@@ -281,7 +281,8 @@ decode_absorb_tc_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMa
         // ------------------------------------------------------------------ TMA producer of the V ring (both
         // CTAs): the two rings fill independently of one another.  V groups in the order (tile, token half); a V slot is free
         // only after P.V of the previous tile, i.e. after Qh Kh^T of this tile has read the same cache rows
-        // as K boxes, so the V boxes come out of L2.
+        // as K boxes, so the V boxes come out of L2 (with column halves, whose ring holds two tiles, V may be
+        // asked for before K; then K comes out of L2).
         if constexpr (PG != 0) {
             constexpr int NB = L::kVRows / PG, NG = 128 / L::kVRows;  // boxes of a column block, groups of a tile
             const int run = lane % NB, mi = lane / NB;

@@ -113,10 +113,10 @@ inline bool absorb_prefers_tokens(const gqla_dims& d, int32_t s_q) {
 
 // Rows per box of a paged decode call on the tensor-core kernels: 0 = the boxes of the packed form (whole tiles, which
 // need pages of a multiple of 128 rows and pieces that start on tile boundaries), 64 / 32 / 16 = the small-page form (the
-// largest that divides the page; the fixed plan's pieces start on multiples of 64 rows), -1 = neither, the generic kernels
-// serve the call.  Shuffled pages, 32 sequences of 300-8000 rows, 128 heads, whole step: 14.0 ms with pages of 64 rows on the
-// generic kernels; here 105 us on the absorb path and 112 us on the GQA path (pages of 16 rows: 107 and 146 us; of 128 rows,
-// which keep one bf16 term of a probability: 70 us on the absorb path).
+// largest that divides the page, at most 32 on the absorb path's pair kernel; the fixed plan's pieces start on multiples of 64
+// rows), -1 = neither, the generic kernels serve the call.  Shuffled pages, 32 sequences of 300-8000 rows, 128 heads, whole
+// step: 14.0 ms with pages of 64 rows on the generic kernels; here 96 us on the absorb path and 112 us on the GQA path (pages of
+// 16 rows: 97 and 146 us; of 128 rows, which keep one bf16 term of a probability: 70 us on the absorb path).
 inline int page_box_rows(const RowMap& rows, bool on_tile_boundaries) {
     if (!rows.paged() || (rows.page_size % kTileRows == 0 && on_tile_boundaries)) return 0;
     return rows.page_size % 64 == 0 ? 64 : (rows.page_size % 32 == 0 ? 32 : (rows.page_size % 16 == 0 ? 16 : -1));
